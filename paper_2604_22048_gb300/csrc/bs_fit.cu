@@ -10,6 +10,7 @@ namespace bs {
 namespace {
 
 using FitKernel = void (*)(const FitParams);
+using PointsKernel = void (*)(const FitParams, int, const int32_t *, const float *, double *, float *);
 
 #define BS_FIT_NC_SWITCH(KERNEL)                 \
     switch ((max_side + 31) / 32) {              \
@@ -30,6 +31,8 @@ FitKernel fit_kernel_for(int max_side, int regs, int n_chains)
     if (regs == 96) BS_FIT_NC_SWITCH(fit_kernel_r96)
     BS_FIT_NC_SWITCH(fit_kernel_r128)
 }
+
+PointsKernel points_kernel_for(int max_side) { BS_FIT_NC_SWITCH(logpost_points_kernel) }
 
 #undef BS_FIT_NC_SWITCH
 
@@ -73,13 +76,11 @@ cudaError_t launch_logpost_points(const FitParams &p, int n_points, const int32_
                                   cudaStream_t stream)
 {
     if (p.profile != 0) return launch_logpost_points_profile(p, n_points, gal_index, theta, logp, grad, stream);
-    const size_t smem = fit_smem_bytes(p.max_side, 1);
-    cudaError_t e = cudaFuncSetAttribute(logpost_points_kernel<0>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = fit_smem_bytes(p.max_side, kPointWarps);
+    PointsKernel k = points_kernel_for(p.max_side);
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int grid = n_points < 4096 ? n_points : 4096;
-    if (grid <= 0) return cudaSuccess;
-    logpost_points_kernel<0><<<grid, 32, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
+    k<<<n_points, 32 * kPointWarps, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
     bs::count_launches(1);
     return cudaGetLastError();
 }

@@ -127,6 +127,12 @@ __device__ __forceinline__ void slot_offsets(int npad, int j, int l, int &ox, in
     }
 }
 
+// cosh of the Moffat transform's integration nodes t_j = j / 4, written by setup_psf:
+// the nodes are the same for every grid point (x cosh t passes the stopping rule's 40
+// before node 64 for any x > 1e-5; later nodes are formed on the spot).
+constexpr int kCoshNodes = 64;
+__shared__ float s_cosh[kCoshNodes];
+
 // (x/2)^nu K_nu(x) from K_nu(x) = int_0^inf exp(-x cosh t) cosh(nu t) dt by the
 // trapezoidal rule (step 1/4); the factor (x/2)^nu is folded into the
 // exponent so the integrand stays bounded for small x.
@@ -137,7 +143,7 @@ __device__ float half_x_pow_knu(float nu, float x)
     float sum = 0.5f * expf(-x + nu * lx);
     for (int j = 1; j < 400; ++j) {
         const float t = j * h;
-        const float ch = coshf(t);
+        const float ch = j < kCoshNodes ? s_cosh[j] : coshf(t);
         const float a = -x * ch;
         const float term = 0.5f * (expf(a + nu * (lx + t)) + expf(a + nu * (lx - t)));
         sum += term;
@@ -146,20 +152,43 @@ __device__ float half_x_pow_knu(float nu, float x)
     return sum * h;
 }
 
-// Transform of the unit-flux PSF at |k| (1/arcsec).
-__device__ float psf_transfer(const bs_psf &ps, float k)
+// A unit-flux PSF's constants, formed once per galaxy.
+struct PsfConst {
+    int kind;
+    float width;      // Gaussian sigma, or the Moffat's rd
+    float nu, norm;   // Moffat: beta - 1 and 2 / Gamma(beta - 1)
+};
+
+__device__ PsfConst psf_const(const bs_psf &ps)
 {
+    PsfConst q;
+    q.kind = ps.kind;
+    q.nu = q.norm = 0.0f;
     if (ps.kind == BS_PSF_GAUSSIAN) {
-        const float s = ps.fwhm * (1.0f / 2.3548200450309493f);
-        return expf(-0.5f * k * k * s * s);
+        q.width = ps.fwhm * (1.0f / 2.3548200450309493f);
+        return q;
     }
-    // Moffat: (2 / Gamma(beta - 1)) (x/2)^(beta-1) K_(beta-1)(x), x = k rd
     const float beta = ps.beta;
-    const float rd = ps.fwhm / (2.0f * sqrtf(exp2f(1.0f / beta) - 1.0f));
-    const float x = k * rd;
+    q.width = ps.fwhm / (2.0f * sqrtf(exp2f(1.0f / beta) - 1.0f));
+    q.nu = beta - 1.0f;
+    q.norm = 2.0f / tgammaf(q.nu);
+    return q;
+}
+
+// The nodes' table (all threads; the caller's next barrier orders it).
+__device__ __forceinline__ void setup_psf()
+{
+    for (int j = threadIdx.x; j < kCoshNodes; j += blockDim.x) s_cosh[j] = coshf(j * 0.25f);
+}
+
+// Transform of the unit-flux PSF at |k| (1/arcsec).
+__device__ float psf_transfer(const PsfConst &ps, float k)
+{
+    if (ps.kind == BS_PSF_GAUSSIAN) return expf(-0.5f * k * k * ps.width * ps.width);
+    // Moffat: (2 / Gamma(beta - 1)) (x/2)^(beta-1) K_(beta-1)(x), x = k rd
+    const float x = k * ps.width;
     if (x == 0.0f) return 1.0f;
-    const float nu = beta - 1.0f;
-    return 2.0f / tgammaf(nu) * half_x_pow_knu(nu, x);
+    return ps.norm * half_x_pow_knu(ps.nu, x);
 }
 
 // sin(pi x) / (pi x)
@@ -186,7 +215,7 @@ __device__ __forceinline__ void row_dft(const void *img, int f64, int64_t off, i
                                         const float2 *tw, float2 *G)
 {
     for (int iy = threadIdx.x; iy < N; iy += blockDim.x) {
-        int idx = (int)(((long long)(N - u) * c) % N);   // -u c mod N
+        int idx = ((N - u) * c) % N;   // -u c mod N
         float re = 0.f, im = 0.f;
         const int64_t rowoff = off + (int64_t)iy * N;
         for (int ix = 0; ix < N; ++ix) {
@@ -205,7 +234,7 @@ __device__ __forceinline__ void row_dft(const void *img, int f64, int64_t off, i
 __device__ __forceinline__ float2 col_dft(const float2 *G, int N, int c, int v, const float2 *tw)
 {
     const int vm = ((v % N) + N) % N;
-    int idx = (int)(((long long)(N - vm) * c) % N);   // -v c mod N
+    int idx = ((N - vm) * c) % N;   // -v c mod N
     float re = 0.f, im = 0.f;
     for (int iy = 0; iy < N; ++iy) {
         const float2 gv = G[iy];
@@ -220,7 +249,7 @@ __device__ __forceinline__ float2 col_dft(const float2 *G, int N, int c, int v, 
 }
 
 // scale x the PSF x pixel transfer of psf `ps` at grid point (u, v).
-__device__ __forceinline__ float transfer_at(const bs_psf &ps, const GalCtx &gc, int u, int v, float scale)
+__device__ __forceinline__ float transfer_at(const PsfConst &ps, const GalCtx &gc, int u, int v, float scale)
 {
     const float kx = u * gc.dk, ky = v * gc.dk;
     return scale * psf_transfer(ps, sqrtf(kx * kx + ky * ky)) * sincpi((float)u * gc.invN) *
@@ -274,7 +303,7 @@ __device__ bool setup_folded(const FitParams &P, int gal, const SmemView &sm, Ga
             row_dft(P.data, P.data_f64, off, N, c, u, sm.tw, sm.G);
             if (P.noise_corr) row_dft(P.noise_corr, 0, off, N, c, u, sm.tw, sm.Gc);
             __syncthreads();
-            const bs_psf ps = P.psf[P.n_psf == 1 ? 0 : (int64_t)gal * J + j];
+            const PsfConst ps = psf_const(P.psf[P.n_psf == 1 ? 0 : (int64_t)gal * J + j]);
             const float sig = P.sigma[(int64_t)gal * J + j];
             for (int vi = tid; vi < npad; vi += nth) {
                 float Cx = 0.f, Cy = 0.f, S = 0.f;
@@ -332,15 +361,157 @@ __device__ bool setup_folded(const FitParams &P, int gal, const SmemView &sm, Ga
     return __syncthreads_or(bad) == 0;
 }
 
+// The stamp's x transforms (all threads): G(u, iy) = sum_ix img[iy][ix] exp(-2 pi i u (ix - c) / N)
+// for every row u of the half plane, left in the table's row u (2 N of its 3 npad
+// floats) until spectrum_rows takes it from there.  A thread takes one u and four image
+// rows, so that a twiddle and its index serve four pixels; consecutive threads take
+// consecutive u of the same rows, so that a pixel load is a broadcast.
+template <typename T>
+__device__ __forceinline__ void row_spectra(const T *__restrict__ img, int N, int c, int H, const float2 *tw,
+                                            float *tab, int rowf)
+{
+    const int items = ((N + 3) >> 2) * H;
+    for (int it = threadIdx.x; it < items; it += blockDim.x) {
+        const int q = it / H, u = it - q * H;
+        const T *p[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) p[r] = img + (size_t)min(4 * q + r, N - 1) * N;
+        float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};
+        int idx = ((N - u) * c) % N;   // -u c mod N
+#pragma unroll 4
+        for (int ix = 0; ix < N; ++ix) {
+            const float2 t = tw[idx];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float d = (float)__ldg(p[r] + ix);
+                re[r] = fmaf(d, t.x, re[r]);
+                im[r] = fmaf(-d, t.y, im[r]);
+            }
+            idx += u;
+            if (idx >= N) idx -= N;
+        }
+        float2 *G = reinterpret_cast<float2 *>(tab + (size_t)u * rowf);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (4 * q + r < N) G[4 * q + r] = make_float2(re[r], im[r]);
+    }
+}
+
+// D(u, v) = sum_iy G(u, iy) exp(-2 pi i v (iy - c) / N), scaled, from the G rows in the
+// table into its D slots, each warp UB rows at a time: a lane's columns of those rows
+// are summed together (one twiddle serves UB rows, one G value all of a lane's columns)
+// and written once the whole warp has read the rows.
+template <int NCT>
+__device__ __forceinline__ void spectrum_rows(const GalCtx &gc, const float2 *tw, float *tab)
+{
+    constexpr int UB = NCT <= 2 ? 4 : 2;
+    constexpr int rowf = 96 * NCT, npad = 32 * NCT;
+    const int N = gc.N, c = gc.c, H = gc.H;
+    const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+    const float sqrt2 = 1.41421356237309515f;
+    for (int u0 = (threadIdx.x >> 5) * UB; u0 < H; u0 += nwarp * UB) {
+        float re[UB][NCT], im[UB][NCT];
+        int idx[NCT], vm[NCT];
+        const float2 *G[UB];
+#pragma unroll
+        for (int r = 0; r < UB; ++r) {
+            G[r] = reinterpret_cast<const float2 *>(tab + (size_t)min(u0 + r, H - 1) * rowf);
+#pragma unroll
+            for (int j = 0; j < NCT; ++j) re[r][j] = im[r][j] = 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < NCT; ++j) {
+            const int v = lane + 32 * j < N ? lane + 32 * j - c : 0;
+            vm[j] = v < 0 ? v + N : v;
+            idx[j] = ((N - vm[j]) * c) % N;   // -v c mod N
+        }
+#pragma unroll 2
+        for (int iy = 0; iy < N; ++iy) {
+            float2 g[UB];
+#pragma unroll
+            for (int r = 0; r < UB; ++r) g[r] = G[r][iy];
+#pragma unroll
+            for (int j = 0; j < NCT; ++j) {
+                const float2 t = tw[idx[j]];
+#pragma unroll
+                for (int r = 0; r < UB; ++r) {   // g * conj(t)
+                    re[r][j] = fmaf(g[r].x, t.x, fmaf(g[r].y, t.y, re[r][j]));
+                    im[r][j] = fmaf(g[r].y, t.x, fmaf(-g[r].x, t.y, im[r][j]));
+                }
+                idx[j] += vm[j];
+                if (idx[j] >= N) idx[j] -= N;
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < UB; ++r) {
+            const int u = u0 + r;
+            if (u >= H) break;
+            const float scale = (u == 0 ? 1.0f : sqrt2) * gc.invN;
+            float *row = tab + (size_t)u * rowf;
+#pragma unroll
+            for (int j = 0; j < NCT; ++j) {
+                int ox, oy, ot;
+                slot_offsets(npad, j, lane, ox, oy, ot);
+                const bool in = lane + 32 * j < N;
+                row[ox] = in ? re[r][j] * scale : 0.f;
+                row[oy] = in ? im[r][j] * scale : 0.f;
+                if (!in) row[ot] = 0.f;
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// T(u, v) of every grid point (all threads).  The PSF depends on u^2 + v^2 only: one
+// value serves (u, +-a) and (a, +-u), so the Moffat's integral runs for the H (H + 1) / 2
+// pairs a <= u instead of the H N points.  Pairs of rows (H - 1 - r, r) hold H + 1
+// values together, which spreads the triangle evenly over the threads.
+template <int NCT>
+__device__ __forceinline__ void transfer_table(const GalCtx &gc, const PsfConst &ps, float *tab)
+{
+    constexpr int rowf = 96 * NCT, npad = 32 * NCT;
+    const int H = gc.H, c = gc.c;
+    const float s0 = gc.invN, s1 = 1.41421356237309515f * gc.invN;
+    const int items = ((H + 1) >> 1) * (H + 1);
+    for (int it = threadIdx.x; it < items; it += blockDim.x) {
+        const int r = it / (H + 1), q = it - r * (H + 1);
+        const bool first = q < H - r;
+        if (!first && 2 * r == H - 1) continue;   // the middle row has no partner
+        const int u = first ? H - 1 - r : r, a = first ? q : q - (H - r);
+        const float kx = u * gc.dk, ky = a * gc.dk;
+        const float f = psf_transfer(ps, sqrtf(kx * kx + ky * ky));
+        const float su = sincpi((float)u * gc.invN), sa = sincpi((float)a * gc.invN);
+        auto put = [&](int row, int v, float val) {
+            int ox, oy, ot;
+            slot_offsets(npad, (v + c) >> 5, (v + c) & 31, ox, oy, ot);
+            tab[(size_t)row * rowf + ot] = val;
+        };
+        const float tu = (u == 0 ? s0 : s1) * f * su * sa;
+        put(u, a, tu);
+        if (a) put(u, -a, tu);
+        if (a != u) {
+            const float ta = (a == 0 ? s0 : s1) * f * sa * su;
+            put(a, u, ta);
+            put(a, -u, ta);
+        }
+    }
+}
+
 // Stage the galaxy's data spectrum and transfer table (all threads of the CTA).
 // The caller has checked side_ok.  Returns false, uniformly, when the galaxy
 // cannot be fitted (a noise correlation without a positive spectrum).
+// The transforms' serial form, one frequency row at a time with a barrier on either side
+// of it, a thread per image row (53 of 128 at 53 px) and the phase index reduced in
+// 64-bit arithmetic, kept most of the warps waiting: 4,000 points of 53 px, each with its
+// own staging, took 1.18 ms against 0.33 ms with all rows and columns spread over four
+// warps; the same operations in the same order give the same table bit for bit.
+template <int NCT>
 __device__ bool setup_galaxy(const FitParams &P, int gal, const SmemView &sm, GalCtx &gc)
 {
     const int N = P.side[gal];
     const int c = (N - 1) / 2;
     const int H = c + 1;
-    const int npad = P.npad;
     const int tid = threadIdx.x, nth = blockDim.x;
     gc.N = N;
     gc.H = H;
@@ -360,39 +531,22 @@ __device__ bool setup_galaxy(const FitParams &P, int gal, const SmemView &sm, Ga
         const float kx = (float)u * gc.dk;
         sm.kxr[u] = make_float2(kx, kx * kx);
     }
+    setup_psf();
     __syncthreads();
     if (P.n_exp > 1 || P.noise_corr) return setup_folded(P, gal, sm, gc);
 
     const float sig = P.sigma[gal];
     gc.inv_b = P.pix_prec ? 1.0f : 1.0f / (sig * sig);   // a covariance carries the noise level
     const int64_t off = P.offsets[gal];
-    const bs_psf ps = P.psf[P.n_psf == 1 ? 0 : gal];
-    const float sqrt2 = 1.41421356237309515f;
-    const int rowf = row_floats(npad);
-    // one frequency row u at a time, so the scratch is a single column G[iy]
-    for (int u = 0; u < H; ++u) {
-        row_dft(P.data, P.data_f64, off, N, c, u, sm.tw, sm.G);
-        __syncthreads();
-        // D(u, v) = sum_iy G[iy] exp(-2 pi i v (iy - c) / N), scaled; transfer T(u, v)
-        float *row = sm.tab + (size_t)u * rowf;
-        const float scale = (u == 0 ? 1.0f : sqrt2) * gc.invN;
-        for (int vi = tid; vi < npad; vi += nth) {
-            float2 Dv = make_float2(0.f, 0.f);
-            float Tv = 0.f;
-            if (vi < N) {
-                const int v = vi - c;
-                const float2 D = col_dft(sm.G, N, c, v, sm.tw);
-                Dv = make_float2(D.x * scale, D.y * scale);
-                Tv = transfer_at(ps, gc, u, v, scale);
-            }
-            int ox, oy, ot;
-            slot_offsets(npad, vi >> 5, vi & 31, ox, oy, ot);
-            row[ox] = Dv.x;
-            row[oy] = Dv.y;
-            row[ot] = Tv;
-        }
-        __syncthreads();
-    }
+    if (P.data_f64)
+        row_spectra(static_cast<const double *>(P.data) + off, N, c, H, sm.tw, sm.tab, 96 * NCT);
+    else
+        row_spectra(static_cast<const float *>(P.data) + off, N, c, H, sm.tw, sm.tab, 96 * NCT);
+    __syncthreads();
+    spectrum_rows<NCT>(gc, sm.tw, sm.tab);
+    __syncthreads();
+    transfer_table<NCT>(gc, psf_const(P.psf[P.n_psf == 1 ? 0 : gal]), sm.tab);
+    __syncthreads();
     return true;
 }
 
@@ -1243,7 +1397,7 @@ __device__ __forceinline__ void fit_loop(const FitParams &P)
             continue;
         }
         GalCtx gc;
-        if (!setup_galaxy(P, gal, sm, gc)) {
+        if (!setup_galaxy<NC>(P, gal, sm, gc)) {
             if (threadIdx.x == 0 && P.status) P.status[gal] = 3;
             __syncthreads();
             if (P.done) publish_galaxy(P, gal);
@@ -1287,9 +1441,10 @@ __global__ void __launch_bounds__(256, 3) fit_kernel_r80(const FitParams P) { fi
 template <int NC>
 __global__ void __launch_bounds__(tc::kThreads, 1) fit_kernel_pix(const FitParams P) { fit_loop<NC, 3>(P); }
 
-// One CTA of 32 threads per point: stage the galaxy, then evaluate.
+// One point by one warp, the galaxy staged: the warp of the CTA's `slot` uses that slot's
+// phase table.
 template <int NC, int PROF>
-__device__ void point_eval(const FitParams &P, const GalCtx &gc, const SmemView &sm, int gal,
+__device__ void point_eval(const FitParams &P, const GalCtx &gc, const SmemView &sm, int gal, int slot,
                            const float *theta, double *logp, float *grad)
 {
     const int lane = threadIdx.x & 31;
@@ -1299,58 +1454,53 @@ __device__ void point_eval(const FitParams &P, const GalCtx &gc, const SmemView 
     float th[6];
 #pragma unroll
     for (int i = 0; i < 6; ++i) th[i] = theta[i];
+    float4 *xph = sm.xph + (size_t)slot * phase_stride(P.h_max);
     double v = -INFINITY;
     float gl = NAN;   // the gradient's component for this lane's parameter (lanes < 6)
     if (in_support(P, th)) {
-        if constexpr (PROF == 3) {
-            float g[6];
-            v = eval_pix<NC>(P, gc, sm, gal, sm.xph, vcol, th, g, true, nullptr);
-            gl = pick6(g, lane < 6 ? lane : 5);
-        } else if constexpr (PROF == 4) {
-            v = eval_dense<NC>(P, gc, dense_view(sm.kxr, P.h_max, P.npad, P.max_side, 0), gal, sm.kxr, sm.xph, vcol,
+        if constexpr (PROF == 4)
+            v = eval_dense<NC>(P, gc, dense_view(sm.kxr, P.h_max, P.npad, P.max_side, slot), gal, sm.kxr, xph, vcol,
                                th, gl, true);
-        } else {
-            v = eval_logpost<NC, PROF>(P, gc, sm.tab, sm.kxr, sm.xph, vcol, th, gl, true);
-        }
+        else
+            v = eval_logpost<NC, PROF>(P, gc, sm.tab, sm.kxr, xph, vcol, th, gl, true);
     }
-    if (threadIdx.x >= 32) return;   // the pixel path's other warps hold the same values
     if (lane == 0 && logp) *logp = v;
     if (grad && lane < 6) grad[lane] = gl;
 }
 
-template <int PROF>
-__global__ void __launch_bounds__(32) logpost_points_kernel(const FitParams P, int n_points,
-                                                            const int32_t *gal_index,
-                                                            const float *theta, double *logp,
-                                                            float *grad)
+// Points: a CTA stages a galaxy with all its warps and each warp then evaluates a point
+// of it.  Point i's CTA serves the run of points of the same galaxy from i to the end of
+// i's aligned block of kPointWarps points; a CTA whose point continues such a run has
+// nothing to do.  The staging (12 H N^2 flop against the evaluation's 33 H N) is
+// what the call costs.
+constexpr int kPointWarps = 4;
+
+template <int NC, int PROF>
+__global__ void __launch_bounds__(32 * kPointWarps, 5) logpost_points_kernel(const FitParams P, int n_points,
+                                                                          const int32_t *gal_index,
+                                                                          const float *theta, double *logp,
+                                                                          float *grad)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const SmemView sm = smem_view(smem_raw, P.h_max, P.npad, P.max_side, 1);
-    for (int i = blockIdx.x; i < n_points; i += gridDim.x) {
-        const int gal = gal_index[i];
-        if (gal < 0 || gal >= P.n_gal || !side_ok(P, P.side[gal])) {
-            if (threadIdx.x == 0 && logp) logp[i] = NAN;
-            if (grad && threadIdx.x < 6) grad[(size_t)i * 6 + threadIdx.x] = NAN;
-            continue;
-        }
-        GalCtx gc;
-        if (!setup_galaxy(P, gal, sm, gc)) {
-            if (threadIdx.x == 0 && logp) logp[i] = NAN;
-            if (grad && threadIdx.x < 6) grad[(size_t)i * 6 + threadIdx.x] = NAN;
-            continue;
-        }
-        if constexpr (PROF == 4) dense_setup(P, gc, sm, 1);
-        const float *th = theta + (size_t)i * 6;
-        double *lp = logp ? logp + i : nullptr;
-        float *gr = grad ? grad + (size_t)i * 6 : nullptr;
-        switch (P.npad >> 5) {     // the table layout follows the launch's slot count
-            case 1: point_eval<1, PROF>(P, gc, sm, gal, th, lp, gr); break;
-            case 2: point_eval<2, PROF>(P, gc, sm, gal, th, lp, gr); break;
-            case 3: point_eval<3, PROF>(P, gc, sm, gal, th, lp, gr); break;
-            default: point_eval<4, PROF>(P, gc, sm, gal, th, lp, gr); break;
-        }
-        __syncthreads();
+    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
+    const SmemView sm = smem_view(smem_raw, P.h_max, P.npad, P.max_side, warps);
+    const int i = blockIdx.x;
+    const int gal = gal_index[i];
+    if (i % warps != 0 && gal_index[i - 1] == gal) return;
+    int end = i + 1;
+    while (end < n_points && end % warps != 0 && gal_index[end] == gal) ++end;
+    GalCtx gc;
+    const bool ok = gal >= 0 && gal < P.n_gal && side_ok(P, P.side[gal]) && setup_galaxy<NC>(P, gal, sm, gc);
+    const int k = i + warp;
+    if (!ok) {
+        if (k < end && (threadIdx.x & 31) == 0 && logp) logp[k] = NAN;
+        if (k < end && grad && (threadIdx.x & 31) < 6) grad[(size_t)k * 6 + (threadIdx.x & 31)] = NAN;
+        return;
     }
+    if constexpr (PROF == 4) dense_setup(P, gc, sm, warps);
+    if (k < end)
+        point_eval<NC, PROF>(P, gc, sm, gal, warp, theta + (size_t)k * 6, logp ? logp + k : nullptr,
+                             grad ? grad + (size_t)k * 6 : nullptr);
 }
 
 // The pixel path's points: one CTA of eight warps per point; the first group of four
@@ -1368,7 +1518,7 @@ __global__ void __launch_bounds__(tc::kThreads, 1) logpost_points_pix_kernel(con
     for (int i = blockIdx.x; i < n_points; i += gridDim.x) {
         const int gal = gal_index[i];
         GalCtx gc;
-        const bool ok = gal >= 0 && gal < P.n_gal && side_ok(P, P.side[gal]) && setup_galaxy(P, gal, sm, gc);
+        const bool ok = gal >= 0 && gal < P.n_gal && side_ok(P, P.side[gal]) && setup_galaxy<NC>(P, gal, sm, gc);
         if (!ok) {
             if (threadIdx.x == 0 && logp) logp[i] = NAN;
             if (grad && threadIdx.x < 6) grad[(size_t)i * 6 + threadIdx.x] = NAN;

@@ -41,11 +41,22 @@ FitKernel kernel_for(int profile, int max_side)
     return profile == BS_PROFILE_SPERGEL ? prof_kernel<1>(max_side) : prof_kernel<2>(max_side);
 }
 
+template <int PROF>
+PointsKernel prof_points(int max_side)
+{
+    switch ((max_side + 31) / 32) {
+        case 1: return logpost_points_kernel<1, PROF>;
+        case 2: return logpost_points_kernel<2, PROF>;
+        case 3: return logpost_points_kernel<3, PROF>;
+        default: return logpost_points_kernel<4, PROF>;
+    }
+}
+
 PointsKernel points_for(int profile, int max_side)
 {
     if (is_pix(profile)) return max_side <= 31 ? logpost_points_pix_kernel<1> : logpost_points_pix_kernel<2>;
-    if (profile == 4) return logpost_points_kernel<4>;
-    return profile == BS_PROFILE_SPERGEL ? logpost_points_kernel<1> : logpost_points_kernel<2>;
+    if (profile == 4) return logpost_points_kernel<1, 4>;
+    return profile == BS_PROFILE_SPERGEL ? prof_points<1>(max_side) : prof_points<2>(max_side);
 }
 
 // Dynamic shared memory of a launch: the pixel-weight path adds the transforms'
@@ -127,13 +138,17 @@ cudaError_t launch_fit_profile(const FitParams &p, int grid, cudaStream_t stream
 cudaError_t launch_logpost_points_profile(const FitParams &p, int n_points, const int32_t *gal_index,
                                           const float *theta, double *logp, float *grad, cudaStream_t stream)
 {
-    const size_t smem = smem_for(p.profile, p.max_side, 1);
+    const int warps = p.profile == 4 ? 1 : kPointWarps;
+    const size_t smem = smem_for(p.profile, p.max_side, warps);
     PointsKernel k = points_for(p.profile, p.max_side);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int grid = n_points < 4096 ? n_points : 4096;
-    if (grid <= 0) return cudaSuccess;
-    k<<<grid, is_pix(p.profile) ? kPixThreads : 32, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
+    if (is_pix(p.profile)) {
+        const int grid = n_points < 4096 ? n_points : 4096;
+        k<<<grid, kPixThreads, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
+    } else {
+        k<<<n_points, 32 * warps, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
+    }
     bs::count_launches(1);
     return cudaGetLastError();
 }
