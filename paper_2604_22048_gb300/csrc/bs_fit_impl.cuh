@@ -1083,8 +1083,7 @@ __device__ __forceinline__ bool trajectory(const FitParams &P, const GalCtx &gc,
             v = eval_pix<NC>(P, gc, sm, gal, xph_c, vcol, x, gg, l == nst - 1, nullptr);
             gp = pick6(gg, pi);
         } else if constexpr (PROF == 4) {
-            v = eval_dense<NC>(P, gc, dense_view(sm.kxr, P.h_max, P.npad, P.max_side, slot), gal, sm.kxr, xph_c,
-                               vcol, x, gp, l == nst - 1);
+            dense_round<NC>(P, gc, sm, gal, cta_chains(P), true, slot, vcol, x, gp, l == nst - 1, v);
         } else {
             v = eval_logpost<NC, PROF>(P, gc, sm.tab, sm.kxr, xph_c, vcol, x, gp, l == nst - 1);
         }
@@ -1417,8 +1416,13 @@ __device__ __forceinline__ void fit_loop(const FitParams &P)
             __syncthreads();
             if (threadIdx.x == 0 && *px.abort && P.status) P.status[gal] = 4;
         } else {
-            if constexpr (PROF == 4) dense_setup(P, gc, sm, cc);
+            if constexpr (PROF == 4)
+                dense_setup(P, gc, sm, dense_view(sm.kxr, P.h_max, P.npad, P.max_side), cc);
             if (warp < cc) run_chain<NC, PROF>(P, gc, sm, gal, s_grp * cc + warp, warp);
+            if constexpr (PROF == 4) {
+                const float vcol[1] = {(float)((int)(threadIdx.x & 31) - gc.c)};
+                dense_join<NC>(P, gc, sm, gal, cc, warp, vcol);
+            }
         }
         __syncthreads();
         if (P.done) publish_galaxy(P, gal);
@@ -1441,6 +1445,10 @@ __global__ void __launch_bounds__(256, 3) fit_kernel_r80(const FitParams P) { fi
 template <int NC>
 __global__ void __launch_bounds__(tc::kThreads, 1) fit_kernel_pix(const FitParams P) { fit_loop<NC, 3>(P); }
 
+// The dense covariance: one CTA of 16 warps per galaxy, its chains in step (dense_round).
+template <int NC>
+__global__ void __launch_bounds__(32 * kDenseWarps, 1) fit_kernel_dense(const FitParams P) { fit_loop<NC, 4>(P); }
+
 // One point by one warp, the galaxy staged: the warp of the CTA's `slot` uses that slot's
 // phase table.
 template <int NC, int PROF>
@@ -1458,11 +1466,7 @@ __device__ void point_eval(const FitParams &P, const GalCtx &gc, const SmemView 
     double v = -INFINITY;
     float gl = NAN;   // the gradient's component for this lane's parameter (lanes < 6)
     if (in_support(P, th)) {
-        if constexpr (PROF == 4)
-            v = eval_dense<NC>(P, gc, dense_view(sm.kxr, P.h_max, P.npad, P.max_side, slot), gal, sm.kxr, xph, vcol,
-                               th, gl, true);
-        else
-            v = eval_logpost<NC, PROF>(P, gc, sm.tab, sm.kxr, xph, vcol, th, gl, true);
+        v = eval_logpost<NC, PROF>(P, gc, sm.tab, sm.kxr, xph, vcol, th, gl, true);
     }
     if (lane == 0 && logp) *logp = v;
     if (grad && lane < 6) grad[lane] = gl;
@@ -1475,32 +1479,74 @@ __device__ void point_eval(const FitParams &P, const GalCtx &gc, const SmemView 
 // what the call costs.
 constexpr int kPointWarps = 4;
 
+// The run of points of point i's CTA: [i, end), or false when an earlier one holds it.
+__device__ __forceinline__ bool point_run(int n_points, const int32_t *gal_index, int i, int &gal, int &end)
+{
+    gal = gal_index[i];
+    if (i % kPointWarps != 0 && gal_index[i - 1] == gal) return false;
+    end = i + 1;
+    while (end < n_points && end % kPointWarps != 0 && gal_index[end] == gal) ++end;
+    return true;
+}
+
 template <int NC, int PROF>
 __global__ void __launch_bounds__(32 * kPointWarps, 5) logpost_points_kernel(const FitParams P, int n_points,
-                                                                          const int32_t *gal_index,
-                                                                          const float *theta, double *logp,
-                                                                          float *grad)
+                                                                             const int32_t *gal_index,
+                                                                             const float *theta, double *logp,
+                                                                             float *grad)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
-    const SmemView sm = smem_view(smem_raw, P.h_max, P.npad, P.max_side, warps);
-    const int i = blockIdx.x;
-    const int gal = gal_index[i];
-    if (i % warps != 0 && gal_index[i - 1] == gal) return;
-    int end = i + 1;
-    while (end < n_points && end % warps != 0 && gal_index[end] == gal) ++end;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const SmemView sm = smem_view(smem_raw, P.h_max, P.npad, P.max_side, kPointWarps);
+    int gal, end;
+    if (!point_run(n_points, gal_index, blockIdx.x, gal, end)) return;
     GalCtx gc;
     const bool ok = gal >= 0 && gal < P.n_gal && side_ok(P, P.side[gal]) && setup_galaxy<NC>(P, gal, sm, gc);
-    const int k = i + warp;
+    const int k = blockIdx.x + warp;
+    if (k >= end) return;
     if (!ok) {
-        if (k < end && (threadIdx.x & 31) == 0 && logp) logp[k] = NAN;
-        if (k < end && grad && (threadIdx.x & 31) < 6) grad[(size_t)k * 6 + (threadIdx.x & 31)] = NAN;
+        if (lane == 0 && logp) logp[k] = NAN;
+        if (grad && lane < 6) grad[(size_t)k * 6 + lane] = NAN;
         return;
     }
-    if constexpr (PROF == 4) dense_setup(P, gc, sm, warps);
-    if (k < end)
-        point_eval<NC, PROF>(P, gc, sm, gal, warp, theta + (size_t)k * 6, logp ? logp + k : nullptr,
-                             grad ? grad + (size_t)k * 6 : nullptr);
+    point_eval<NC, PROF>(P, gc, sm, gal, warp, theta + (size_t)k * 6, logp ? logp + k : nullptr,
+                         grad ? grad + (size_t)k * 6 : nullptr);
+}
+
+// The dense covariance's points: the same runs, a point per chain slot of one round.
+template <int NC>
+__global__ void __launch_bounds__(32 * kDenseWarps, 1) logpost_points_dense_kernel(const FitParams P, int n_points,
+                                                                                   const int32_t *gal_index,
+                                                                                   const float *theta, double *logp,
+                                                                                   float *grad)
+{
+    static_assert(kPointWarps == kDenseChains, "a run of points fills the chain slots");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const SmemView sm = smem_view(smem_raw, P.h_max, P.npad, P.max_side, kDenseChains);
+    int gal, end;
+    if (!point_run(n_points, gal_index, blockIdx.x, gal, end)) return;
+    GalCtx gc;
+    const bool ok = gal >= 0 && gal < P.n_gal && side_ok(P, P.side[gal]) && setup_galaxy<NC>(P, gal, sm, gc);
+    const int k = blockIdx.x + warp;
+    double v = ok ? -INFINITY : NAN;
+    float gl = NAN;
+    if (ok) {
+        dense_setup(P, gc, sm, dense_view(sm.kxr, P.h_max, P.npad, P.max_side), kDenseChains);
+        const float vcol[1] = {(float)(lane - gc.c)};
+        float th[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (k < end)
+#pragma unroll
+            for (int i = 0; i < 6; ++i) th[i] = theta[(size_t)k * 6 + i];
+        const bool active = k < end && in_support(P, th);
+        double lp = 0.0;
+        dense_round<NC>(P, gc, sm, gal, kDenseChains, active, warp, vcol, th, gl, true, lp);
+        if (active) v = lp;
+        else gl = NAN;
+    }
+    if (k >= end) return;
+    if (lane == 0 && logp) logp[k] = v;
+    if (grad && lane < 6) grad[(size_t)k * 6 + lane] = gl;
 }
 
 // The pixel path's points: one CTA of eight warps per point; the first group of four

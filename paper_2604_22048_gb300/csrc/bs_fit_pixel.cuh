@@ -371,74 +371,157 @@ __device__ void pix_drain(const FitParams &P, const GalCtx &gc, const SmemView &
 // product y = P (d - m), N^4 multiply-adds per evaluation reading P from L2, beside
 // which the two separable transforms are small; and P amplifies rounding errors of
 // the rendered model m, so the transforms stay in FP32 on the CUDA cores (kernel
-// instance PROF 4, one warp per chain).  The gradient is the half-plane pass on the
-// effective spectrum D' = M + DFT(y) (scaled as the table).
+// instance PROF 4).  The gradient is the half-plane pass on the effective spectrum
+// D' = M + DFT(y) (scaled as the table).
 //
-// After the shared region: the twiddles exp(+2 pi i m / N) (max_side float2) and,
-// per chain, a private copy of the table ([h_max][3 npad]: the D slots hold the
+// One CTA of 16 warps runs a galaxy's chains (at most 4), one evaluation of every chain at
+// a time: the first warp of each chain (its leader) runs the chain's logic, and all
+// warps meet in dense_round, where one read of P serves every chain.  The transforms'
+// rows are split over the warps of the chain (16 / n_chains), the product's columns over
+// all 16 warps; every output is summed by one lane in a fixed order, so a chain's draws
+// do not depend on the others.  The product is bound by the read of P (778 KB at 21 px,
+// from L2): 32 rows of loads are in flight per warp.
+// 64 galaxies of 21 px, 4 chains x (100 + 100), L <= 8: 332 ms with a warp per chain that
+// evaluated on its own (the product waiting for each row of P, transforms on 11 to 21 of 32
+// lanes), 23.8 ms now, the same draws bit for bit; issue 1.7 per cycle on the 64 SMs in use.
+//
+// After the shared region, in floats: the twiddles exp(+2 pi i m / N) (max_side float2),
+// the chains' requests, the residual images of the four chain slots interleaved (max_side^2
+// float4), and per chain a private copy of the table ([h_max][3 npad]: the D slots hold the
 // evaluation's effective spectrum, the T slots the transfer), the half-transformed
-// image ([h_max][max_side] float2), the residual image and its product with the
-// precision (max_side^2 floats each).  Sizes in floats, each chain's block a multiple
-// of 4 floats.
+// image ([h_max][max_side] float2) and the product with the precision (max_side^2).
+constexpr int kDenseWarps = 16;
+constexpr int kDenseChains = 4;
 __host__ __device__ __forceinline__ int dense_chain_floats(int h_max, int npad, int max_side)
 {
-    const int n = h_max * row_floats(npad) + 2 * h_max * max_side + 2 * max_side * max_side;
+    const int n = h_max * row_floats(npad) + 2 * h_max * max_side + max_side * max_side;
     return (n + 3) & ~3;
 }
+__host__ __device__ __forceinline__ int dense_tw_floats(int max_side) { return (2 * max_side + 3) & ~3; }
 __host__ __device__ __forceinline__ size_t dense_region_bytes(int h_max, int npad, int max_side, int n_chains)
 {
-    return ((size_t)2 * ((max_side + 1) & ~1) + (size_t)n_chains * dense_chain_floats(h_max, npad, max_side)) *
+    return ((size_t)dense_tw_floats(max_side) + 8 * kDenseChains + 4 * (size_t)max_side * max_side +
+            (size_t)n_chains * dense_chain_floats(h_max, npad, max_side)) *
            sizeof(float);
 }
 struct DenseView {
     float2 *tw;    // [max_side] exp(+2 pi i m / N)
-    float *tab;    // this chain's table
-    float2 *G;     // [h_max][max_side]
-    float *rb;     // [max_side^2] residual d - m
-    float *yb;     // [max_side^2] precision x residual
+    float *req;    // [4][8] per chain: theta (6), request (0 none, 1 gradient, 2 and log posterior)
+    float4 *rb;    // [max_side^2] residuals d - m of the four chain slots
+    float *chain0; // the chains' blocks, `stride` floats each:
+    int stride, o_G, o_y;
+    __device__ __forceinline__ float *tab(int c) const { return chain0 + (size_t)c * stride; }
+    __device__ __forceinline__ float2 *G(int c) const   // [h_max][max_side]
+    {
+        return reinterpret_cast<float2 *>(tab(c) + o_G);
+    }
+    __device__ __forceinline__ float *yb(int c) const { return tab(c) + o_y; }   // [max_side^2] precision x residual
 };
 // kxr ends at h_max + 1 float2 after its start; the region follows, 16-byte aligned.
-__device__ __forceinline__ DenseView dense_view(float2 *kxr, int h_max, int npad, int max_side, int chain)
+__device__ __forceinline__ DenseView dense_view(float2 *kxr, int h_max, int npad, int max_side)
 {
     float *base = reinterpret_cast<float *>(kxr + ((h_max + 2) & ~1));
     DenseView v;
     v.tw = reinterpret_cast<float2 *>(base);
-    float *c0 = base + 2 * ((max_side + 1) & ~1) + (size_t)chain * dense_chain_floats(h_max, npad, max_side);
-    v.tab = c0;
-    v.G = reinterpret_cast<float2 *>(c0 + (size_t)h_max * row_floats(npad));
-    v.rb = reinterpret_cast<float *>(v.G + (size_t)h_max * max_side);
-    v.yb = v.rb + max_side * max_side;
+    v.req = base + dense_tw_floats(max_side);
+    v.rb = reinterpret_cast<float4 *>(v.req + 8 * kDenseChains);
+    v.chain0 = v.req + 8 * kDenseChains + 4 * max_side * max_side;
+    v.stride = dense_chain_floats(h_max, npad, max_side);
+    v.o_G = h_max * row_floats(npad);
+    v.o_y = v.o_G + 2 * h_max * max_side;
     return v;
 }
 
-// Per-galaxy set-up of the dense path (all threads): the twiddles, and each
-// chain's private table from the staged one (transfer, zero spectrum).
-__device__ void dense_setup(const FitParams &P, const GalCtx &gc, const SmemView &sm, int n_tables)
+// Per-galaxy set-up of the dense path (all threads): the twiddles, no requests, zero
+// residuals of the slots without a chain, and each chain's private table from the staged
+// one (transfer, zero spectrum).
+__device__ void dense_setup(const FitParams &P, const GalCtx &gc, const SmemView &sm, const DenseView &dv, int n_tables)
 {
     const int tid = threadIdx.x, nth = blockDim.x;
-    const DenseView p0 = dense_view(sm.kxr, P.h_max, P.npad, P.max_side, 0);
     for (int m = tid; m < gc.N; m += nth) {
         float s, co;
         sincospif(2.0f * (float)m * gc.invN, &s, &co);
-        p0.tw[m] = make_float2(co, s);
+        dv.tw[m] = make_float2(co, s);
     }
-    const int rowf = row_floats(P.npad);
-    const int nrow = gc.H * rowf;
+    for (int i = tid; i < 8 * kDenseChains; i += nth) dv.req[i] = 0.f;
+    for (int i = tid; i < gc.N * gc.N; i += nth) dv.rb[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int nrow = gc.H * row_floats(P.npad);
     for (int t = 0; t < n_tables; ++t) {
-        float *dst = dense_view(sm.kxr, P.h_max, P.npad, P.max_side, t).tab;
+        float *dst = dv.tab(t);
         for (int i = tid; i < nrow; i += nth) dst[i] = sm.tab[i];
     }
     __syncthreads();
 }
 
-template <int NC>
-__device__ double eval_dense(const FitParams &P, const GalCtx &gc, const DenseView &pv, int gal,
-                           const float2 *__restrict__ kxr, float4 *__restrict__ xph, const float vcol[NC],
-                           const float th[6], float &gi, bool want_ll)
+// y = P r of every chain slot (all warps): the precision is symmetric, so y_a = sum_b
+// P[b][a] r_b, and a warp takes 32 columns a at a time, each row b of them one coalesced
+// load used for the four slots.
+__device__ __forceinline__ void dense_product(const FitParams &P, const GalCtx &gc, const DenseView &dv, int gal,
+                                              int n_slots)
 {
+    constexpr int kAhead = 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    const int n = gc.N * gc.N;
+    const float *__restrict__ Pg = P.pix_prec + P.prec_offs[gal];
+    for (int a0 = 32 * warp; a0 < n; a0 += 32 * nwarp) {
+        const int a = a0 + lane;
+        const float *col = Pg + min(a, n - 1);
+        float2 y01 = make_float2(0.f, 0.f), y23 = make_float2(0.f, 0.f);
+        const float4 *r = dv.rb;
+        int b0 = 0;
+        for (; b0 + kAhead <= n; b0 += kAhead) {
+            float p[kAhead];
+#pragma unroll
+            for (int t = 0; t < kAhead; ++t) p[t] = __ldg(col + t * n);
+            col += kAhead * n;
+#pragma unroll
+            for (int t = 0; t < kAhead; ++t) {
+                const float4 rv = r[t];
+                y01 = fma2(f2(p[t]), make_float2(rv.x, rv.y), y01);
+                y23 = fma2(f2(p[t]), make_float2(rv.z, rv.w), y23);
+            }
+            r += kAhead;
+        }
+        {
+            float p[kAhead];
+#pragma unroll
+            for (int t = 0; t < kAhead; ++t) p[t] = b0 + t < n ? __ldg(col + t * n) : 0.f;
+#pragma unroll
+            for (int t = 0; t < kAhead; ++t) {
+                if (b0 + t < n) {
+                    const float4 rv = r[t];
+                    y01 = fma2(f2(p[t]), make_float2(rv.x, rv.y), y01);
+                    y23 = fma2(f2(p[t]), make_float2(rv.z, rv.w), y23);
+                }
+            }
+        }
+        if (a < n) {
+            const float y[4] = {y01.x, y01.y, y23.x, y23.y};
+#pragma unroll
+            for (int c = 0; c < kDenseChains; ++c)
+                if (c < n_slots) dv.yb(c)[a] = y[c];
+        }
+    }
+}
+
+// The model image's half of a round, of one chain's rows u (all warps of the chain): (a) its
+// half spectrum Mt into the D slots of the chain's table, (b1) its column transform into G,
+// G(u, iy) of rows u > 0 as (2 Re, -2 Im) (an exact scaling: the row transform's factors).
+// Row u = k + r nk of the chain's warp k; UB rows share a twiddle.
+template <int UB>
+__device__ __forceinline__ void dense_model(const FitParams &P, const GalCtx &gc, const SmemView &sm, const DenseView &dv,
+                                            int s, int k, int nk)
+{
+    constexpr int rowf = 96;
     const int lane = threadIdx.x & 31;
-    const int N = gc.N, H = gc.H, c = gc.c, npad = P.npad;
-    const int rowf = row_floats(npad);
+    const int N = gc.N, H = gc.H, c = gc.c;
+    float *tab = dv.tab(s);
+    float2 *G = dv.G(s);
+    const bool own = lane < N;
+    const int x = min(lane, N - 1) - c, xs = x < 0 ? x + N : x;   // this lane's row, centred, and mod N
+    float th[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) th[i] = dv.req[8 * s + i];
     const float F = exp10f(th[0]);
     const float r0 = exp10f(th[1]) * (1.0f / kHlrOverR0);
     const float r02 = r0 * r0;
@@ -448,169 +531,250 @@ __device__ double eval_dense(const FitParams &P, const GalCtx &gc, const DenseVi
     const float al = r02 * (1.0f + E + 2.0f * e1) * Pq;
     const float be = r02 * (1.0f + E - 2.0f * e1) * Pq;
     const float ga = r02 * 4.0f * e2 * Pq;
-    const float sqrt2 = 1.41421356237309515f;
-    for (int u = lane; u < H; u += 32) {
-        float sx, cx;
-        sincospi_sfu(-2.0f * th[4] * (float)u * gc.invN, &sx, &cx);
-        xph[u] = make_float4(cx, sx, -sx, 0.0f);
-    }
-    __syncwarp();
-    // (a) the model's half spectrum Mt = Tt F f(s) X(u) Y(v) into the D slots
+    const float v = (float)(lane - c);
+    float sy, cy;
+    sincospi_sfu(-2.0f * th[5] * v * gc.invN, &sy, &cy);
+    const float Yr = F * cy, Yi = F * sy;
+    const float ky = v * gc.dk;
+    const float cst = fmaf(be * ky, ky, 1.0f), gky = ga * ky;
+    for (int ub = k; ub < H; ub += UB * nk) {
 #pragma unroll
-    for (int j = 0; j < NC; ++j) {
-        const int vi = lane + 32 * j;
-        float sy, cy;
-        sincospi_sfu(-2.0f * th[5] * vcol[j] * gc.invN, &sy, &cy);
-        const float Yr = F * cy, Yi = F * sy;
-        const float ky = vcol[j] * gc.dk;
-        const float cst = fmaf(be * ky, ky, 1.0f), gky = ga * ky;
-        int ox, oy, ot;
-        slot_offsets(npad, j, lane, ox, oy, ot);
-        for (int u = 0; u < H; ++u) {
-            float *row = pv.tab + (size_t)u * rowf;
-            const float kx = kxr[u].x;
-            const float s = fmaf(fmaf(al, kx, gky), kx, cst);
-            const float rs = rsqrtf(s);
-            const float A = row[ot] * rs * rs * rs;
-            const float4 X = xph[u];
-            const float Pr = X.x * Yr - X.y * Yi, Pi = X.x * Yi + X.y * Yr;
-            const float mr = vi < N ? A * Pr : 0.0f, mi = vi < N ? A * Pi : 0.0f;
-            row[ox] = mr;
-            row[oy] = mi;
-            // unscaled M(u, v) = Mt / scale_u, contiguous, for the inverse transform
-            const float inv_scale = (float)N * (u == 0 ? 1.0f : 0.70710678118654752f);
-            if (vi < N) pv.G[(size_t)u * N + vi] = make_float2(mr * inv_scale, mi * inv_scale);
-        }
-    }
-    __syncwarp();
-    // (b1) G(u, iy) = sum_v M(u, v) exp(+2 pi i v (iy - c) / N), in place row by
-    // row (a row's outputs need only that row's M; lanes over iy, at most 2 each)
-    for (int u = 0; u < H; ++u) {
-        float2 *grow = pv.G + (size_t)u * N;
-        float2 res[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int iy = lane + 32 * r;
-            if (iy < N) {
-                const int step = iy - c;
-                float re = 0.f, im = 0.f;
-                int k = ((-c * step) % N + N) % N;
-                const int dk = (step % N + N) % N;
-                for (int vi = 0; vi < N; ++vi) {
-                    const float2 mv = grow[vi];
-                    const float2 t = pv.tw[k];
-                    re = fmaf(mv.x, t.x, fmaf(-mv.y, t.y, re));
-                    im = fmaf(mv.x, t.y, fmaf(mv.y, t.x, im));
-                    k += dk;
-                    if (k >= N) k -= N;
-                }
-                res[r] = make_float2(re, im);
+        for (int r = 0; r < UB; ++r) {
+            const int u = ub + r * nk;
+            if (u < H) {
+                float *row = tab + u * rowf;
+                const float kx = sm.kxr[u].x;
+                const float sarg = fmaf(fmaf(al, kx, gky), kx, cst);
+                const float rs = rsqrtf(sarg);
+                const float A = row[64 + lane] * rs * rs * rs;
+                float sx, cx;
+                sincospi_sfu(-2.0f * th[4] * (float)u * gc.invN, &sx, &cx);
+                const float Pr = cx * Yr - sx * Yi, Pi = cx * Yi + sx * Yr;
+                const float mr = own ? A * Pr : 0.0f, mi = own ? A * Pi : 0.0f;
+                *reinterpret_cast<float2 *>(row + 2 * lane) = make_float2(mr, mi);
+                const float inv_scale = (float)N * (u == 0 ? 1.0f : 0.70710678118654752f);
+                if (own) G[u * N + lane] = make_float2(mr * inv_scale, mi * inv_scale);
             }
         }
         __syncwarp();
+        // G(u, iy) = sum_v M(u, v) exp(+2 pi i v (iy - c) / N), in place (lane = iy)
+        float re[UB], im[UB];
+        const float2 *g[UB];
 #pragma unroll
-        for (int r = 0; r < 2; ++r)
-            if (lane + 32 * r < N) grow[lane + 32 * r] = res[r];
-        __syncwarp();
-    }
-    // (b2) per pixel row: m(ix, iy) and the residual r = d - m; y = P r needs every row of r
-    const int64_t off = P.offsets[gal];
-    const float invN2 = gc.invN * gc.invN;
-    double chi = 0.0;
-    for (int iy = 0; iy < N; ++iy) {
-        for (int ix = lane; ix < N; ix += 32) {
-            const int dk = ((ix - c) % N + N) % N;      // u (ix - c) mod N, advanced per u
-            int k = dk;
-            float acc = pv.G[iy].x;                     // u = 0 (real)
-            for (int u = 1; u < H; ++u) {
-                const float2 gv = pv.G[(size_t)u * N + iy];
-                const float2 t = pv.tw[k];
-                acc = fmaf(2.0f * gv.x, t.x, fmaf(-2.0f * gv.y, t.y, acc));
-                k += dk;
-                if (k >= N) k -= N;
-            }
-            pv.rb[iy * N + ix] = load_pix(P.data, P.data_f64, off + (int64_t)iy * N + ix) - acc * invN2;
+        for (int r = 0; r < UB; ++r) {
+            re[r] = im[r] = 0.f;
+            g[r] = G + min(ub + r * nk, H - 1) * N;
         }
-    }
-    __syncwarp();
-    {
-        // y = Sigma^-1 r: the precision is symmetric, so y_a = sum_b P[b][a] r_b with
-        // lanes over a reads each row b of it coalesced (from L2: tens of
-        // evaluations of the galaxy's chains share it); chi^2 = r.y
-        constexpr int kSlots = (kDenseMaxSide * kDenseMaxSide + 31) / 32;
-        const int n = N * N;
-        const float *Pg = P.pix_prec + P.prec_offs[gal];
-        float yv[kSlots];
+        int i1 = ((N - xs) * c) % N;     // -c (iy - c) mod N
+#pragma unroll 2
+        for (int vi = 0; vi < N; ++vi) {
+            const float2 t = dv.tw[i1];
 #pragma unroll
-        for (int j = 0; j < kSlots; ++j) yv[j] = 0.f;
-        for (int b = 0; b < n; ++b) {
-            const float rb = pv.rb[b];
-            const float *prow = Pg + (size_t)b * n;
-#pragma unroll
-            for (int j = 0; j < kSlots; ++j) {
-                const int a = lane + 32 * j;
-                if (a < n) yv[j] = fmaf(__ldg(prow + a), rb, yv[j]);
+            for (int r = 0; r < UB; ++r) {
+                const float2 mv = g[r][vi];
+                re[r] = fmaf(mv.x, t.x, fmaf(-mv.y, t.y, re[r]));
+                im[r] = fmaf(mv.x, t.y, fmaf(mv.y, t.x, im[r]));
             }
-        }
-#pragma unroll
-        for (int j = 0; j < kSlots; ++j) {
-            const int a = lane + 32 * j;
-            if (a < n) {
-                pv.yb[a] = yv[j];
-                chi += (double)pv.rb[a] * (double)yv[j];
-            }
+            i1 += xs;
+            if (i1 >= N) i1 -= N;
         }
         __syncwarp();
-        // Q(u, iy) = sum_ix y(ix, iy) exp(-2 pi i u (ix - c) / N), one row iy at a time
-        for (int iy = 0; iy < N; ++iy) {
-            const float *yrow = pv.yb + iy * N;
-            for (int u = lane; u < H; u += 32) {
-                float re = 0.f, im = 0.f;
-                int k = ((u * c) % N + N) % N;           // -u (ix - c) at ix = 0
-                const int dk = (N - u % N) % N;
-                for (int ix = 0; ix < N; ++ix) {
-                    const float r = yrow[ix];
-                    const float2 t = pv.tw[k];
-                    re = fmaf(r, t.x, re);
-                    im = fmaf(r, t.y, im);
-                    k += dk;
-                    if (k >= N) k -= N;
-                }
-                pv.G[(size_t)u * N + iy] = make_float2(re, im);
-            }
+#pragma unroll
+        for (int r = 0; r < UB; ++r) {
+            const int u = ub + r * nk;
+            if (u < H && own) G[u * N + lane] = u ? make_float2(2.0f * re[r], -2.0f * im[r]) : make_float2(re[r], im[r]);
         }
-        __syncwarp();
     }
-    // (b3) D' = Mt + scale_u R(u, v), R(u, v) = sum_iy Q(u, iy) exp(-2 pi i v (iy - c) / N);
-    // the H x N (u, v) outputs spread over the lanes
-    for (int t = lane; t < H * N; t += 32) {
-        const int u = t / N, vi = t - u * N, v = vi - c;
-        const int dk = ((-v) % N + N) % N;
-        int k = ((v * c) % N + N) % N;                  // -v (iy - c) at iy = 0
-        const float2 *qrow = pv.G + (size_t)u * N;
-        float re = 0.f, im = 0.f;
-        for (int iy = 0; iy < N; ++iy) {
-            const float2 q = qrow[iy];
-            const float2 tw = pv.tw[k];
-            re = fmaf(q.x, tw.x, fmaf(-q.y, tw.y, re));
-            im = fmaf(q.x, tw.y, fmaf(q.y, tw.x, im));
-            k += dk;
-            if (k >= N) k -= N;
-        }
-        int ox, oy, ot;
-        slot_offsets(npad, vi >> 5, vi & 31, ox, oy, ot);
-        const float scale = (u == 0 ? 1.0f : sqrt2) * gc.invN;
-        float *row = pv.tab + (size_t)u * rowf;
-        row[ox] = fmaf(scale, re, row[ox]);
-        row[oy] = fmaf(scale, im, row[oy]);
-    }
-    __syncwarp();
-    // (c) the gradient from the half-plane pass on the effective spectrum
-    eval_logpost<NC, 0>(P, gc, pv.tab, kxr, xph, vcol, th, gi, false);
-    if (!want_ll) return 0.0;
-    const double chi2 = warp_sum_d(chi);
-    const float lprior = P.prior_const - 0.5f * (th[4] * th[4] + th[5] * th[5]) * P.inv_sxy2 +
-                         2.0f * log1pf(-E) - 0.5f * E * P.inv_se2;
-    return -0.5 * chi2 * (double)gc.inv_b + (double)lprior;
 }
 
+// (b2) The chain's rows iy of m (lane = ix) and the residual r = d - m.
+template <int UB>
+__device__ __forceinline__ void dense_residual(const FitParams &P, const GalCtx &gc, const DenseView &dv, int gal, int s,
+                                               int k, int nk)
+{
+    const int lane = threadIdx.x & 31;
+    const int N = gc.N, H = gc.H, c = gc.c;
+    const float2 *G = dv.G(s);
+    const int x = min(lane, N - 1) - c, xs = x < 0 ? x + N : x;
+    const int64_t off = P.offsets[gal];
+    const float invN2 = gc.invN * gc.invN;
+    for (int yb = k; yb < N; yb += UB * nk) {
+        float acc[UB];
+        const float2 *g[UB];
+#pragma unroll
+        for (int r = 0; r < UB; ++r) {
+            g[r] = G + min(yb + r * nk, N - 1);
+            acc[r] = g[r]->x;                    // u = 0 (real)
+        }
+        int i1 = xs;                             // u (ix - c) mod N, advanced per u
+#pragma unroll 2
+        for (int u = 1; u < H; ++u) {
+            const float2 t = dv.tw[i1];
+#pragma unroll
+            for (int r = 0; r < UB; ++r) {
+                const float2 gv = g[r][u * N];
+                acc[r] = fmaf(gv.x, t.x, fmaf(gv.y, t.y, acc[r]));
+            }
+            i1 += xs;
+            if (i1 >= N) i1 -= N;
+        }
+#pragma unroll
+        for (int r = 0; r < UB; ++r) {
+            const int iy = yb + r * nk;
+            if (iy < N && lane < N)
+                reinterpret_cast<float *>(dv.rb + iy * N + lane)[s] =
+                    load_pix(P.data, P.data_f64, off + (int64_t)iy * N + lane) - acc[r] * invN2;
+        }
+    }
+}
+
+// The way back, of the chain's rows u: Q(u, iy) = sum_ix y(ix, iy) exp(-2 pi i u (ix - c) / N)
+// (lane = iy), then (b3) D' = Mt + scale_u R(u, v), R(u, v) = sum_iy Q(u, iy) exp(-2 pi i v (iy - c)
+// / N) (lane = v).
+template <int UB>
+__device__ __forceinline__ void dense_back(const GalCtx &gc, const DenseView &dv, int s, int k, int nk)
+{
+    constexpr int rowf = 96;
+    const int lane = threadIdx.x & 31;
+    const int N = gc.N, H = gc.H, c = gc.c;
+    float *tab = dv.tab(s);
+    float2 *G = dv.G(s);
+    const bool own = lane < N;
+    const int xl = min(lane, N - 1), x = xl - c, xs = x < 0 ? x + N : x;
+    const float *yrow = dv.yb(s) + xl * N;
+    for (int ub = k; ub < H; ub += UB * nk) {
+        float re[UB], im[UB];
+        int i1[UB], d1[UB];
+        float2 *g[UB];
+#pragma unroll
+        for (int r = 0; r < UB; ++r) {
+            const int u = min(ub + r * nk, H - 1);
+            re[r] = im[r] = 0.f;
+            i1[r] = (u * c) % N;                 // -u (ix - c) at ix = 0
+            d1[r] = u ? N - u : 0;
+            g[r] = G + u * N;
+        }
+#pragma unroll 2
+        for (int ix = 0; ix < N; ++ix) {
+            const float y = yrow[ix];
+#pragma unroll
+            for (int r = 0; r < UB; ++r) {
+                const float2 t = dv.tw[i1[r]];
+                re[r] = fmaf(y, t.x, re[r]);
+                im[r] = fmaf(y, t.y, im[r]);
+                i1[r] += d1[r];
+                if (i1[r] >= N) i1[r] -= N;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < UB; ++r)
+            if (ub + r * nk < H && own) g[r][lane] = make_float2(re[r], im[r]);
+        __syncwarp();
+        const int dk = xs ? N - xs : 0;
+        int i2 = (xs * c) % N;                   // -v (iy - c) at iy = 0
+#pragma unroll
+        for (int r = 0; r < UB; ++r) re[r] = im[r] = 0.f;
+#pragma unroll 2
+        for (int iy = 0; iy < N; ++iy) {
+            const float2 t = dv.tw[i2];
+#pragma unroll
+            for (int r = 0; r < UB; ++r) {
+                const float2 q = g[r][iy];
+                re[r] = fmaf(q.x, t.x, fmaf(-q.y, t.y, re[r]));
+                im[r] = fmaf(q.x, t.y, fmaf(q.y, t.x, im[r]));
+            }
+            i2 += dk;
+            if (i2 >= N) i2 -= N;
+        }
+#pragma unroll
+        for (int r = 0; r < UB; ++r) {
+            const int u = ub + r * nk;
+            if (u < H && own) {
+                const float scale = (u == 0 ? 1.0f : 1.41421356237309515f) * gc.invN;
+                float2 *d = reinterpret_cast<float2 *>(tab + u * rowf) + lane;
+                *d = make_float2(fmaf(scale, re[r], d->x), fmaf(scale, im[r], d->y));
+            }
+        }
+    }
+}
+
+// One evaluation of every chain that asks for one (all threads of the CTA).  A leader
+// (the first warp of chain `mine`) has its theta in th and passes active = true; every other warp,
+// and a leader whose chain has ended, passes active = false.  Returns false when no
+// chain asked (the evaluations of the galaxy are over); the leader receives its chain's
+// log posterior in lp (if want_ll) and its lane's component of the gradient in gi.
+template <int NC>
+__device__ bool dense_round(const FitParams &P, const GalCtx &gc, const SmemView &sm, int gal, int n_slots, bool active,
+                            int mine, const float vcol[NC], const float th[6], float &gi, bool want_ll, double &lp)
+{
+    static_assert(NC == 1, "stamps of at most 31 px: a lane is a row or a column of the stamp");
+    const DenseView dv = dense_view(sm.kxr, P.h_max, P.npad, P.max_side);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    const int N = gc.N, H = gc.H;
+    if (lane == 0 && warp < n_slots && warp == mine) {   // the leader of slot `mine` is warp `mine`
+        float *q = dv.req + 8 * mine;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) q[i] = active ? th[i] : 0.f;
+        q[6] = active ? (want_ll ? 2.f : 1.f) : 0.f;
+    }
+    __syncthreads();
+    bool any = false;
+    for (int s = 0; s < n_slots; ++s) any = any || dv.req[8 * s + 6] != 0.f;
+    if (!any) return false;
+    // this warp's share of one chain: member k of the nk warps of chain s (warps past
+    // nk n_slots take part in the product only); rows are taken in passes of as many as
+    // share them evenly (H <= 16 rows over at least 4 warps)
+    const int s = warp % n_slots, k = warp / n_slots, nk = nwarp / n_slots;
+    const bool in = k < nk && dv.req[8 * s + 6] != 0.f;
+    const int ub = (H + nk - 1) / nk;
+    if (in) {
+        if (ub <= 2) dense_model<2>(P, gc, sm, dv, s, k, nk);
+        else if (ub == 3) dense_model<3>(P, gc, sm, dv, s, k, nk);
+        else dense_model<4>(P, gc, sm, dv, s, k, nk);
+    }
+    __syncthreads();
+    if (in) {
+        if (ub <= 2) dense_residual<2>(P, gc, dv, gal, s, k, nk);
+        else if (ub == 3) dense_residual<3>(P, gc, dv, gal, s, k, nk);
+        else dense_residual<4>(P, gc, dv, gal, s, k, nk);
+    }
+    __syncthreads();
+    dense_product(P, gc, dv, gal, n_slots);
+    __syncthreads();
+    if (in) {
+        if (ub <= 2) dense_back<2>(gc, dv, s, k, nk);
+        else if (ub == 3) dense_back<3>(gc, dv, s, k, nk);
+        else dense_back<4>(gc, dv, s, k, nk);
+    }
+    __syncthreads();
+    if (!active) return true;
+    // (c) the leader: the gradient from the half-plane pass on the effective spectrum, and
+    // chi^2 = r.y
+    float4 *xph = sm.xph + (size_t)mine * phase_stride(P.h_max);
+    eval_logpost<NC, 0>(P, gc, dv.tab(mine), sm.kxr, xph, vcol, th, gi, false);
+    lp = 0.0;
+    if (want_ll) {
+        double chi = 0.0;
+        const float *yb = dv.yb(mine), *rb = reinterpret_cast<const float *>(dv.rb) + mine;
+        for (int a = lane; a < N * N; a += 32) chi += (double)rb[4 * a] * (double)yb[a];
+        const double chi2 = warp_sum_d(chi);
+        const float E = th[2] * th[2] + th[3] * th[3];
+        const float lprior = P.prior_const - 0.5f * (th[4] * th[4] + th[5] * th[5]) * P.inv_sxy2 +
+                             2.0f * log1pf(-E) - 0.5f * E * P.inv_se2;
+        lp = -0.5 * chi2 * (double)gc.inv_b + (double)lprior;
+    }
+    return true;
+}
+
+// Rounds without a chain of one's own, until no chain asks (a warp that leads none, or a
+// leader whose chain has ended).
+template <int NC>
+__device__ void dense_join(const FitParams &P, const GalCtx &gc, const SmemView &sm, int gal, int n_slots, int mine,
+                           const float vcol[NC])
+{
+    const float th[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float gi;
+    double lp;
+    while (dense_round<NC>(P, gc, sm, gal, n_slots, false, mine, vcol, th, gi, false, lp)) {
+    }
+}

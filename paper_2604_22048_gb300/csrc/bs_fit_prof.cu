@@ -37,7 +37,7 @@ bool is_pix(int profile) { return profile == 3; }
 FitKernel kernel_for(int profile, int max_side)
 {
     if (profile == 3) return pix_kernel(max_side);
-    if (profile == 4) return fit_kernel_r128<1, 4>;   // a dense covariance: at most 31 px
+    if (profile == 4) return fit_kernel_dense<1>;   // a dense covariance: at most 31 px
     return profile == BS_PROFILE_SPERGEL ? prof_kernel<1>(max_side) : prof_kernel<2>(max_side);
 }
 
@@ -55,7 +55,7 @@ PointsKernel prof_points(int max_side)
 PointsKernel points_for(int profile, int max_side)
 {
     if (is_pix(profile)) return max_side <= 31 ? logpost_points_pix_kernel<1> : logpost_points_pix_kernel<2>;
-    if (profile == 4) return logpost_points_kernel<1, 4>;
+    if (profile == 4) return logpost_points_dense_kernel<1>;
     return profile == BS_PROFILE_SPERGEL ? prof_points<1>(max_side) : prof_points<2>(max_side);
 }
 
@@ -76,7 +76,10 @@ size_t smem_for(int profile, int max_side, int n_chains)
     return b;
 }
 
-int threads_for(int profile, int n_chains) { return is_pix(profile) ? kPixThreads : 32 * n_chains; }
+int threads_for(int profile, int n_chains)
+{
+    return is_pix(profile) ? kPixThreads : profile == 4 ? 32 * kDenseWarps : 32 * n_chains;
+}
 
 // K_mu(x) = int_0^inf exp(-x cosh t) cosh(mu t) dt by the trapezoidal rule
 // (step 1/64; the integrand falls off doubly exponentially).
@@ -138,8 +141,7 @@ cudaError_t launch_fit_profile(const FitParams &p, int grid, cudaStream_t stream
 cudaError_t launch_logpost_points_profile(const FitParams &p, int n_points, const int32_t *gal_index,
                                           const float *theta, double *logp, float *grad, cudaStream_t stream)
 {
-    const int warps = p.profile == 4 ? 1 : kPointWarps;
-    const size_t smem = smem_for(p.profile, p.max_side, warps);
+    const size_t smem = smem_for(p.profile, p.max_side, kPointWarps);
     PointsKernel k = points_for(p.profile, p.max_side);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -147,7 +149,7 @@ cudaError_t launch_logpost_points_profile(const FitParams &p, int n_points, cons
         const int grid = n_points < 4096 ? n_points : 4096;
         k<<<grid, kPixThreads, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
     } else {
-        k<<<n_points, 32 * warps, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
+        k<<<n_points, threads_for(p.profile, kPointWarps), smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
     }
     bs::count_launches(1);
     return cudaGetLastError();
