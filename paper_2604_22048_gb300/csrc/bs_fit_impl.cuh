@@ -774,40 +774,6 @@ __device__ __forceinline__ void half_plane(Sums<NCT> &S, const SlotConst<NCT> &K
     }
 }
 
-// Sums over the warp of NV <= 8 per-lane values, returned in every lane with
-// identical bits.  Recursive halving: at each xor distance a lane keeps half
-// of its values and receives the partner's partial sums of them, so after
-// distances 16, 8, 4 lane l holds value (l >> 2) & 7 summed over 8 lanes; two
-// butterfly steps finish it (commutative adds, so the 4 lanes of a group
-// agree) and one shuffle per value broadcasts it from lane 4 j.
-template <int NV>
-__device__ __forceinline__ void warp_sum_n(float (&v)[NV])
-{
-    static_assert(NV >= 5 && NV <= 8, "four values per half at the first step");
-    const int lane = threadIdx.x & 31;
-    float r4[4];
-    const bool h16 = lane & 16;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float lo = v[k], hi = k + 4 < NV ? v[k + 4] : 0.0f;
-        const float keep = h16 ? hi : lo, send = h16 ? lo : hi;
-        r4[k] = keep + __shfl_xor_sync(BS_FULL_MASK, send, 16);
-    }
-    float r2[2];
-    const bool h8 = lane & 8;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const float keep = h8 ? r4[k + 2] : r4[k], send = h8 ? r4[k] : r4[k + 2];
-        r2[k] = keep + __shfl_xor_sync(BS_FULL_MASK, send, 8);
-    }
-    const bool h4 = lane & 4;
-    float r = (h4 ? r2[1] : r2[0]) + __shfl_xor_sync(BS_FULL_MASK, h4 ? r2[0] : r2[1], 4);
-    r += __shfl_xor_sync(BS_FULL_MASK, r, 2);
-    r += __shfl_xor_sync(BS_FULL_MASK, r, 1);
-#pragma unroll
-    for (int j = 0; j < NV; ++j) v[j] = __shfl_sync(BS_FULL_MASK, r, 4 * j);
-}
-
 // The model's shape at th (Sec. 3.3 forward model): flux, r0^2 and the coefficients
 // of the sheared quadratic form r0^2 q(k) = al kx^2 + be ky^2 + ga kx ky.
 struct Shape {
