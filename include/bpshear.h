@@ -580,7 +580,8 @@ bs_status bs_shear_loglike(const bs_shear_data *data, double g1, double g2,
  *   points  host double [n_points][3] = (g1, g2, alpha), each |g| < 1, alpha > 0.
  *   out     double [n_points][4] = {value, d/dg1, d/dg2, d/dalpha} per point,
  *           on the device, or on the host when out_on_host != 0 (the call
- *           then synchronises `stream` after each group of 4 points).
+ *           then synchronises `stream`: once with the workspace of
+ *           bs_shear_workspace_bytes and up to 512 points).
  * data->b must be NULL.  Results agree with bs_shear_loglike up to the
  * summation order (a different reduction layout).  Workspace:
  * bs_shear_workspace_bytes.  n_points == 0 returns BS_OK at once. */

@@ -382,17 +382,23 @@ bs_status bs_fp64_peak(double *tflops, void *stream)
     return BS_OK;
 }
 
+// bs_shear_loglike_multi: passes whose points one launch finalizes, and host results staged on the
+// device between copies.
+static constexpr int kMultiSlots = bs::kFinalizePoints / bs::kMultiPoints;
+static constexpr int kStagePoints = 512;
+
 size_t bs_shear_workspace_bytes(int64_t n_gal, int32_t K)
 {
     (void)n_gal;
     (void)K;
     // per-block partials of the 4-output kernel, of the all-free one or of the
-    // several-point one, plus the device copy of the results
+    // several-point one (kMultiSlots passes, so that their points are finalized
+    // together), plus the device copy of the results
     const size_t a = (size_t)bs::shear_grid_blocks() * 4, b = (size_t)bs::shear_full_grid_blocks() * bs::kShearFullOut;
-    const size_t c = (size_t)bs::shear_multi_grid_blocks() * bs::kMultiPoints * 4;
+    const size_t c = (size_t)kMultiSlots * bs::shear_multi_grid_blocks() * bs::kMultiPoints * 4;
     size_t m = a > b ? a : b;
     m = m > c ? m : c;
-    return (m + 4 * bs::kMultiPoints + bs::kShearFullOut) * sizeof(double);
+    return (m + 4 * (size_t)kStagePoints + bs::kShearFullOut) * sizeof(double);
 }
 
 static bs_status validate_shear(const bs_shear_data *d, const char *who)
@@ -419,7 +425,7 @@ bs_status bs_shear_loglike(const bs_shear_data *d, double g1, double g2, double 
     bs_status st = bs::shear_prepare(d, g1, g2, alpha, L, add, alpha_scale, "bs_shear_loglike");
     if (st != BS_OK) return st;
     if (!out) return fail(BS_ERR_INVALID_ARG, "bs_shear_loglike: NULL out");
-    const int grid = bs::shear_grid_blocks();
+    const int grid = bs::shear_grid_blocks(), used = bs::shear_grid_for(d->n_gal);
     const size_t need = (size_t)(grid * 4 + 4) * sizeof(double);
     if (!workspace || workspace_bytes < need)
         return fail(BS_ERR_OUT_OF_MEMORY, "bs_shear_loglike: workspace of %zu bytes needed", need);
@@ -429,11 +435,11 @@ bs_status bs_shear_loglike(const bs_shear_data *d, double g1, double g2, double 
     cudaError_t e;
     if (d->n_gal > 0) {
         L.partials = partials;
-        e = bs::launch_shear(L, grid, s);
+        e = bs::launch_shear(L, used, s);
         if (e != cudaSuccess) return cuda_fail(e, "bs_shear_loglike: launch");
         bs::count_launches(1);
     }
-    const int n_part = d->n_gal > 0 ? grid : 0;
+    const int n_part = d->n_gal > 0 ? used : 0;
     e = bs::launch_shear_finalize(partials, n_part, add[0], add[1], add[2], add[3], alpha_scale, dev_out, s);
     if (e != cudaSuccess) return cuda_fail(e, "bs_shear_loglike: finalize");
     bs::count_launches(1);
@@ -463,43 +469,75 @@ bs_status bs_shear_loglike_multi(const bs_shear_data *d, int32_t n_points, const
         return fail(BS_ERR_OUT_OF_MEMORY, "%s: workspace of %zu bytes needed", who, need);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     double *partials = static_cast<double *>(workspace);
-    double *host_stage = partials + (size_t)grid * NP * 4;
+    // A batch of at least kFinalizePoints points finalizes the points of kMultiSlots passes in one
+    // launch (a finalize is a few us of one SM, 4 of them as much as a small pass), where
+    // the workspace holds their partials; fewer points keep a finalize each.  Results for the
+    // host are staged and copied once per stage_cap points: a copy each pass would
+    // leave the GPU idle for its round trip.
+    const size_t pass_doubles = (size_t)grid * NP * 4, ws_doubles = workspace_bytes / sizeof(double);
+    const int slots = n_points >= bs::kFinalizePoints && ws_doubles >= kMultiSlots * pass_doubles + 4 * bs::kFinalizePoints
+                          ? kMultiSlots : 1;
+    double *stage = partials + slots * pass_doubles;
+    const size_t stage_cap = (ws_doubles - slots * pass_doubles) / 4 / (size_t)(slots * NP) * (slots * NP);
+    const int used = (int)((d->n_gal + 31) / 32 < grid ? (d->n_gal + 31) / 32 : grid);   // CTAs of a pass
+    bs::ShearFinalizeBatch F;
+    F.n_points = 0;
+    int staged = 0, copied = 0;      // points whose results lie in the stage, points copied out
     for (int start = 0; start < n_points; start += NP) {
         const int np = n_points - start < NP ? n_points - start : NP;
         bs::ShearMultiLaunch M;
-        double add[NP][4], ascale[NP];
+        const int base = F.n_points;     // points of the batch before this pass
         for (int p = 0; p < np; ++p) {
             const double *x = points + 3 * (size_t)(start + p);
             bs::ShearLaunch L;
-            st = bs::shear_prepare(d, x[0], x[1], x[2], L, add[p], ascale[p], who);
+            st = bs::shear_prepare(d, x[0], x[1], x[2], L, F.add[base + p], F.alpha_scale[base + p], who);
             if (st != BS_OK) return st;
             if (p == 0) M.s = L;
+            M.c[p] = L.c;
             M.g1[p] = L.g1;
             M.g2[p] = L.g2;
-            M.a2[p] = L.a2;
         }
-        for (int p = np; p < NP; ++p) M.g1[p] = M.g2[p] = M.a2[p] = 0.f;
+        for (int p = np; p < NP; ++p) {
+            M.c[p] = M.c[0];
+            M.g1[p] = M.g2[p] = 0.f;
+        }
         M.n_points = np;
-        M.partials = partials;
+        const size_t part_stride = 4 * (size_t)used;      // of one point
+        M.partials = partials + base * part_stride;
         cudaError_t e;
         if (d->n_gal > 0) {
-            e = bs::launch_shear_multi(M, grid, s);
+            e = bs::launch_shear_multi(M, used, s);
             if (e != cudaSuccess) return cuda_fail(e, "bs_shear_loglike_multi: launch");
             bs::count_launches(1);
         }
-        const int n_part = d->n_gal > 0 ? grid : 0;
-        double *dev_out = out_on_host ? host_stage : out + 4 * (size_t)start;
-        for (int p = 0; p < np; ++p) {
-            e = bs::launch_shear_finalize(partials + (size_t)p * grid * 4, n_part, add[p][0], add[p][1], add[p][2],
-                                          add[p][3], ascale[p], dev_out + 4 * p, s);
+        F.n_points += np;
+        const bool last = start + np == n_points;
+        if (F.n_points < slots * NP && !last) continue;
+        const int n_part = d->n_gal > 0 ? used : 0;
+        const int first = start + np - F.n_points;        // first point of the batch
+        double *dev_out = out_on_host ? stage + 4 * (size_t)staged : out + 4 * (size_t)first;
+        if (slots > 1) {
+            e = bs::launch_shear_finalize_batch(partials, part_stride, n_part, F, dev_out, s);
             if (e != cudaSuccess) return cuda_fail(e, "bs_shear_loglike_multi: finalize");
             bs::count_launches(1);
+        } else {
+            for (int p = 0; p < np; ++p) {
+                const double *add = F.add[p];
+                e = bs::launch_shear_finalize(partials + p * part_stride, n_part, add[0], add[1], add[2], add[3],
+                                              F.alpha_scale[p], dev_out + 4 * p, s);
+                if (e != cudaSuccess) return cuda_fail(e, "bs_shear_loglike_multi: finalize");
+                bs::count_launches(1);
+            }
         }
-        if (out_on_host) {
-            e = cudaMemcpyAsync(out + 4 * (size_t)start, host_stage, 4 * np * sizeof(double), cudaMemcpyDeviceToHost,
-                                s);
+        staged += F.n_points;
+        F.n_points = 0;
+        if (out_on_host && (last || (size_t)staged + slots * NP > stage_cap)) {
+            e = cudaMemcpyAsync(out + 4 * (size_t)copied, stage, 4 * (size_t)staged * sizeof(double),
+                                cudaMemcpyDeviceToHost, s);
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
             if (e != cudaSuccess) return cuda_fail(e, "bs_shear_loglike_multi: copy");
+            copied += staged;
+            staged = 0;
         }
     }
     return BS_OK;
@@ -1013,6 +1051,22 @@ bs_status shear_prepare(const bs_shear_data *d, double g1, double g2, double alp
     L.c0 = (float)(1.4426950408889634 / (2.0 * (double)d->sigma_e0 * d->sigma_e0));
     L.r2 = d->trunc_r * d->trunc_r;
     L.partials = nullptr;
+    {
+        // products and sum rounded one by one, whatever the host compiler contracts
+        const volatile float a = L.a2 * 0.6931471805599453f;
+        const volatile float p1 = L.g1 * L.g1, p2 = L.g2 * L.g2, gg = p1 + p2;
+        auto twice = [](float x) { return make_float2(x, x); };
+        L.c.g1 = twice(L.g1);
+        L.c.g2 = twice(L.g2);
+        L.c.a2n = twice(-L.a2);
+        L.c.an = twice(a);
+        L.c.nan = twice(-a);
+        L.c.nk = twice(-L.kappa);
+        L.c.c0 = twice(L.c0);
+        L.c.gg = twice(gg);
+        L.c.m2 = twice(-2.0f);
+        L.c.r2 = L.r2;
+    }
     // The per-sample terms see g and 1/(2 alpha^2) rounded to FP32; the
     // per-galaxy constants are taken at the same rounded values, so that the
     // total is the likelihood at one (g, alpha), a smooth function of it.

@@ -109,7 +109,18 @@ cudaError_t launch_render(int n, const float *theta, const float *shear, const i
                           const int32_t *side, int max_side, const bs_psf *psf, int n_psf,
                           float pixel_scale, float *out, cudaStream_t stream);
 
+// Constants of one (g, alpha) point, each twice for the packed arithmetic, formed on the host
+// so that the kernels read them from the launch's parameters and keep no registers
+// for them.
+struct ShearConst {
+    float2 g1, g2;                   // g
+    float2 a2n, an, nan, nk;         // -a2 (log2 units), a = 1/(2 alpha^2), -a, -kappa
+    float2 c0;                       // log2(e)/(2 sigma_e0^2)
+    float2 gg, m2;                   // |g|^2, -2
+    float r2;
+};
 struct ShearLaunch {
+    ShearConst c;
     const float *e1, *e2, *b;
     const float *w;   // per-galaxy weight of the galaxy's term, or NULL (all 1)
     long long n_gal;
@@ -131,18 +142,31 @@ struct ShearFullLaunch {
 };
 constexpr int kShearFullOut = 9;   // value, d/d(g1, g2, sigma_e, mu_f, sigma_f, a_f, mu_s, sigma_s)
 
+// CTAs of a one-point pass that fill the GPU (the size of the workspace), and of a pass
+// over n_gal galaxies: no more than one per 32 of them.
 int shear_grid_blocks();
+int shear_grid_for(long long n_gal);
 double shear_weight_total(const bs_shear_data *d);
 // Several (g1, g2, alpha) points per pass over the samples (no b).
 constexpr int kMultiPoints = 4;
 struct ShearMultiLaunch {
-    ShearLaunch s;                  // data, K, family, kappa, c0, r2, w (g1, g2, a2 unused)
+    ShearLaunch s;                  // data, K, family, w (the point unused)
     int n_points;                   // 1..kMultiPoints
-    float g1[kMultiPoints], g2[kMultiPoints], a2[kMultiPoints];
+    ShearConst c[kMultiPoints];
+    float g1[kMultiPoints], g2[kMultiPoints];
     double *partials;               // [kMultiPoints][grid][4]
 };
 int shear_multi_grid_blocks();
 cudaError_t launch_shear_multi(const ShearMultiLaunch &m, int grid, cudaStream_t stream);
+// Finalize the points of several passes in one launch: point q's partials (n_part blocks of
+// 4) start at partials + q part_stride, its results at out + 4 q.
+constexpr int kFinalizePoints = 16;
+struct ShearFinalizeBatch {
+    double add[kFinalizePoints][4], alpha_scale[kFinalizePoints];
+    int n_points;
+};
+cudaError_t launch_shear_finalize_batch(const double *partials, size_t part_stride, int n_part,
+                                        const ShearFinalizeBatch &b, double *out, cudaStream_t stream);
 int shear_full_grid_blocks();
 cudaError_t launch_shear(const ShearLaunch &s, int grid, cudaStream_t stream);
 cudaError_t launch_shear_full(const ShearFullLaunch &f, int grid, cudaStream_t stream);

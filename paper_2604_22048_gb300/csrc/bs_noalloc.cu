@@ -77,6 +77,7 @@ extern "C" bs_status bs_shear_loglike_noalloc(const bs_shear_data *data, double 
                              "bs_shear_loglike_noalloc: this device needs %d partial slots, the static "
                              "scratch holds %d; use bs_shear_loglike with a workspace",
                              grid, kNoAllocBlocks);
+    const int used = bs::shear_grid_for(data->n_gal);
     double *scratch = nullptr;
     st = scratch_for_current_device(&scratch);
     if (st != BS_OK) return st;
@@ -84,12 +85,12 @@ extern "C" bs_status bs_shear_loglike_noalloc(const bs_shear_data *data, double 
     cudaError_t e;
     if (data->n_gal > 0) {
         L.partials = scratch;
-        e = bs::launch_shear(L, grid, s);
+        e = bs::launch_shear(L, used, s);
         if (e != cudaSuccess)
             return bs::set_error(BS_ERR_CUDA, "bs_shear_loglike_noalloc: launch: %s", cudaGetErrorString(e));
         bs::count_launches(1);
     }
-    e = bs::launch_shear_finalize(scratch, data->n_gal > 0 ? grid : 0, add[0], add[1], add[2], add[3],
+    e = bs::launch_shear_finalize(scratch, data->n_gal > 0 ? used : 0, add[0], add[1], add[2], add[3],
                                   alpha_scale, out, s);
     if (e != cudaSuccess)
         return bs::set_error(BS_ERR_CUDA, "bs_shear_loglike_noalloc: finalize: %s", cudaGetErrorString(e));

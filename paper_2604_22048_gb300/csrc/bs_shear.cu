@@ -28,6 +28,7 @@
 // accumulated in FP64 and written as per-block partials; a one-block kernel
 // sums the partials in a fixed order (deterministic) and adds the
 // per-galaxy constants.
+#include <atomic>
 #include <cmath>
 
 #include <cuda.h>            // CUtensorMap and its enums (types only: the encoder is looked up at run time)
@@ -94,34 +95,6 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b)
         : "=f"(d.x), "=f"(d.y)
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
     return d;
-}
-
-// Per-launch constants in registers.
-struct ShearConst {
-    float2 g1, g2, ng1, ng2;         // g, -g
-    float2 a2n, an, nan, nk;         // -a2 (log2 units), a = 1/(2 alpha^2), -a, -kappa
-    float2 c0;                       // log2(e)/(2 sigma_e0^2)
-    float2 gg, m2;                   // |g|^2, -2
-    float r2;
-};
-
-__device__ __forceinline__ ShearConst shear_const(const ShearLaunch &s)
-{
-    ShearConst c;
-    const float a = s.a2 * kLn2;
-    c.g1 = f2(s.g1);
-    c.g2 = f2(s.g2);
-    c.ng1 = f2(-s.g1);
-    c.ng2 = f2(-s.g2);
-    c.a2n = f2(-s.a2);
-    c.an = f2(a);
-    c.nan = f2(-a);
-    c.nk = f2(-s.kappa);
-    c.c0 = f2(s.c0);
-    c.gg = f2(s.g1 * s.g1 + s.g2 * s.g2);
-    c.m2 = f2(-2.0f);
-    c.r2 = s.r2;
-    return c;
 }
 
 // Two samples: the weight split as exp2(x) f, with x = c0 |eps'|^2 -
@@ -278,14 +251,14 @@ __device__ __forceinline__ void eval_chunk(const ShearConst &c, const Chunk &ch,
     }
 }
 
-// Merge the lanes of a galaxy's group and add the galaxy's log-sum-exp and
-// softmax-weighted derivative sums, times the galaxy's weight w[n] (1 when w
-// is NULL; a zero weight drops the galaxy), to the lane-0 accumulators; (g1, g2)
-// is the shear of the evaluation.
+// Merge the lanes of a galaxy's group and add the galaxy's terms, times the galaxy's weight
+// w[n] (1 when w is NULL; a zero weight drops the galaxy), to the accumulators of the
+// group's first four lanes: lane 0 the log-sum-exp (log2), lanes 1-3 the softmax-weighted
+// derivative sums, each lane one of them: the FP64 pipe takes 16 cycles an operation for the
+// whole SM, so the four go through it side by side.  (g1, g2) is the shear of the evaluation.
 template <int G = kGroup>
 __device__ __forceinline__ void finish_galaxy(const Lse &L, float g1, float g2, unsigned gmask, int sub,
-                                              const float *w, long long n, double &av, double &a1, double &a2,
-                                              double &aq)
+                                              const float *w, long long n, double &acc)
 {
     float m = L.m;
     const float tr = L.tr.x + L.tr.y;
@@ -306,18 +279,21 @@ __device__ __forceinline__ void finish_galaxy(const Lse &L, float g1, float g2, 
         tq = tq * ca + oq * cb;
         m = mn;
     }
-    if (sub == 0) {
-        const double wn = w ? (double)__ldg(w + n) : 1.0;
-        if (wn == 0.0) return;
-        if (sw > 0.f) {
-            const float inv = 1.0f / sw;
-            av += wn * ((double)m + log2_total(sw));
-            a1 += wn * (double)(-2.0f * t1 * inv);
-            a2 += wn * (double)(-2.0f * t2 * inv);
-            aq += wn * (double)(tq * inv);
-        } else {
-            av = -INFINITY;
-        }
+    if (sub >= 4) return;
+    const float wf = w ? __ldg(w + n) : 1.0f;
+    if (wf == 0.0f) return;
+    if (sw > 0.f) {
+        const float inv = 1.0f / sw;
+        const float d = sub == 1 ? -2.0f * t1 * inv : sub == 2 ? -2.0f * t2 * inv : tq * inv;
+        // lane 0: m + log2(sw), the other lanes d + 0
+        int e;
+        const float l = log2f(frexpf(sw, &e));   // as log2_total
+        double v = (double)(sub == 0 ? m : d);
+        if (sub == 0) v += (double)e + (double)l;
+        if (w) v *= (double)wf;
+        acc += v;
+    } else if (sub == 0) {
+        acc = -INFINITY;
     }
 }
 
@@ -327,22 +303,16 @@ __device__ __forceinline__ void lse_reset(Lse &L)
     L.sw = L.t1 = L.t2 = L.tq = L.tr = f2(0.f);
 }
 
-// Block reduction of the four FP64 accumulators into this block's partials.
-__device__ __forceinline__ void block_partials(const ShearLaunch &s, double av, double a1, double a2, double aq)
+// Block reduction of the lanes' FP64 accumulators (quantity = lane of the group of G, the
+// first four) into this block's partials.
+template <int G>
+__device__ __forceinline__ void block_partials(const ShearLaunch &s, double acc)
 {
     __shared__ double red[kShearThreads / 32][4];
     const int lane = threadIdx.x & 31;
-    av = warp_sum_d(av);
-    a1 = warp_sum_d(a1);
-    a2 = warp_sum_d(a2);
-    aq = warp_sum_d(aq);
-    const int w = threadIdx.x >> 5;
-    if (lane == 0) {
-        red[w][0] = av;
-        red[w][1] = a1;
-        red[w][2] = a2;
-        red[w][3] = aq;
-    }
+#pragma unroll
+    for (int o = 16; o >= G; o >>= 1) acc += __shfl_xor_sync(BS_FULL_MASK, acc, o);
+    if (lane < 4) red[threadIdx.x >> 5][lane] = acc;
     __syncthreads();
     if (threadIdx.x < 4) {
         double t = 0.0;
@@ -354,16 +324,16 @@ __device__ __forceinline__ void block_partials(const ShearLaunch &s, double av, 
 // Any K and alignment: scalar loads into two register buffers in turn (the
 // next chunk's loads in flight while the current one is evaluated).
 template <int FAMILY, bool HAS_B>
-__global__ void __launch_bounds__(kShearThreads, 3) shear_kernel(const ShearLaunch s)
+__global__ void __launch_bounds__(kShearThreads, 3) shear_kernel(const __grid_constant__ ShearLaunch s)
 {
     const int lane = threadIdx.x & 31;
     const int sub = lane & (kGroup - 1);
     const unsigned gmask = 0xFFu << (lane & ~(kGroup - 1));
     const long long group = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kGroup;
     const long long ngroups = (long long)gridDim.x * blockDim.x / kGroup;
-    const ShearConst c = shear_const(s);
+    const ShearConst &c = s.c;
     const int K = s.K;
-    double av = 0.0, a1 = 0.0, a2 = 0.0, aq = 0.0;
+    double acc = 0.0;
 
     for (long long n = group; n < s.n_gal; n += ngroups) {
         const long long base = n * (long long)K;
@@ -382,9 +352,9 @@ __global__ void __launch_bounds__(kShearThreads, 3) shear_kernel(const ShearLaun
             eval_chunk<FAMILY, HAS_B>(c, B, L);
             k0 += 4 * kGroup;
         }
-        finish_galaxy(L, s.g1, s.g2, gmask, sub, s.w, n, av, a1, a2, aq);
+        finish_galaxy(L, s.g1, s.g2, gmask, sub, s.w, n, acc);
     }
-    block_partials(s, av, a1, a2, aq);
+    block_partials<kGroup>(s, acc);
 }
 
 // Asynchronous 16-byte global -> shared copies (L2 only), grouped per chunk.
@@ -425,7 +395,7 @@ __host__ __device__ constexpr size_t async_smem_bytes(bool has_b)
 // does not drain between galaxies.  A lane only reads the slots it filled,
 // after cp.async.wait_group; no barrier is needed.
 template <int FAMILY, bool HAS_B>
-__global__ void __launch_bounds__(kShearThreads, HAS_B ? 3 : kAsyncBlocks) shear_kernel_async(const ShearLaunch s)
+__global__ void __launch_bounds__(kShearThreads, HAS_B ? 3 : kAsyncBlocks) shear_kernel_async(const __grid_constant__ ShearLaunch s)
 {
     extern __shared__ float4 sbuf[];
     constexpr int NV = HAS_B ? 3 : 2;
@@ -435,13 +405,13 @@ __global__ void __launch_bounds__(kShearThreads, HAS_B ? 3 : kAsyncBlocks) shear
     const unsigned gmask = ((1u << kAGroup) - 1u) << (lane & ~(kAGroup - 1));
     const long long group = ((long long)blockIdx.x * blockDim.x + tid) / kAGroup;
     const long long ngroups = (long long)gridDim.x * blockDim.x / kAGroup;
-    const ShearConst c = shear_const(s);
+    const ShearConst &c = s.c;
     const int K = s.K;
     constexpr int span = kChunk * kAGroup;                   // samples of a group per chunk step
     const int cpg = (K + span - 1) / span;                   // chunks per galaxy per lane
     const long long my_gal = group < s.n_gal ? (s.n_gal - 1 - group) / ngroups + 1 : 0;
     const long long n_items = my_gal * cpg;
-    double av = 0.0, a1 = 0.0, a2 = 0.0, aq = 0.0;
+    double acc = 0.0;
     // slot (stage, array, half) of this thread
     auto slot = [&](int st, int arr, int q) -> float4 * {
         return &sbuf[((st * NV + arr) * kQuads + q) * kShearThreads + tid];
@@ -496,13 +466,13 @@ __global__ void __launch_bounds__(kShearThreads, HAS_B ? 3 : kAsyncBlocks) shear
         cst = cst + 1 == kStages ? 0 : cst + 1;
         if (++cc == cpg) {
             cc = 0;
-            finish_galaxy<kAGroup>(L, s.g1, s.g2, gmask, sub, s.w, cn, av, a1, a2, aq);
+            finish_galaxy<kAGroup>(L, s.g1, s.g2, gmask, sub, s.w, cn, acc);
             cn += ngroups;
             lse_reset(L);
         }
     }
     cp_async_wait<0>();
-    block_partials(s, av, a1, a2, aq);
+    block_partials<kAGroup>(s, acc);
 }
 
 // ---- Tensor-memory-accelerator tiles (no b): a CTA streams tiles of kTileG
@@ -528,9 +498,11 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)_
 
 // Wait for the phase of the given parity.  Each try_wait may suspend the warp
 // in hardware for up to 20 us until the phase completes (no busy loop taking
-// issue slots from the computing warps); the limit is checked between tries.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_t t0)
+// issue slots from the computing warps).  The clock for the limit of two seconds is
+// read only once a try has failed: most waits find their phase complete.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 {
+    uint64_t t0 = 0;
     for (;;) {
         uint32_t ok;
         asm volatile(
@@ -542,6 +514,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_
         if (ok) return true;
         uint64_t t;
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        if (t0 == 0) t0 = t;
         if (t - t0 > 2000000000ull) return false;
     }
 }
@@ -586,9 +559,7 @@ struct TmaRing {
         if (p_item >= n_items || !p_ok) return;
         const int st = p_item % kTmaStages;
         if (p_item >= kTmaStages) {   // the stage's previous item has been read by every warp
-            uint64_t t0;
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-            if (!mbar_wait(smem_u32(&empty[st]), (uint32_t)((p_item / kTmaStages - 1) & 1), t0)) {
+            if (!mbar_wait(smem_u32(&empty[st]), (uint32_t)((p_item / kTmaStages - 1) & 1))) {
                 p_ok = false;
                 return;
             }
@@ -618,10 +589,8 @@ struct TmaRing {
     // all threads: wait until item's stage has landed (false, in every lane, on a timeout)
     __device__ bool wait_full(int item) const
     {
-        uint64_t t0;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
         return __all_sync(BS_FULL_MASK,
-                          mbar_wait(smem_u32(&full[item % kTmaStages]), (uint32_t)((item / kTmaStages) & 1), t0));
+                          mbar_wait(smem_u32(&full[item % kTmaStages]), (uint32_t)((item / kTmaStages) & 1)));
     }
     // all threads of a warp, after reading item's stage
     __device__ void release(int item) const
@@ -636,10 +605,8 @@ struct TmaRing {
     {
         __syncthreads();
         if (threadIdx.x == 0) {
-            uint64_t t1;
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
             for (int it = p_item - kTmaStages; it < p_item; ++it)
-                if (it >= 0) mbar_wait(smem_u32(&full[it % kTmaStages]), (uint32_t)((it / kTmaStages) & 1), t1);
+                if (it >= 0) mbar_wait(smem_u32(&full[it % kTmaStages]), (uint32_t)((it / kTmaStages) & 1));
         }
     }
 };
@@ -661,21 +628,23 @@ __device__ __forceinline__ bool tma_quad(const TmaRing &R, int item, int K, int 
 
 template <int FAMILY>
 __global__ void __launch_bounds__(kShearThreads, kAsyncBlocks)
-    shear_kernel_tma(const ShearLaunch s, const __grid_constant__ CUtensorMap m1, const __grid_constant__ CUtensorMap m2)
+    shear_kernel_tma(const __grid_constant__ ShearLaunch s, const __grid_constant__ CUtensorMap m1, const __grid_constant__ CUtensorMap m2)
 {
     extern __shared__ __align__(128) unsigned char tma_raw[];
     __shared__ __align__(8) uint64_t full[kTmaStages], empty[kTmaStages];
+    __shared__ int s_fail;
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int sub = tid & (kAGroup - 1), gl = tid / kAGroup;
     const unsigned gmask = ((1u << kAGroup) - 1u) << (lane & ~(kAGroup - 1));
-    const ShearConst c = shear_const(s);
+    const ShearConst &c = s.c;
     const int K = s.K;
+    if (tid == 0) s_fail = 0;
     TmaRing R;
-    R.init(tma_raw, full, empty, s.n_gal, K);
+    R.init(tma_raw, full, empty, s.n_gal, K);   // (its barrier also orders the reset above)
     if (tid == 0)
         for (int t = 0; t < kTmaStages - 1; ++t) R.issue(&m1, &m2);
-    double av = 0.0, a1 = 0.0, a2 = 0.0, aq = 0.0;
+    double acc = 0.0;
     Lse L;
     lse_reset(L);
     bool failed = false;
@@ -697,15 +666,15 @@ __global__ void __launch_bounds__(kShearThreads, kAsyncBlocks)
         }
         R.release(item);
         if (++chunk == R.cpg) {
-            if (n < s.n_gal) finish_galaxy<kAGroup>(L, s.g1, s.g2, gmask, sub, s.w, n, av, a1, a2, aq);
+            if (n < s.n_gal) finish_galaxy<kAGroup>(L, s.g1, s.g2, gmask, sub, s.w, n, acc);
             lse_reset(L);
             chunk = 0;
             tile += gridDim.x;
         }
     }
-    if (failed || (tid == 0 && !R.p_ok)) av = a1 = a2 = aq = NAN;
-    R.drain();
-    block_partials(s, av, a1, a2, aq);
+    if (failed || (tid == 0 && !R.p_ok)) s_fail = 1;
+    R.drain();                                  // (begins with a barrier)
+    block_partials<kAGroup>(s, s_fail ? NAN : acc);
 }
 
 // The tensor-map encoder of the driver, looked up once through the runtime
@@ -740,28 +709,35 @@ bool make_sample_map(CUtensorMap &m, const float *base, long long n_gal, int K)
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-__global__ void __launch_bounds__(256) shear_finalize_kernel(const double *partials, int n_part,
-                                                              double add_value, double add_g1,
-                                                              double add_g2, double add_alpha,
-                                                              double alpha_scale, double *out)
+// Sum the partials of a point (n_part blocks of 4) and add the per-galaxy constants: a warp per
+// quantity, so that the blocks' partials are read in one round trip and no barrier is
+// needed; a fixed order.
+__device__ __forceinline__ void finalize_point(const double *partials, int n_part, const double *add, double alpha_scale,
+                                               double *out)
 {
-    __shared__ double red[256][4];
-    double t[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int i = threadIdx.x; i < n_part; i += blockDim.x)
-        for (int k = 0; k < 4; ++k) t[k] += partials[(size_t)i * 4 + k];
-    for (int k = 0; k < 4; ++k) red[threadIdx.x][k] = t[k];
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o)
-            for (int k = 0; k < 4; ++k) red[threadIdx.x][k] += red[threadIdx.x + o][k];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        out[0] = red[0][0] * 0.6931471805599453 + add_value;
-        out[1] = red[0][1] + add_g1;
-        out[2] = red[0][2] + add_g2;
-        out[3] = red[0][3] * alpha_scale + add_alpha;
-    }
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double t = 0.0;
+#pragma unroll 8
+    for (int i = lane; i < n_part; i += 32) t += partials[(size_t)i * 4 + k];
+    t = warp_sum_d(t);
+    if (lane == 0) out[k] = t * (k == 0 ? 0.6931471805599453 : k == 3 ? alpha_scale : 1.0) + add[k];
+}
+
+struct ShearFinalize {
+    double add[4], alpha_scale;
+};
+__global__ void __launch_bounds__(128) shear_finalize_kernel(const double *partials, int n_part,
+                                                             const __grid_constant__ ShearFinalize f, double *out)
+{
+    finalize_point(partials, n_part, f.add, f.alpha_scale, out);
+}
+
+__global__ void __launch_bounds__(128) shear_finalize_batch_kernel(const double *partials, size_t part_stride, int n_part,
+                                                                   const __grid_constant__ ShearFinalizeBatch f,
+                                                                   double *out)
+{
+    const int q = blockIdx.x;
+    finalize_point(partials + q * part_stride, n_part, f.add[q], f.alpha_scale[q], out + 4 * q);
 }
 
 // ---- all properties free ----------------------------------------------------
@@ -968,17 +944,8 @@ cudaError_t launch_fb(const ShearLaunch &s, int grid, bool vec, cudaStream_t st)
 // its own shared-memory slot (one writer), summed over the block in a fixed
 // order; partials are laid out per point so that each point is finalized as
 // a single-point pass.
-__device__ __forceinline__ ShearConst shear_const_point(const ShearMultiLaunch &m, int p)
-{
-    ShearLaunch s = m.s;
-    s.g1 = m.g1[p];
-    s.g2 = m.g2[p];
-    s.a2 = m.a2[p];
-    return shear_const(s);
-}
-
 template <int FAMILY>
-__global__ void __launch_bounds__(kShearThreads, 2) shear_kernel_multi(const ShearMultiLaunch m)
+__global__ void __launch_bounds__(kShearThreads, 2) shear_kernel_multi(const __grid_constant__ ShearMultiLaunch m)
 {
     constexpr int NP = kMultiPoints;
     constexpr int kGroups = kShearThreads / kGroup;
@@ -1005,7 +972,7 @@ __global__ void __launch_bounds__(kShearThreads, 2) shear_kernel_multi(const She
         auto eval_all = [&](const Chunk &ch) {
 #pragma unroll
             for (int p = 0; p < NP; ++p)
-                if (p < m.n_points) eval_chunk<FAMILY, false>(shear_const_point(m, p), ch, L[p]);
+                if (p < m.n_points) eval_chunk<FAMILY, false>(m.c[p], ch, L[p]);
         };
         load_chunk<false>(s, base, k0, K, A);
         for (;;) {
@@ -1021,14 +988,9 @@ __global__ void __launch_bounds__(kShearThreads, 2) shear_kernel_multi(const She
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
             if (p < m.n_points) {
-                double av = 0.0, a1 = 0.0, a2 = 0.0, aq = 0.0;
-                finish_galaxy(L[p], m.g1[p], m.g2[p], gmask, sub, s.w, n, av, a1, a2, aq);
-                if (sub == 0) {
-                    acc[gi][p][0] += av;
-                    acc[gi][p][1] += a1;
-                    acc[gi][p][2] += a2;
-                    acc[gi][p][3] += aq;
-                }
+                double t = 0.0;
+                finish_galaxy(L[p], m.g1[p], m.g2[p], gmask, sub, s.w, n, t);
+                if (sub < 4) acc[gi][p][sub] += t;
             }
         }
     }
@@ -1043,18 +1005,45 @@ __global__ void __launch_bounds__(kShearThreads, 2) shear_kernel_multi(const She
 
 }  // namespace
 
+namespace {
+
+// SMs x resident CTAs of a kernel on the current device, asked of the runtime once per device
+// (every evaluation of a likelihood needs it).
+struct GridCache {
+    std::atomic<int> blocks[64] = {};
+};
+template <typename K>
+int resident_grid(GridCache &cache, K kernel, size_t smem)
+{
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64) {
+        const int known = cache.blocks[dev].load(std::memory_order_relaxed);
+        if (known > 0) return known;
+    }
+    int sms = 0, nb = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kShearThreads, smem);
+    if (sms <= 0 || nb <= 0) return sms > 0 ? sms : 1;      // not kept: the next call asks again
+    if (dev >= 0 && dev < 64) cache.blocks[dev].store(sms * nb, std::memory_order_relaxed);
+    return sms * nb;
+}
+
+GridCache g_grid_one, g_grid_full, g_grid_multi;
+
+}  // namespace
+
 int shear_grid_blocks()
 {
-    int dev = 0, sms = 0, nb = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(shear_kernel_async<BS_EPRIOR_BA14, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)async_smem_bytes(false));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, shear_kernel_async<BS_EPRIOR_BA14, false>, kShearThreads,
-                                                  async_smem_bytes(false));
-    if (sms <= 0) sms = 1;
-    if (nb <= 0) nb = 1;
-    return sms * nb;
+    return resident_grid(g_grid_one, shear_kernel_async<BS_EPRIOR_BA14, false>, async_smem_bytes(false));
+}
+
+int shear_grid_for(long long n_gal)
+{
+    const int full = shear_grid_blocks();
+    const long long want = (n_gal + 31) / 32;
+    return want < 1 ? 1 : want < full ? (int)want : full;
 }
 
 cudaError_t launch_shear(const ShearLaunch &s, int grid, cudaStream_t stream)
@@ -1070,16 +1059,7 @@ cudaError_t launch_shear(const ShearLaunch &s, int grid, cudaStream_t stream)
               : launch_fb<BS_EPRIOR_TRUNC_GAUSS, false>(s, grid, vec, stream);
 }
 
-int shear_full_grid_blocks()
-{
-    int dev = 0, sms = 0, nb = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, shear_full_kernel<BS_EPRIOR_BA14>, kShearThreads, 0);
-    if (sms <= 0) sms = 1;
-    if (nb <= 0) nb = 1;
-    return sms * nb;
-}
+int shear_full_grid_blocks() { return resident_grid(g_grid_full, shear_full_kernel<BS_EPRIOR_BA14>, 0); }
 
 cudaError_t launch_shear_full(const ShearFullLaunch &f, int grid, cudaStream_t stream)
 {
@@ -1103,16 +1083,7 @@ cudaError_t launch_shear_finalize_n(const double *partials, int n_part, int n_ou
     return cudaGetLastError();
 }
 
-int shear_multi_grid_blocks()
-{
-    int dev = 0, sms = 0, nb = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, shear_kernel_multi<BS_EPRIOR_BA14>, kShearThreads, 0);
-    if (sms <= 0) sms = 1;
-    if (nb <= 0) nb = 1;
-    return sms * nb;
-}
+int shear_multi_grid_blocks() { return resident_grid(g_grid_multi, shear_kernel_multi<BS_EPRIOR_BA14>, 0); }
 
 // Several points per pass with the samples streamed in tiles (K a multiple of 4,
 // 16-byte aligned rows, no b): the one-point tile kernel's ring and lane layout, each
@@ -1122,7 +1093,7 @@ int shear_multi_grid_blocks()
 // partials are NaN.
 template <int FAMILY>
 __global__ void __launch_bounds__(kShearThreads, 2)
-    shear_kernel_tma_multi(const ShearMultiLaunch m, const __grid_constant__ CUtensorMap m1,
+    shear_kernel_tma_multi(const __grid_constant__ ShearMultiLaunch m, const __grid_constant__ CUtensorMap m1,
                            const __grid_constant__ CUtensorMap m2)
 {
     constexpr int NP = kMultiPoints;
@@ -1164,7 +1135,7 @@ __global__ void __launch_bounds__(kShearThreads, 2)
                 if (tma_quad(R, item, K, chunk, h, ch)) {
 #pragma unroll
                     for (int p = 0; p < NP; ++p)
-                        if (p < m.n_points) eval_chunk<FAMILY, false>(shear_const_point(m, p), ch, L[p]);
+                        if (p < m.n_points) eval_chunk<FAMILY, false>(m.c[p], ch, L[p]);
                 }
             }
         }
@@ -1174,14 +1145,9 @@ __global__ void __launch_bounds__(kShearThreads, 2)
 #pragma unroll
                 for (int p = 0; p < NP; ++p) {
                     if (p < m.n_points) {
-                        double av = 0.0, a1 = 0.0, a2 = 0.0, aq = 0.0;
-                        finish_galaxy<kAGroup>(L[p], m.g1[p], m.g2[p], gmask, sub, s.w, n, av, a1, a2, aq);
-                        if (sub == 0) {
-                            acc[gl][p][0] += av;
-                            acc[gl][p][1] += a1;
-                            acc[gl][p][2] += a2;
-                            acc[gl][p][3] += aq;
-                        }
+                        double t = 0.0;
+                        finish_galaxy<kAGroup>(L[p], m.g1[p], m.g2[p], gmask, sub, s.w, n, t);
+                        acc[gl][p][sub] += t;
                     }
                 }
             }
@@ -1228,8 +1194,16 @@ cudaError_t launch_shear_finalize(const double *partials, int n_part, double add
                                   double add_g1, double add_g2, double add_alpha,
                                   double alpha_scale, double *out, cudaStream_t stream)
 {
-    shear_finalize_kernel<<<1, 256, 0, stream>>>(partials, n_part, add_value, add_g1, add_g2,
-                                                 add_alpha, alpha_scale, out);
+    const ShearFinalize f = {{add_value, add_g1, add_g2, add_alpha}, alpha_scale};
+    shear_finalize_kernel<<<1, 128, 0, stream>>>(partials, n_part, f, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_shear_finalize_batch(const double *partials, size_t part_stride, int n_part,
+                                        const ShearFinalizeBatch &b, double *out, cudaStream_t stream)
+{
+    if (b.n_points < 1 || b.n_points > kFinalizePoints) return cudaErrorInvalidValue;
+    shear_finalize_batch_kernel<<<b.n_points, 128, 0, stream>>>(partials, part_stride, n_part, b, out);
     return cudaGetLastError();
 }
 
