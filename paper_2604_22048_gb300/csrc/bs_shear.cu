@@ -18,8 +18,7 @@
 // Each galaxy's K samples are read by a group of lanes: when K % 4 == 0 and the
 // rows are 16-byte aligned, 4 lanes per galaxy read 12-sample chunks from tiles
 // of 64 galaxies x 48 samples that the tensor memory accelerator streams into
-// shared memory (without b), or from a per-lane cp.async ring (with b); otherwise
-// 8 lanes per galaxy with scalar loads one chunk ahead.  The
+// shared memory; otherwise 8 lanes per galaxy with scalar loads one chunk ahead.  The
 // arithmetic runs on pairs of samples in packed FP32x2 instructions, x is
 // kept in log2 units for the MUFU exp2, and the group keeps
 // an online log-sum-exp (a reference log weight that may lag the running
@@ -95,6 +94,24 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b)
         : "=f"(d.x), "=f"(d.y)
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
     return d;
+}
+
+// The point's constants from the launch's parameters into registers.  Left to the compiler they
+// are loaded again at every use (two per packed operand), which took a fifth of the
+// one-point pass's issue slots.
+__device__ __forceinline__ void hold(float2 &v) { asm volatile("" : "+f"(v.x), "+f"(v.y)); }
+__device__ __forceinline__ ShearConst held(const ShearConst &k)
+{
+    ShearConst c = k;
+    hold(c.g1);
+    hold(c.g2);
+    hold(c.a2n);
+    hold(c.an);
+    hold(c.nan);
+    hold(c.nk);
+    hold(c.c0);
+    hold(c.gg);
+    return c;
 }
 
 // Two samples: the weight split as exp2(x) f, with x = c0 |eps'|^2 -
@@ -194,6 +211,45 @@ __device__ __forceinline__ void mask_missing(const Chunk &ch, float2 (&x)[2])
     if (ch.nvalid < 1) x[0].x = -INFINITY;
 }
 
+// The sums of a pair with weights e.
+__device__ __forceinline__ void add_pair(Lse &L, float2 e, float2 e1, float2 e2, float2 ru, float2 pp, float2 rr,
+                                         float2 qq)
+{
+    const float2 er = mul2(e, ru);
+    const float2 erp = mul2(er, pp);
+    L.sw = add2(L.sw, e);
+    L.t1 = fma2(erp, e1, L.t1);
+    L.t2 = fma2(erp, e2, L.t2);
+    L.tr = fma2(er, rr, L.tr);
+    L.tq = fma2(e, qq, L.tq);
+}
+
+// exp2(x + nm) f
+__device__ __forceinline__ float2 pair_weight(float2 x, float2 nm, float2 f)
+{
+    const float2 d = add2(x, nm);
+    return mul2(make_float2(ex2_ftz(d.x), ex2_ftz(d.y)), f);
+}
+
+// The first four samples of a galaxy (L as lse_reset leaves it): their largest log2 weight is the
+// reference, unless every weight is zero.
+template <int FAMILY, bool HAS_B>
+__device__ __forceinline__ void eval_first(const ShearConst &c, const Chunk &ch, Lse &L)
+{
+    float2 x[2], fw[2], ru[2], pp[2], rr[2], qq[2];
+    const float2 e1[2] = {make_float2(ch.e1.x, ch.e1.y), make_float2(ch.e1.z, ch.e1.w)};
+    const float2 e2[2] = {make_float2(ch.e2.x, ch.e2.y), make_float2(ch.e2.z, ch.e2.w)};
+    const float2 bb[2] = {make_float2(ch.b.x, ch.b.y), make_float2(ch.b.z, ch.b.w)};
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        pair_terms<FAMILY, HAS_B>(c, e1[h], e2[h], bb[h], x[h], fw[h], ru[h], pp[h], rr[h], qq[h]);
+    const float mloc = fmaxf(fmaxf(x[0].x, x[0].y), fmaxf(x[1].x, x[1].y));
+    if (mloc - L.m > 32.0f) L.m = mloc;
+    const float2 nm = f2(-L.m);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) add_pair(L, pair_weight(x[h], nm, fw[h]), e1[h], e2[h], ru[h], pp[h], rr[h], qq[h]);
+}
+
 template <int FAMILY, bool HAS_B>
 __device__ __forceinline__ void eval_chunk(const ShearConst &c, const Chunk &ch, Lse &L)
 {
@@ -239,15 +295,22 @@ __device__ __forceinline__ void eval_chunk(const ShearConst &c, const Chunk &ch,
         }
     }
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const float2 e = ew[h];
-        const float2 er = mul2(e, ru[h]);
-        const float2 erp = mul2(er, pp[h]);
-        L.sw = add2(L.sw, e);
-        L.t1 = fma2(erp, e1[h], L.t1);
-        L.t2 = fma2(erp, e2[h], L.t2);
-        L.tr = fma2(er, rr[h], L.tr);
-        L.tq = fma2(e, qq[h], L.tq);
+    for (int h = 0; h < 2; ++h) add_pair(L, ew[h], e1[h], e2[h], ru[h], pp[h], rr[h], qq[h]);
+}
+
+// A lane's NQ quads of chunk `chunk` of a galaxy, of which nq exist.
+template <int FAMILY, bool HAS_B, int NQ, class Quad>
+__device__ __forceinline__ void eval_lane_chunk(const ShearConst &c, int chunk, int nq, Quad quad, Lse &L)
+{
+    if (chunk == 0) {
+        if (nq > 0) eval_first<FAMILY, HAS_B>(c, quad(0), L);
+#pragma unroll
+        for (int h = 1; h < NQ; ++h)
+            if (h < nq) eval_chunk<FAMILY, HAS_B>(c, quad(h), L);
+    } else {
+#pragma unroll
+        for (int h = 0; h < NQ; ++h)
+            if (h < nq) eval_chunk<FAMILY, HAS_B>(c, quad(h), L);
     }
 }
 
@@ -357,141 +420,34 @@ __global__ void __launch_bounds__(kShearThreads, 3) shear_kernel(const __grid_co
     block_partials<kGroup>(s, acc);
 }
 
-// Asynchronous 16-byte global -> shared copies (L2 only), grouped per chunk.
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
-{
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// 4 lanes per galaxy and 12-sample chunks: a group spans 48 samples per step
-// (336 slots for K = 300), the ring's per-chunk bookkeeping is shared by 12
-// samples per lane.  Launch bounds for 3 CTAs (24 warps) per SM leave 80
-// registers, so that the chunk's exponentials and sums are not serialised for
-// lack of them (measured with the tile-streamed kernel below: 2,080 passes/s
-// against 1,993 at 4 CTAs and 64 registers and 1,934 at 2 CTAs).  Measured on
-// one GPU for this kernel at 4 CTAs: 8 lanes x 8 samples x 3 stages (3 CTAs)
-// 1,793 passes/s, 4 x 16 x 2 (3 CTAs) 1,864, 4 x 8 x 2 1,883, 4 x 12 x 2 1,904.
-constexpr int kAGroup = 4;     // lanes per galaxy
-constexpr int kStages = 2;     // chunks per lane in flight, this one included
-constexpr int kAsyncBlocks = 3;   // CTAs per SM the launch bounds target (80 registers)
-constexpr int kChunk = 12;     // samples per lane per chunk (kChunk / 4 16-byte copies per array)
+constexpr int kAGroup = 4;     // lanes per galaxy of the tile-streamed kernels
+constexpr int kChunk = 12;     // samples per lane per chunk
 constexpr int kQuads = kChunk / 4;
 
-__host__ __device__ constexpr size_t async_smem_bytes(bool has_b)
-{
-    return (size_t)kStages * (has_b ? 3 : 2) * kQuads * kShearThreads * sizeof(float4);
-}
-
-// K % 4 == 0 and 16-byte aligned rows: each lane streams its 12-sample chunks
-// through a kStages-deep ring of its own shared-memory slots with cp.async,
-// over the flattened sequence (galaxy, chunk) of its group, so the pipeline
-// does not drain between galaxies.  A lane only reads the slots it filled,
-// after cp.async.wait_group; no barrier is needed.
-template <int FAMILY, bool HAS_B>
-__global__ void __launch_bounds__(kShearThreads, HAS_B ? 3 : kAsyncBlocks) shear_kernel_async(const __grid_constant__ ShearLaunch s)
-{
-    extern __shared__ float4 sbuf[];
-    constexpr int NV = HAS_B ? 3 : 2;
-    const int tid = threadIdx.x;
-    const int lane = tid & 31;
-    const int sub = lane & (kAGroup - 1);
-    const unsigned gmask = ((1u << kAGroup) - 1u) << (lane & ~(kAGroup - 1));
-    const long long group = ((long long)blockIdx.x * blockDim.x + tid) / kAGroup;
-    const long long ngroups = (long long)gridDim.x * blockDim.x / kAGroup;
-    const ShearConst &c = s.c;
-    const int K = s.K;
-    constexpr int span = kChunk * kAGroup;                   // samples of a group per chunk step
-    const int cpg = (K + span - 1) / span;                   // chunks per galaxy per lane
-    const long long my_gal = group < s.n_gal ? (s.n_gal - 1 - group) / ngroups + 1 : 0;
-    const long long n_items = my_gal * cpg;
-    double acc = 0.0;
-    // slot (stage, array, half) of this thread
-    auto slot = [&](int st, int arr, int q) -> float4 * {
-        return &sbuf[((st * NV + arr) * kQuads + q) * kShearThreads + tid];
-    };
-
-    // issuer position: galaxy, chunk, ring slot
-    long long in = group;
-    int ic = 0, ist = 0;
-    auto issue = [&]() {
-        if (in < s.n_gal) {
-            const int k0 = kChunk * sub + span * ic;
-            const long long off = in * (long long)K + k0;
-#pragma unroll
-            for (int h = 0; h < kQuads; ++h) {
-                if (k0 + 4 * h < K) {
-                    cp_async16(slot(ist, 0, h), s.e1 + off + 4 * h);
-                    cp_async16(slot(ist, 1, h), s.e2 + off + 4 * h);
-                    if (HAS_B) cp_async16(slot(ist, 2, h), s.b + off + 4 * h);
-                }
-            }
-            if (++ic == cpg) {
-                ic = 0;
-                in += ngroups;
-            }
-        }
-        cp_async_commit();
-        ist = ist + 1 == kStages ? 0 : ist + 1;
-    };
-#pragma unroll
-    for (int t = 0; t < kStages - 1; ++t) issue();
-
-    Lse L;
-    lse_reset(L);
-    int cc = 0, cst = 0;     // consumer: chunk within the galaxy, ring slot
-    long long cn = group;    // consumer galaxy
-    for (long long t = 0; t < n_items; ++t) {
-        issue();
-        cp_async_wait<kStages - 1>();
-        const int k0 = kChunk * sub + span * cc;
-#pragma unroll
-        for (int h = 0; h < kQuads; ++h) {
-            Chunk ch;
-            ch.nvalid = k0 + 4 * h < K ? 4 : 0;
-            ch.full = ch.nvalid == 4;
-            if (ch.full) {
-                ch.e1 = *slot(cst, 0, h);
-                ch.e2 = *slot(cst, 1, h);
-                ch.b = HAS_B ? *slot(cst, 2, h) : make_float4(0.f, 0.f, 0.f, 0.f);
-                eval_chunk<FAMILY, HAS_B>(c, ch, L);
-            }
-        }
-        cst = cst + 1 == kStages ? 0 : cst + 1;
-        if (++cc == cpg) {
-            cc = 0;
-            finish_galaxy<kAGroup>(L, s.g1, s.g2, gmask, sub, s.w, cn, acc);
-            cn += ngroups;
-            lse_reset(L);
-        }
-    }
-    cp_async_wait<0>();
-    block_partials<kAGroup>(s, acc);
-}
-
-// ---- Tensor-memory-accelerator tiles (no b): a CTA streams tiles of kTileG
-// consecutive galaxies x kTileK samples of e1 and e2 with 2-D
-// cp.async.bulk.tensor loads into a kTmaStages-deep ring; one thread issues both
+// ---- Tensor-memory-accelerator tiles (K a multiple of 4, 16-byte aligned rows): a CTA streams
+// tiles of kTileG consecutive galaxies x kTileK samples of e1 and e2 (and b) with 2-D
+// cp.async.bulk.tensor loads into a ring of two or three stages; one thread issues the
 // loads of a stage and arms the stage's mbarrier with their byte count, and the
 // others wait on it.  Thread t serves galaxy t / 4 of the tile and its samples
-// [12 (t mod 4), + 12) of each chunk (the cp.async kernel's group of 4 lanes and
-// 12-sample chunks).  Galaxies past n_gal and samples past K arrive zero-filled and
+// [12 (t mod 4), + 12) of each chunk.  Galaxies past n_gal and samples past K arrive zero-filled and
 // are masked by index.  A wait gives up after two seconds: the CTA then writes NaN
 // partials, so that the pass's value is NaN.
 constexpr int kTileG = kShearThreads / kAGroup;   // 64 galaxies per tile
 constexpr int kTileK = kChunk * kAGroup;          // 48 samples per chunk
-constexpr int kTmaStages = 3;
+// stages of a ring of NV arrays: 72 KB either way, so that 3 CTAs fit an SM
+__host__ __device__ constexpr int tma_stages(int nv) { return nv == 3 ? 2 : 3; }
+// Launch bounds for 2 CTAs per SM, of whose 128 registers the compiler takes 78: 3 CTAs are resident
+// and nothing is rebuilt or spilled.  10^6 x 300 (no b): 446 us so (5.4 TB/s), 472 us bounded
+// for 3 CTAs, 476 us before the constants were held, 539 us with 4 stages (2 CTAs fit).
+// With b, 3.6 GB: 612 us; 712 us through per-lane cp.async copies, whose kernel this
+// replaced.  What is left is the memory: the warps' waits find their tile late, and
+// deeper rings per warp or L2 prefetches of whole tiles made the pass slower (516-690 us).
+constexpr int kTmaBlocks = 2;
 constexpr int kTileFloats = kTileG * kTileK;      // one array's box, 12 KB
 
-__host__ __device__ constexpr size_t tma_smem_bytes()
+__host__ __device__ constexpr size_t tma_smem_bytes(bool has_b)
 {
-    return (size_t)kTmaStages * 2 * kTileFloats * sizeof(float) + 128;   // + alignment of the ring
+    return (size_t)tma_stages(has_b ? 3 : 2) * (has_b ? 3 : 2) * kTileFloats * sizeof(float) + 128;   // + alignment of the ring
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -519,12 +475,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
     }
 }
 
-// The CTA's ring of kTmaStages stages, each one tile-chunk of e1 and e2, with a
+// The CTA's ring of kStages stages, each one tile-chunk of NV arrays (e1, e2 and b), with a
 // "full" mbarrier per stage (armed by the producer with the stage's byte count) and an
 // "empty" one (one arrival per warp once the warp has read the stage).  Thread 0 is
 // the producer: it issues item i (tile blockIdx.x + t gridDim.x, chunk c) after the
 // stage's previous item has been released.  Every wait gives up after two seconds.
+template <int NV>
 struct TmaRing {
+    static constexpr int kStages = tma_stages(NV);
     float *ring;
     uint64_t *full, *empty;
     int cpg, n_items;
@@ -545,7 +503,7 @@ struct TmaRing {
         n_items = my_tiles * cpg;
         p_tile = blockIdx.x;
         if (threadIdx.x == 0) {
-            for (int st = 0; st < kTmaStages; ++st) {
+            for (int st = 0; st < kStages; ++st) {
                 asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&full[st])) : "memory");
                 asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&empty[st])), "r"(kWarps)
                              : "memory");
@@ -554,32 +512,30 @@ struct TmaRing {
         }
         __syncthreads();
     }
-    __device__ void issue(const CUtensorMap *m1, const CUtensorMap *m2)
+    __device__ void issue(const CUtensorMap *m1, const CUtensorMap *m2, const CUtensorMap *m3)
     {
         if (p_item >= n_items || !p_ok) return;
-        const int st = p_item % kTmaStages;
-        if (p_item >= kTmaStages) {   // the stage's previous item has been read by every warp
-            if (!mbar_wait(smem_u32(&empty[st]), (uint32_t)((p_item / kTmaStages - 1) & 1))) {
+        const int st = p_item % kStages;
+        if (p_item >= kStages) {   // the stage's previous item has been read by every warp
+            if (!mbar_wait(smem_u32(&empty[st]), (uint32_t)((p_item / kStages - 1) & 1))) {
                 p_ok = false;
                 return;
             }
         }
         const uint32_t bar = smem_u32(&full[st]);
-        const uint32_t d1 = smem_u32(ring + (size_t)st * 2 * kTileFloats), d2 = d1 + kTileFloats * 4;
+        const uint32_t d = smem_u32(ring + (size_t)st * NV * kTileFloats);
         const int x = p_chunk * kTileK, y = (int)(p_tile * kTileG);
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
-                     "r"((uint32_t)(2 * kTileFloats * 4))
+                     "r"((uint32_t)(NV * kTileFloats * 4))
                      : "memory");
-        asm volatile(
-            "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
-                "r"(d1),
-            "l"(m1), "r"(x), "r"(y), "r"(bar)
-            : "memory");
-        asm volatile(
-            "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
-                "r"(d2),
-            "l"(m2), "r"(x), "r"(y), "r"(bar)
-            : "memory");
+        const CUtensorMap *maps[3] = {m1, m2, m3};
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+            asm volatile(
+                "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
+                    "r"(d + v * kTileFloats * 4),
+                "l"(maps[v]), "r"(x), "r"(y), "r"(bar)
+                : "memory");
         ++p_item;
         if (++p_chunk == cpg) {
             p_chunk = 0;
@@ -590,14 +546,14 @@ struct TmaRing {
     __device__ bool wait_full(int item) const
     {
         return __all_sync(BS_FULL_MASK,
-                          mbar_wait(smem_u32(&full[item % kTmaStages]), (uint32_t)((item / kTmaStages) & 1)));
+                          mbar_wait(smem_u32(&full[item % kStages]), (uint32_t)((item / kStages) & 1)));
     }
     // all threads of a warp, after reading item's stage
     __device__ void release(int item) const
     {
         __syncwarp();
         if ((threadIdx.x & 31) == 0)
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[item % kTmaStages]))
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[item % kStages]))
                          : "memory");
     }
     // all threads, at the end: loads still in flight land in the ring (waited for, with the limit)
@@ -605,45 +561,53 @@ struct TmaRing {
     {
         __syncthreads();
         if (threadIdx.x == 0) {
-            for (int it = p_item - kTmaStages; it < p_item; ++it)
-                if (it >= 0) mbar_wait(smem_u32(&full[it % kTmaStages]), (uint32_t)((it / kTmaStages) & 1));
+            for (int it = p_item - kStages; it < p_item; ++it)
+                if (it >= 0) mbar_wait(smem_u32(&full[it % kStages]), (uint32_t)((it / kStages) & 1));
         }
     }
 };
 
-// Quad h (4 consecutive samples) of this thread's part of chunk `chunk` of its
-// galaxy (4 lanes per galaxy, 12 samples each) in item's stage; false past K.
-__device__ __forceinline__ bool tma_quad(const TmaRing &R, int item, int K, int chunk, int h, Chunk &ch)
+// Quad h (4 consecutive samples) of this thread's part of a chunk of its galaxy (4 lanes
+// per galaxy, 12 samples each) in item's stage, and how many quads of it lie below K.
+template <int NV>
+__device__ __forceinline__ Chunk tma_quad(const TmaRing<NV> &R, int item, int h)
 {
     const int tid = threadIdx.x, sub = tid & (kAGroup - 1), gl = tid / kAGroup;
-    if (chunk * kTileK + kChunk * sub + 4 * h >= K) return false;
-    const float *r1 = R.ring + (size_t)(item % kTmaStages) * 2 * kTileFloats + gl * kTileK + kChunk * sub + 4 * h;
+    const float *r1 = R.ring + (size_t)(item % TmaRing<NV>::kStages) * NV * kTileFloats + gl * kTileK + kChunk * sub + 4 * h;
+    Chunk ch;
     ch.nvalid = 4;
     ch.full = true;
     ch.e1 = *reinterpret_cast<const float4 *>(r1);
     ch.e2 = *reinterpret_cast<const float4 *>(r1 + kTileFloats);
-    ch.b = make_float4(0.f, 0.f, 0.f, 0.f);
-    return true;
+    ch.b = NV == 3 ? *reinterpret_cast<const float4 *>(r1 + 2 * kTileFloats) : make_float4(0.f, 0.f, 0.f, 0.f);
+    return ch;
+}
+__device__ __forceinline__ int tma_quads(int K, int chunk)
+{
+    const int left = (K - chunk * kTileK - kChunk * (int)(threadIdx.x & (kAGroup - 1)) + 3) >> 2;
+    return left < 0 ? 0 : left < kQuads ? left : kQuads;
 }
 
-template <int FAMILY>
-__global__ void __launch_bounds__(kShearThreads, kAsyncBlocks)
-    shear_kernel_tma(const __grid_constant__ ShearLaunch s, const __grid_constant__ CUtensorMap m1, const __grid_constant__ CUtensorMap m2)
+template <int FAMILY, bool HAS_B>
+__global__ void __launch_bounds__(kShearThreads, kTmaBlocks)
+    shear_kernel_tma(const __grid_constant__ ShearLaunch s, const __grid_constant__ CUtensorMap m1,
+                     const __grid_constant__ CUtensorMap m2, const __grid_constant__ CUtensorMap m3)
 {
     extern __shared__ __align__(128) unsigned char tma_raw[];
-    __shared__ __align__(8) uint64_t full[kTmaStages], empty[kTmaStages];
+    constexpr int NV = HAS_B ? 3 : 2, NS = tma_stages(NV);
+    __shared__ __align__(8) uint64_t full[NS], empty[NS];
     __shared__ int s_fail;
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int sub = tid & (kAGroup - 1), gl = tid / kAGroup;
     const unsigned gmask = ((1u << kAGroup) - 1u) << (lane & ~(kAGroup - 1));
-    const ShearConst &c = s.c;
+    const ShearConst c = held(s.c);
     const int K = s.K;
     if (tid == 0) s_fail = 0;
-    TmaRing R;
+    TmaRing<NV> R;
     R.init(tma_raw, full, empty, s.n_gal, K);   // (its barrier also orders the reset above)
     if (tid == 0)
-        for (int t = 0; t < kTmaStages - 1; ++t) R.issue(&m1, &m2);
+        for (int t = 0; t < NS - 1; ++t) R.issue(&m1, &m2, &m3);
     double acc = 0.0;
     Lse L;
     lse_reset(L);
@@ -651,18 +615,15 @@ __global__ void __launch_bounds__(kShearThreads, kAsyncBlocks)
     int chunk = 0;
     long long tile = blockIdx.x;
     for (int item = 0; item < R.n_items; ++item) {
-        if (tid == 0) R.issue(&m1, &m2);
+        if (tid == 0) R.issue(&m1, &m2, &m3);
         if (!R.wait_full(item)) {
             failed = true;
             break;
         }
         const long long n = tile * kTileG + gl;
         if (n < s.n_gal) {
-#pragma unroll
-            for (int h = 0; h < kQuads; ++h) {
-                Chunk ch;
-                if (tma_quad(R, item, K, chunk, h, ch)) eval_chunk<FAMILY, false>(c, ch, L);
-            }
+            eval_lane_chunk<FAMILY, HAS_B, kQuads>(c, chunk, tma_quads(K, chunk),
+                                                   [&](int h) { return tma_quad(R, item, h); }, L);
         }
         R.release(item);
         if (++chunk == R.cpg) {
@@ -910,28 +871,20 @@ __global__ void __launch_bounds__(256) shear_finalize_n_kernel(const double *par
 template <int FAMILY, bool HAS_B>
 cudaError_t launch_fb(const ShearLaunch &s, int grid, bool vec, cudaStream_t st)
 {
-    if (vec && !HAS_B) {
-        // e1, e2 as tensor maps, streamed in tiles by the tensor memory accelerator
-        CUtensorMap m1, m2;
-        if (make_sample_map(m1, s.e1, s.n_gal, s.K) && make_sample_map(m2, s.e2, s.n_gal, s.K)) {
-            const cudaError_t e = cudaFuncSetAttribute(shear_kernel_tma<FAMILY>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       (int)tma_smem_bytes());
+    if (vec) {
+        // the samples as tensor maps, streamed in tiles by the tensor memory accelerator
+        CUtensorMap m1, m2, m3;
+        if (make_sample_map(m1, s.e1, s.n_gal, s.K) && make_sample_map(m2, s.e2, s.n_gal, s.K) &&
+            make_sample_map(m3, HAS_B ? s.b : s.e1, s.n_gal, s.K)) {
+            constexpr size_t smem = tma_smem_bytes(HAS_B);
+            const cudaError_t e = cudaFuncSetAttribute(shear_kernel_tma<FAMILY, HAS_B>,
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
-            shear_kernel_tma<FAMILY><<<grid, kShearThreads, tma_smem_bytes(), st>>>(s, m1, m2);
+            shear_kernel_tma<FAMILY, HAS_B><<<grid, kShearThreads, smem, st>>>(s, m1, m2, m3);
             return cudaGetLastError();
         }
     }
-    if (vec) {
-        // the ring (48 KB, 72 KB with b) plus the static reduction buffer is
-        // above the default dynamic shared-memory limit
-        const cudaError_t e = cudaFuncSetAttribute(shear_kernel_async<FAMILY, HAS_B>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)async_smem_bytes(HAS_B));
-        if (e != cudaSuccess) return e;
-        shear_kernel_async<FAMILY, HAS_B><<<grid, kShearThreads, async_smem_bytes(HAS_B), st>>>(s);
-    } else
-        shear_kernel<FAMILY, HAS_B><<<grid, kShearThreads, 0, st>>>(s);
+    shear_kernel<FAMILY, HAS_B><<<grid, kShearThreads, 0, st>>>(s);
     return cudaGetLastError();
 }
 
@@ -1036,7 +989,7 @@ GridCache g_grid_one, g_grid_full, g_grid_multi;
 
 int shear_grid_blocks()
 {
-    return resident_grid(g_grid_one, shear_kernel_async<BS_EPRIOR_BA14, false>, async_smem_bytes(false));
+    return resident_grid(g_grid_one, shear_kernel_tma<BS_EPRIOR_TRUNC_GAUSS, false>, tma_smem_bytes(false));
 }
 
 int shear_grid_for(long long n_gal)
@@ -1098,7 +1051,7 @@ __global__ void __launch_bounds__(kShearThreads, 2)
 {
     constexpr int NP = kMultiPoints;
     extern __shared__ __align__(128) unsigned char tma_raw[];
-    __shared__ __align__(8) uint64_t full[kTmaStages], empty[kTmaStages];
+    __shared__ __align__(8) uint64_t full[tma_stages(2)], empty[tma_stages(2)];
     __shared__ double acc[kTileG][NP][4];
     __shared__ int s_fail;
     const ShearLaunch &s = m.s;
@@ -1111,10 +1064,10 @@ __global__ void __launch_bounds__(kShearThreads, 2)
         for (int p = 0; p < NP; ++p)
             for (int i = 0; i < 4; ++i) acc[gl][p][i] = 0.0;
     if (tid == 0) s_fail = 0;
-    TmaRing R;
+    TmaRing<2> R;
     R.init(tma_raw, full, empty, s.n_gal, K);   // (its barrier also orders the resets above)
     if (tid == 0)
-        for (int t = 0; t < kTmaStages - 1; ++t) R.issue(&m1, &m2);
+        for (int t = 0; t < tma_stages(2) - 1; ++t) R.issue(&m1, &m2, nullptr);
     Lse L[NP];
 #pragma unroll
     for (int p = 0; p < NP; ++p) lse_reset(L[p]);
@@ -1122,17 +1075,18 @@ __global__ void __launch_bounds__(kShearThreads, 2)
     int chunk = 0;
     long long tile = blockIdx.x;
     for (int item = 0; item < R.n_items; ++item) {
-        if (tid == 0) R.issue(&m1, &m2);
+        if (tid == 0) R.issue(&m1, &m2, nullptr);
         if (!R.wait_full(item)) {
             failed = true;
             break;
         }
         const long long n = tile * kTileG + gl;
         if (n < s.n_gal) {
+            const int nq = tma_quads(K, chunk);
 #pragma unroll
             for (int h = 0; h < kQuads; ++h) {
-                Chunk ch;
-                if (tma_quad(R, item, K, chunk, h, ch)) {
+                if (h < nq) {
+                    const Chunk ch = tma_quad(R, item, h);
 #pragma unroll
                     for (int p = 0; p < NP; ++p)
                         if (p < m.n_points) eval_chunk<FAMILY, false>(m.c[p], ch, L[p]);
@@ -1178,9 +1132,9 @@ cudaError_t launch_shear_multi(const ShearMultiLaunch &m, int grid, cudaStream_t
         auto k = s.family == BS_EPRIOR_BA14 ? shear_kernel_tma_multi<BS_EPRIOR_BA14>
                                             : shear_kernel_tma_multi<BS_EPRIOR_TRUNC_GAUSS>;
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)tma_smem_bytes());
+                                                   (int)tma_smem_bytes(false));
         if (e != cudaSuccess) return e;
-        k<<<grid, kShearThreads, tma_smem_bytes(), stream>>>(m, m1, m2);
+        k<<<grid, kShearThreads, tma_smem_bytes(false), stream>>>(m, m1, m2);
         return cudaGetLastError();
     }
     if (m.s.family == BS_EPRIOR_BA14)
