@@ -66,18 +66,6 @@ __device__ __forceinline__ float rcp_ftz(float x)
     return r;
 }
 
-// log2 of a galaxy's sum of weights (a normal positive float), once per galaxy:
-// the exponent exactly and the mantissa's logarithm, in [-1, 0), to about
-// 6e-8 by the accurate log2f.  The hardware approximation's absolute error
-// (about 2^-22, the same sign for sums of the same size) would add up over
-// 10^6 galaxies to a shift of the total of a few tenths of a nat.
-__device__ __forceinline__ double log2_total(float x)
-{
-    int e;
-    const float m = frexpf(x, &e);      // x = m 2^e, m in [0.5, 1)
-    return (double)e + (double)log2f(m);
-}
-
 // Packed FP32x2 arithmetic: two samples per instruction, each half rounded
 // like the scalar operation.
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
@@ -350,7 +338,11 @@ __device__ __forceinline__ void finish_galaxy(const Lse &L, float g1, float g2, 
         const float d = sub == 1 ? -2.0f * t1 * inv : sub == 2 ? -2.0f * t2 * inv : tq * inv;
         // lane 0: m + log2(sw), the other lanes d + 0
         int e;
-        const float l = log2f(frexpf(sw, &e));   // as log2_total
+        // log2 of the sum of weights: the exponent exactly and the mantissa's logarithm, in [-1, 0),
+        // to about 6e-8 by the accurate log2f.  The hardware approximation's absolute error
+        // (about 2^-22, the same sign for sums of the same size) would add up over
+        // 10^6 galaxies to a shift of the total of a few tenths of a nat.
+        const float l = log2f(frexpf(sw, &e));
         double v = (double)(sub == 0 ? m : d);
         if (sub == 0) v += (double)e + (double)l;
         if (w) v *= (double)wf;
@@ -704,7 +696,9 @@ __global__ void __launch_bounds__(128) shear_finalize_batch_kernel(const double 
 // ---- all properties free ----------------------------------------------------
 
 // log Phi(t) and the inverse Mills ratio phi(t)/Phi(t) of the standard normal,
-// through erfcx on the left tail so that neither underflows.
+// through erfcx on the left tail so that neither underflows.  On the right, 1 - Phi = q below
+// 2^-25 makes 1 - q round to 1 and log1p(-q) to -q (from t = 6), and from t = 14.5 on both q
+// and phi underflow to 0: the shorter forms give the bits of the general one.
 __device__ __forceinline__ void log_ndtr_mills(float t, float &lphi, float &r)
 {
     if (t < 0.0f) {
@@ -712,132 +706,200 @@ __device__ __forceinline__ void log_ndtr_mills(float t, float &lphi, float &r)
         const float ex = erfcxf(u);                 // exp(u^2) erfc(u)
         lphi = logf(0.5f * ex) - u * u;
         r = 0.79788456080286536f / ex;              // sqrt(2/pi) / erfcx
+    } else if (t >= 14.5f) {
+        lphi = -0.0f;
+        r = 0.0f;
     } else {
         const float q = 0.5f * erfcf(t * 0.70710678118654752f);   // 1 - Phi(t)
-        lphi = log1pf(-q);
-        r = 0.39894228040143268f * expf(-0.5f * t * t) / (1.0f - q);
+        const float ph = 0.39894228040143268f * expf(-0.5f * t * t);
+        if (t >= 6.0f) {
+            lphi = -q;
+            r = ph;
+        } else {
+            lphi = log1pf(-q);
+            r = ph / (1.0f - q);
+        }
     }
 }
 
+// The running sums of one lane, in pairs for the packed arithmetic: the reference log2 weight, the
+// sum of weights, (t1, t2) on the shear, (sum w Q, sum w y), and sum w of (z - a r, z (z - a r)),
+// (r z, y^2).
 struct FullAcc {
-    float m, sw, t1, t2, tq, h[5];
+    float m, sw;
+    float2 t, qy, h01, h24;
 };
 
-// One sample: log2 weight of the ellipticity part (as pair_terms, scalar) plus
+// Two samples of a lane in packed arithmetic (each half rounded like the scalar
+// operation): log2 weight of the ellipticity part (as pair_terms, with the logarithm) plus
 // the flux/size log prior ratio up to per-galaxy constants,
 //   -z^2/2 + log Phi(a z) - y^2/2,  z = (lf - mu_f)/sigma_f, y = (ls - mu_s)/sigma_s,
 // and the factors of its derivatives (times sigma where that is constant):
-//   (z - a r), z (z - a r), r z, y, y^2,  r = phi(a z)/Phi(a z).
+//   (z - a r), z (z - a r), r z, y, y^2,  r = phi(a z)/Phi(a z);
+// then the two samples in turn into the sums.  na, nb: (log Phi, r, z) of the two.
 template <int FAMILY>
-__device__ __forceinline__ void full_sample(const ShearFullLaunch &f, float an, float e1, float e2, float lf,
-                                            float ls, bool valid, FullAcc &A)
+__device__ __forceinline__ void full_pair(const ShearFullLaunch &f, const ShearConst &c, float2 e1, float2 e2, float2 ls,
+                                          const float4 &na, const float4 &nb, int n_valid, FullAcc &A)
 {
-    const ShearLaunch &s = f.s;
-    const float Ep = fmaf(e1, e1, e2 * e2);
-    const float ge = fmaf(s.g1, e1, s.g2 * e2);
-    const float U = fmaf(s.g1 * s.g1 + s.g2 * s.g2, Ep, fmaf(-2.0f, ge, 1.0f));   // Lagrange form
-    const float n1 = e1 - s.g1, n2 = e2 - s.g2;
-    const float rU = rcp_ftz(U);
-    const float Q = fmaf(n1, n1, n2 * n2) * rU;
-    const float larg = FAMILY == BS_EPRIOR_TRUNC_GAUSS ? U * (1.0f - Ep) : U;
-    const float lgk = FAMILY == BS_EPRIOR_TRUNC_GAUSS ? -2.0f : -s.kappa;
-    float x = fmaf(s.c0, Ep, fmaf(lgk, lg2_ftz(larg), -s.a2 * Q));
-    if (FAMILY == BS_EPRIOR_TRUNC_GAUSS && !(Q < s.r2)) x = -INFINITY;
-    const float aqk = fmaf(an, Q, -s.kappa);
-    const float du1 = fmaf(-s.g1, Ep, e1);
-    const float du2 = fmaf(-s.g2, Ep, e2);
-    const float c1 = fmaf(du1, aqk, -an * n1);
-    const float c2 = fmaf(du2, aqk, -an * n2);
-    const float z = (lf - f.mu_f) * f.inv_sf;
-    const float y = (ls - f.mu_s) * f.inv_ss;
-    float lphi, r;
-    log_ndtr_mills(f.a_f * z, lphi, r);
-    x = fmaf(kLog2e, lphi - 0.5f * fmaf(z, z, y * y), x);
-    if (!valid) x = -INFINITY;
-    if (x > A.m) {
-        const float sc = ex2_ftz(A.m - x);
-        A.sw *= sc;
-        A.t1 *= sc;
-        A.t2 *= sc;
-        A.tq *= sc;
-#pragma unroll
-        for (int i = 0; i < 5; ++i) A.h[i] *= sc;
-        A.m = x;
+    const float2 Ep = fma2(e1, e1, mul2(e2, e2));
+    const float2 ge = fma2(c.g1, e1, mul2(c.g2, e2));
+    const float2 U = fma2(c.gg, Ep, fma2(f2(-2.0f), ge, f2(1.0f)));   // Lagrange form
+    const float2 n1 = sub2(e1, c.g1), n2 = sub2(e2, c.g2);
+    const float2 rU = make_float2(rcp_ftz(U.x), rcp_ftz(U.y));
+    const float2 Q = mul2(fma2(n1, n1, mul2(n2, n2)), rU);
+    const float2 larg = FAMILY == BS_EPRIOR_TRUNC_GAUSS ? mul2(U, sub2(f2(1.0f), Ep)) : U;
+    const float lgk = FAMILY == BS_EPRIOR_TRUNC_GAUSS ? -2.0f : -4.0f;    // -kappa of the family
+    const float2 lg = make_float2(lg2_ftz(larg.x), lg2_ftz(larg.y));
+    float2 x = fma2(c.c0, Ep, fma2(f2(lgk), lg, mul2(c.a2n, Q)));
+    if (FAMILY == BS_EPRIOR_TRUNC_GAUSS) {
+        if (!(Q.x < c.r2)) x.x = -INFINITY;
+        if (!(Q.y < c.r2)) x.y = -INFINITY;
     }
-    const float e = ex2_ftz(x - A.m);
-    const float er = e * rU;
-    const float h0 = fmaf(-f.a_f, r, z);
-    A.sw += e;
-    A.t1 = fmaf(er, c1, A.t1);
-    A.t2 = fmaf(er, c2, A.t2);
-    A.tq = fmaf(e, Q, A.tq);
-    A.h[0] = fmaf(e, h0, A.h[0]);
-    A.h[1] = fmaf(e, z * h0, A.h[1]);
-    A.h[2] = fmaf(e, r * z, A.h[2]);
-    A.h[3] = fmaf(e, y, A.h[3]);
-    A.h[4] = fmaf(e, y * y, A.h[4]);
+    const float2 aqk = fma2(c.an, Q, c.nk);
+    const float2 du1 = fma2(f2(-f.s.g1), Ep, e1), du2 = fma2(f2(-f.s.g2), Ep, e2);
+    const float2 c1 = fma2(du1, aqk, mul2(c.nan, n1)), c2 = fma2(du2, aqk, mul2(c.nan, n2));
+    const float2 lphi = make_float2(na.x, nb.x), r = make_float2(na.y, nb.y), z = make_float2(na.z, nb.z);
+    const float2 y = mul2(sub2(ls, f2(f.mu_s)), f2(f.inv_ss));
+    const float2 yy = mul2(y, y);
+    x = fma2(f2(kLog2e), fma2(f2(-0.5f), fma2(z, z, yy), lphi), x);
+    const float2 h0 = fma2(f2(-f.a_f), r, z);
+    const float2 zh = mul2(z, h0), rz = mul2(r, z);
+    auto add = [&](float xs, float q, float ru, float d1, float d2, float v0, float v1, float v2, float vy, float vyy) {
+        if (xs > A.m) {
+            const float2 sc = f2(ex2_ftz(A.m - xs));
+            A.sw *= sc.x;
+            A.t = mul2(A.t, sc);
+            A.qy = mul2(A.qy, sc);
+            A.h01 = mul2(A.h01, sc);
+            A.h24 = mul2(A.h24, sc);
+            A.m = xs;
+        }
+        const float e = ex2_ftz(xs - A.m);
+        A.sw += e;
+        A.t = fma2(f2(e * ru), make_float2(d1, d2), A.t);
+        A.qy = fma2(f2(e), make_float2(q, vy), A.qy);
+        A.h01 = fma2(f2(e), make_float2(v0, v1), A.h01);
+        A.h24 = fma2(f2(e), make_float2(v2, vyy), A.h24);
+    };
+    if (n_valid > 0) add(x.x, Q.x, rU.x, c1.x, c2.x, h0.x, zh.x, rz.x, y.x, yy.x);
+    if (n_valid > 1) add(x.y, Q.y, rU.y, c1.y, c2.y, h0.y, zh.y, rz.y, y.y, yy.y);
 }
 
+// A warp takes four galaxies, eight lanes each (lane j of eight: samples j, j + 8, ...), in blocks
+// of 32 samples.  The normal-CDF terms of a block are formed first, one galaxy at a time over
+// all 32 lanes: a galaxy's samples are mostly on one side of mu_f, so that the branches
+// of log_ndtr_mills seldom diverge, which four galaxies side by side do; they pass through
+// shared memory to the lanes that sum them.  Bound by instruction issue.
+// 100,000 x 300: 0.45 ms with the terms formed where they are summed, in scalar arithmetic, an
+// output at a time through the FP64 pipe; 0.30 ms now (0.40 with prefetched loads and the FP64
+// sums side by side alone).
 template <int FAMILY>
-__global__ void __launch_bounds__(kShearThreads, 2) shear_full_kernel(const ShearFullLaunch f)
+__global__ void __launch_bounds__(kShearThreads, 3) shear_full_kernel(const __grid_constant__ ShearFullLaunch f)
 {
+    __shared__ float4 s_norm[kShearThreads / 32][4][33];   // (log Phi, r, z) per galaxy and sample of the block
     const ShearLaunch &s = f.s;
-    const int lane = threadIdx.x & 31;
-    const int sub = lane & (kGroup - 1);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int sub = lane & (kGroup - 1), g = lane / kGroup;
     const unsigned gmask = 0xFFu << (lane & ~(kGroup - 1));
-    const long long group = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kGroup;
     const long long ngroups = (long long)gridDim.x * blockDim.x / kGroup;
-    const float an = s.a2 * kLn2;
+    const ShearConst c = held(s.c);
     const int K = s.K;
-    double acc[kShearFullOut];
-#pragma unroll
-    for (int i = 0; i < kShearFullOut; ++i) acc[i] = 0.0;
+    double acc = 0.0, acc8 = 0.0;   // output `sub` of the first eight; the ninth (lane 0)
 
-    for (long long n = group; n < s.n_gal; n += ngroups) {
-        const long long base = n * (long long)K;
+    for (long long n0 = ((long long)blockIdx.x * (kShearThreads / 32) + warp) * 4; n0 < s.n_gal; n0 += ngroups) {
+        const long long n = n0 + g;                        // this lane's galaxy
+        const bool live = n < s.n_gal;
+        const float *p1 = s.e1 + n * (long long)K, *p2 = s.e2 + n * (long long)K;
+        const float *pf = f.lf + n0 * (long long)K, *ps = f.ls + n * (long long)K;
+        const int ng = s.n_gal - n0 < 4 ? (int)(s.n_gal - n0) : 4;
         FullAcc A;
         A.m = -1e30f;
-        A.sw = A.t1 = A.t2 = A.tq = 0.f;
+        A.sw = 0.f;
+        A.t = A.qy = A.h01 = A.h24 = f2(0.f);
+        for (int kb = 0; kb < K; kb += 32) {
+            float v1[4], v2[4], vs[4];
 #pragma unroll
-        for (int i = 0; i < 5; ++i) A.h[i] = 0.f;
-        for (int k = sub; k < K; k += kGroup) {
-            const long long j = base + k;
-            full_sample<FAMILY>(f, an, __ldg(s.e1 + j), __ldg(s.e2 + j), __ldg(f.lf + j), __ldg(f.ls + j), true, A);
+            for (int t = 0; t < 4; ++t) {
+                const int k = kb + 8 * t + sub;
+                const bool in = live && k < K;
+                v1[t] = in ? __ldg(p1 + k) : 0.f;
+                v2[t] = in ? __ldg(p2 + k) : 0.f;
+                vs[t] = in ? __ldg(ps + k) : 0.f;
+            }
+            float vf[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                vf[j] = j < ng && kb + lane < K ? __ldg(pf + (long long)j * K + kb + lane) : f.mu_f;
+#pragma unroll 1
+            for (int j = 0; j < ng; ++j) {
+                const float lf = j == 0 ? vf[0] : j == 1 ? vf[1] : j == 2 ? vf[2] : vf[3];
+                const float z = (lf - f.mu_f) * f.inv_sf;
+                float lphi = 0.f, r = 0.f;
+                if (kb + lane < K) log_ndtr_mills(f.a_f * z, lphi, r);
+                s_norm[warp][j][lane] = make_float4(lphi, r, z, 0.f);
+            }
+            __syncwarp();
+            if (live) {
+                const float4 *sn = s_norm[warp][g];
+#pragma unroll
+                for (int t = 0; t < 4; t += 2) {
+                    const int k = kb + 8 * t + sub;
+                    if (k < K)
+                        full_pair<FAMILY>(f, c, make_float2(v1[t], v1[t + 1]), make_float2(v2[t], v2[t + 1]),
+                                          make_float2(vs[t], vs[t + 1]), sn[8 * t + sub], sn[8 * t + 8 + sub],
+                                          k + 8 < K ? 2 : 1, A);
+                }
+            }
+            __syncwarp();
         }
-        // merge the 8 lanes of the group
-        float v[10] = {A.m, A.sw, A.t1, A.t2, A.tq, A.h[0], A.h[1], A.h[2], A.h[3], A.h[4]};
+        if (!live) continue;
+    // merge the 8 lanes of the group
+        float u[10] = {A.m, A.sw, A.t.x, A.t.y, A.qy.x, A.h01.x, A.h01.y, A.h24.x, A.qy.y, A.h24.y};
 #pragma unroll
         for (int o = kGroup / 2; o > 0; o >>= 1) {
             float w[10];
 #pragma unroll
-            for (int i = 0; i < 10; ++i) w[i] = __shfl_xor_sync(gmask, v[i], o, kGroup);
-            const float mn = fmaxf(v[0], w[0]);
-            const float ca = ex2_ftz(v[0] - mn), cb = ex2_ftz(w[0] - mn);
+            for (int i = 0; i < 10; ++i) w[i] = __shfl_xor_sync(gmask, u[i], o, kGroup);
+            const float mn = fmaxf(u[0], w[0]);
+            const float ca = ex2_ftz(u[0] - mn), cb = ex2_ftz(w[0] - mn);
 #pragma unroll
-            for (int i = 1; i < 10; ++i) v[i] = v[i] * ca + w[i] * cb;
-            v[0] = mn;
+            for (int i = 1; i < 10; ++i) u[i] = u[i] * ca + w[i] * cb;
+            u[0] = mn;
         }
-        const double wn = sub == 0 && s.w ? (double)__ldg(s.w + n) : 1.0;
-        if (sub == 0 && wn != 0.0) {
-            if (v[1] > 0.f) {
-                const float inv = 1.0f / v[1];
-                acc[0] += wn * ((double)v[0] + log2_total(v[1]));
-                acc[1] += wn * (double)(-2.0f * v[2] * inv);
-                acc[2] += wn * (double)(-2.0f * v[3] * inv);
-                acc[3] += wn * (double)(v[4] * inv);
+        // lane 0 takes the log-sum-exp and the last derivative sum, lanes 1-7 a derivative sum
+        // each (one pass through the FP64 pipe for the eight)
+        const float wf = s.w ? __ldg(s.w + n) : 1.0f;
+        if (wf != 0.0f) {
+            if (u[1] > 0.f) {
+                const float inv = 1.0f / u[1];
+                float d = -2.0f * u[2] * inv;
+                if (sub == 2) d = -2.0f * u[3] * inv;
 #pragma unroll
-                for (int i = 0; i < 5; ++i) acc[4 + i] += wn * (double)(v[5 + i] * inv);
-            } else {
-                acc[0] = -INFINITY;
+                for (int i = 4; i < 9; ++i)
+                    if (sub == i - 1) d = u[i] * inv;
+                int e;
+                const float l = log2f(frexpf(u[1], &e));   // as finish_galaxy
+                double t = (double)(sub == 0 ? u[0] : d);
+                if (sub == 0) t += (double)e + (double)l;
+                acc += s.w ? (double)wf * t : t;
+                if (sub == 0) {
+                    const double t8 = (double)(u[9] * inv);
+                    acc8 += s.w ? (double)wf * t8 : t8;
+                }
+            } else if (sub == 0) {
+                acc = -INFINITY;
             }
         }
     }
     __shared__ double red[kShearThreads / 32][kShearFullOut];
 #pragma unroll
-    for (int i = 0; i < kShearFullOut; ++i) acc[i] = warp_sum_d(acc[i]);
+    for (int o = 16; o >= kGroup; o >>= 1) {
+        acc += __shfl_xor_sync(BS_FULL_MASK, acc, o);
+        acc8 += __shfl_xor_sync(BS_FULL_MASK, acc8, o);
+    }
     const int w = threadIdx.x >> 5;
-    if (lane == 0)
-        for (int i = 0; i < kShearFullOut; ++i) red[w][i] = acc[i];
+    if (lane < kGroup) red[w][lane] = acc;
+    if (lane == 0) red[w][kShearFullOut - 1] = acc8;
     __syncthreads();
     if (threadIdx.x < kShearFullOut) {
         double t = 0.0;
@@ -850,22 +912,17 @@ struct FinalizeN {
     double scale[kShearFullOut], add[kShearFullOut];
 };
 
-__global__ void __launch_bounds__(256) shear_finalize_n_kernel(const double *partials, int n_part, int n_out,
-                                                                FinalizeN c, double *out)
+// A warp per output, as finalize_point.
+__global__ void __launch_bounds__(32 * kShearFullOut) shear_finalize_n_kernel(const double *partials, int n_part, int n_out,
+                                                                              const __grid_constant__ FinalizeN c,
+                                                                              double *out)
 {
-    __shared__ double red[256];
-    for (int k = 0; k < n_out; ++k) {
-        double t = 0.0;
-        for (int i = threadIdx.x; i < n_part; i += blockDim.x) t += partials[(size_t)i * n_out + k];
-        red[threadIdx.x] = t;
-        __syncthreads();
-        for (int o = 128; o > 0; o >>= 1) {
-            if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) out[k] = red[0] * c.scale[k] + c.add[k];
-        __syncthreads();
-    }
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double t = 0.0;
+#pragma unroll 8
+    for (int i = lane; i < n_part; i += 32) t += partials[(size_t)i * n_out + k];
+    t = warp_sum_d(t);
+    if (lane == 0) out[k] = t * c.scale[k] + c.add[k];
 }
 
 template <int FAMILY, bool HAS_B>
@@ -1032,7 +1089,7 @@ cudaError_t launch_shear_finalize_n(const double *partials, int n_part, int n_ou
         c.scale[i] = i < n_out ? scale[i] : 0.0;
         c.add[i] = i < n_out ? add[i] : 0.0;
     }
-    shear_finalize_n_kernel<<<1, 256, 0, stream>>>(partials, n_part, n_out, c, out);
+    shear_finalize_n_kernel<<<1, 32 * n_out, 0, stream>>>(partials, n_part, n_out, c, out);
     return cudaGetLastError();
 }
 
