@@ -183,9 +183,10 @@ __device__ __forceinline__ void load_chunk(const ShearLaunch &s, long long base,
     ch.b = make_float4(tb[0], tb[1], tb[2], tb[3]);
 }
 
-// Online log-sum-exp state of one lane (both halves share the maximum).
+// Online log-sum-exp state of one lane (both halves share the reference).
 struct Lse {
-    float m;
+    float m;                 // the reference log2 weight
+    float mx;                // largest log2 weight seen (the tile kernels: eval_quad)
     float2 sw, t1, t2, tq;   // t_i: sum of weight rU p eps'_i
     float2 tr;               // sum of weight rU r
 };
@@ -286,21 +287,27 @@ __device__ __forceinline__ void eval_chunk(const ShearConst &c, const Chunk &ch,
     for (int h = 0; h < 2; ++h) add_pair(L, ew[h], e1[h], e2[h], ru[h], pp[h], rr[h], qq[h]);
 }
 
-// A lane's NQ quads of chunk `chunk` of a galaxy, of which nq exist.
-template <int FAMILY, bool HAS_B, int NQ, class Quad>
-__device__ __forceinline__ void eval_lane_chunk(const ShearConst &c, int chunk, int nq, Quad quad, Lse &L)
+// Four samples of a galaxy after its first four, against the reference as it stands: no test and
+// no branch, so that consecutive quads and points overlap.  eval_chunk's rescaling (a log
+// weight above the reference by more than 32) is left to the galaxy's end, where the largest log
+// weight seen tells whether it was ever due (lse_jumped) and the lane's samples are then taken
+// again by eval_chunk (replay_lane).  Posterior samples of one galaxy span far less.
+template <int FAMILY, bool HAS_B>
+__device__ __forceinline__ void eval_quad(const ShearConst &c, const Chunk &ch, Lse &L)
 {
-    if (chunk == 0) {
-        if (nq > 0) eval_first<FAMILY, HAS_B>(c, quad(0), L);
+    const float2 nm = f2(-L.m);
+    const float2 e1[2] = {make_float2(ch.e1.x, ch.e1.y), make_float2(ch.e1.z, ch.e1.w)};
+    const float2 e2[2] = {make_float2(ch.e2.x, ch.e2.y), make_float2(ch.e2.z, ch.e2.w)};
+    const float2 bb[2] = {make_float2(ch.b.x, ch.b.y), make_float2(ch.b.z, ch.b.w)};
 #pragma unroll
-        for (int h = 1; h < NQ; ++h)
-            if (h < nq) eval_chunk<FAMILY, HAS_B>(c, quad(h), L);
-    } else {
-#pragma unroll
-        for (int h = 0; h < NQ; ++h)
-            if (h < nq) eval_chunk<FAMILY, HAS_B>(c, quad(h), L);
+    for (int h = 0; h < 2; ++h) {
+        float2 x, fw, ru, pp, rr, qq;
+        pair_terms<FAMILY, HAS_B>(c, e1[h], e2[h], bb[h], x, fw, ru, pp, rr, qq);
+        L.mx = fmaxf(L.mx, fmaxf(x.x, x.y));
+        add_pair(L, pair_weight(x, nm, fw), e1[h], e2[h], ru, pp, rr, qq);
     }
 }
+__device__ __forceinline__ bool lse_jumped(const Lse &L) { return L.mx - L.m > 32.0f; }
 
 // Merge the lanes of a galaxy's group and add the galaxy's terms, times the galaxy's weight
 // w[n] (1 when w is NULL; a zero weight drops the galaxy), to the accumulators of the
@@ -355,8 +362,14 @@ __device__ __forceinline__ void finish_galaxy(const Lse &L, float g1, float g2, 
 __device__ __forceinline__ void lse_reset(Lse &L)
 {
     L.m = -1e30f;
+    L.mx = -INFINITY;
     L.sw = L.t1 = L.t2 = L.tq = L.tr = f2(0.f);
 }
+
+// One lane's samples of galaxy n (tile kernels' assignment: 12 of every 48) by eval_chunk, from
+// the start.
+template <int FAMILY, bool HAS_B>
+__device__ __noinline__ Lse replay_lane(const ShearLaunch &s, const ShearConst &c, long long n, int sub);
 
 // Block reduction of the lanes' FP64 accumulators (quantity = lane of the group of G, the
 // first four) into this block's partials.
@@ -454,7 +467,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
     for (;;) {
         uint32_t ok;
         asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+                        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+
             "selp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(ok)
             : "r"(bar), "r"(parity), "r"(20000u)
@@ -603,6 +617,15 @@ __global__ void __launch_bounds__(kShearThreads, kTmaBlocks)
     double acc = 0.0;
     Lse L;
     lse_reset(L);
+    // With b the pass waits for memory (2 CTAs per SM, 570 us at 10^6 x 300; 612 us with
+    // eval_chunk at 3); without, it is eval_chunk's fewer registers that pay (446 us at 3 CTAs,
+    // 461 us with eval_quad at 3, 476 us at 2).
+    auto one_quad = [&](const Chunk &ch) {
+        if constexpr (HAS_B)
+            eval_quad<FAMILY, HAS_B>(c, ch, L);
+        else
+            eval_chunk<FAMILY, HAS_B>(c, ch, L);
+    };
     bool failed = false;
     int chunk = 0;
     long long tile = blockIdx.x;
@@ -614,12 +637,25 @@ __global__ void __launch_bounds__(kShearThreads, kTmaBlocks)
         }
         const long long n = tile * kTileG + gl;
         if (n < s.n_gal) {
-            eval_lane_chunk<FAMILY, HAS_B, kQuads>(c, chunk, tma_quads(K, chunk),
-                                                   [&](int h) { return tma_quad(R, item, h); }, L);
+            const int nq = tma_quads(K, chunk);
+            if (chunk == 0) {
+                if (nq > 0) eval_first<FAMILY, HAS_B>(c, tma_quad(R, item, 0), L);
+            } else if (nq > 0) {
+                one_quad(tma_quad(R, item, 0));
+            }
+#pragma unroll
+            for (int h = 1; h < kQuads; ++h)
+                if (h < nq) one_quad(tma_quad(R, item, h));
         }
         R.release(item);
         if (++chunk == R.cpg) {
-            if (n < s.n_gal) finish_galaxy<kAGroup>(L, s.g1, s.g2, gmask, sub, s.w, n, acc);
+            if (n < s.n_gal) {
+                if constexpr (HAS_B) {
+                    if (lse_jumped(L)) L = replay_lane<FAMILY, HAS_B>(s, s.c, n, sub);
+                    __syncwarp(gmask);
+                }
+                finish_galaxy<kAGroup>(L, s.g1, s.g2, gmask, sub, s.w, n, acc);
+            }
             lse_reset(L);
             chunk = 0;
             tile += gridDim.x;
@@ -628,6 +664,21 @@ __global__ void __launch_bounds__(kShearThreads, kTmaBlocks)
     if (failed || (tid == 0 && !R.p_ok)) s_fail = 1;
     R.drain();                                  // (begins with a barrier)
     block_partials<kAGroup>(s, s_fail ? NAN : acc);
+}
+
+template <int FAMILY, bool HAS_B>
+__device__ __noinline__ Lse replay_lane(const ShearLaunch &s, const ShearConst &c, long long n, int sub)
+{
+    Lse L;
+    lse_reset(L);
+    const long long base = n * (long long)s.K;
+    for (int k0 = kChunk * sub; k0 < s.K; k0 += kTileK)
+        for (int k = k0; k < k0 + kChunk && k < s.K; k += 4) {
+            Chunk ch;
+            load_chunk<HAS_B>(s, base, k, s.K, ch);
+            eval_chunk<FAMILY, HAS_B>(c, ch, L);
+        }
+    return L;
 }
 
 // The tensor-map encoder of the driver, looked up once through the runtime
@@ -1040,18 +1091,25 @@ int resident_grid(GridCache &cache, K kernel, size_t smem)
     return sms * nb;
 }
 
-GridCache g_grid_one, g_grid_full, g_grid_multi;
+GridCache g_grid_one, g_grid_b, g_grid_full, g_grid_multi;
 
 }  // namespace
 
-int shear_grid_blocks()
+static int shear_grid_resident(bool has_b)
 {
-    return resident_grid(g_grid_one, shear_kernel_tma<BS_EPRIOR_TRUNC_GAUSS, false>, tma_smem_bytes(false));
+    return has_b ? resident_grid(g_grid_b, shear_kernel_tma<BS_EPRIOR_TRUNC_GAUSS, true>, tma_smem_bytes(true))
+                 : resident_grid(g_grid_one, shear_kernel_tma<BS_EPRIOR_TRUNC_GAUSS, false>, tma_smem_bytes(false));
 }
 
-int shear_grid_for(long long n_gal)
+int shear_grid_blocks()
 {
-    const int full = shear_grid_blocks();
+    const int a = shear_grid_resident(false), b = shear_grid_resident(true);
+    return a > b ? a : b;
+}
+
+int shear_grid_for(long long n_gal, bool has_b)
+{
+    const int full = shear_grid_resident(has_b);
     const long long want = (n_gal + 31) / 32;
     return want < 1 ? 1 : want < full ? (int)want : full;
 }
@@ -1101,7 +1159,8 @@ int shear_multi_grid_blocks() { return resident_grid(g_grid_multi, shear_kernel_
 // state; a galaxy's 4 lanes put their FP64 totals per point in their own shared-memory
 // slot, summed over the block in a fixed order.  On a wait that gives up, the block's
 // partials are NaN.
-template <int FAMILY>
+// FULL: all kMultiPoints points are asked for (no test between them).
+template <int FAMILY, bool FULL>
 __global__ void __launch_bounds__(kShearThreads, 2)
     shear_kernel_tma_multi(const __grid_constant__ ShearMultiLaunch m, const __grid_constant__ CUtensorMap m1,
                            const __grid_constant__ CUtensorMap m2)
@@ -1144,9 +1203,15 @@ __global__ void __launch_bounds__(kShearThreads, 2)
             for (int h = 0; h < kQuads; ++h) {
                 if (h < nq) {
                     const Chunk ch = tma_quad(R, item, h);
+                    if (h == 0 && chunk == 0) {
 #pragma unroll
-                    for (int p = 0; p < NP; ++p)
-                        if (p < m.n_points) eval_chunk<FAMILY, false>(m.c[p], ch, L[p]);
+                        for (int p = 0; p < NP; ++p)
+                            if (FULL || p < m.n_points) eval_first<FAMILY, false>(m.c[p], ch, L[p]);
+                    } else {
+#pragma unroll
+                        for (int p = 0; p < NP; ++p)
+                            if (FULL || p < m.n_points) eval_quad<FAMILY, false>(m.c[p], ch, L[p]);
+                    }
                 }
             }
         }
@@ -1157,6 +1222,8 @@ __global__ void __launch_bounds__(kShearThreads, 2)
                 for (int p = 0; p < NP; ++p) {
                     if (p < m.n_points) {
                         double t = 0.0;
+                        if (lse_jumped(L[p])) L[p] = replay_lane<FAMILY, false>(s, m.c[p], n, sub);
+                        __syncwarp(gmask);
                         finish_galaxy<kAGroup>(L[p], m.g1[p], m.g2[p], gmask, sub, s.w, n, t);
                         acc[gl][p][sub] += t;
                     }
@@ -1186,8 +1253,11 @@ cudaError_t launch_shear_multi(const ShearMultiLaunch &m, int grid, cudaStream_t
                      ((reinterpret_cast<uintptr_t>(s.e2) & 15) == 0) && s.b == nullptr;
     CUtensorMap m1, m2;
     if (vec && make_sample_map(m1, s.e1, s.n_gal, s.K) && make_sample_map(m2, s.e2, s.n_gal, s.K)) {
-        auto k = s.family == BS_EPRIOR_BA14 ? shear_kernel_tma_multi<BS_EPRIOR_BA14>
-                                            : shear_kernel_tma_multi<BS_EPRIOR_TRUNC_GAUSS>;
+        const bool full = m.n_points == kMultiPoints;
+        auto k = s.family == BS_EPRIOR_BA14
+                     ? (full ? shear_kernel_tma_multi<BS_EPRIOR_BA14, true> : shear_kernel_tma_multi<BS_EPRIOR_BA14, false>)
+                     : (full ? shear_kernel_tma_multi<BS_EPRIOR_TRUNC_GAUSS, true>
+                             : shear_kernel_tma_multi<BS_EPRIOR_TRUNC_GAUSS, false>);
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)tma_smem_bytes(false));
         if (e != cudaSuccess) return e;
