@@ -41,7 +41,8 @@ __device__ void pix_tc_setup(const FitParams &P, const GalCtx &gc, const SmemVie
         tc::st8(tl + (lo ? tc::kColAFlo : tc::kColAF) + k0, v);
     }
     // the complex-to-real constant: rows ix < 64, K (re, u | im, u):
-    // (w_u / N^2) (cos, -sin)(2 pi u (ix - c) / N); rows 64.. zero
+    // (w_u / N^2) (cos, -sin)(2 pi u (ix - c) / N); rows 64 + ix again, so that the model image
+    // comes out in both halves of the accumulator's lanes
     const float wn = 1.0f / ((float)N * (float)N);
     for (int k0 = 0; k0 < 64; k0 += 8) {
         float v[8];
@@ -49,8 +50,8 @@ __device__ void pix_tc_setup(const FitParams &P, const GalCtx &gc, const SmemVie
         for (int j = 0; j < 8; ++j) {
             const int k = k0 + j, q = k >> 5, u = k & 31;
             float co = 0.f, sn = 0.f;
-            if (row < N && u < H) {
-                int m = (u * (row - c)) % N;
+            if (a < N && u < H) {
+                int m = (u * (a - c)) % N;
                 if (m < 0) m += N;
                 sincospif(2.0f * (float)m / (float)N, &sn, &co);
                 const float wu = u ? 2.0f * wn : wn;
@@ -79,17 +80,21 @@ __device__ void pix_tc_setup(const FitParams &P, const GalCtx &gc, const SmemVie
 // commits, everyone waits for the given parity).  K runs over n_q halves of nk steps
 // of 8: step (q, k) reads A at TMEM column a + q a_q + 8 k (its low part a_lo columns
 // further) and B at b + q b_q + 288 k bytes (the data operand: leading offset 144 B,
-// row groups sbo_b apart).  Returns false (for every thread) if the wait gave up; the
-// CTA is then aborted with that parity pending.
+// row groups sbo_b apart).  `failed` carries whether this thread's last wait gave up: the barrier
+// before the issue shares it, and returns false for every thread (nothing issued, the CTA
+// aborted with the previous product's parity pending).
 struct TcGemm {
     uint32_t a, a_q, a_lo, b, b_q, sbo_b, id;
     int n_q, nk;
 };
-__device__ __forceinline__ bool tc_run(const PixTc &px, const TcGemm &G, uint32_t parity)
+__device__ __forceinline__ bool tc_run(const PixTc &px, const TcGemm &G, uint32_t parity, bool &failed)
 {
     tc::fence_async_smem();
     tc::fence_before();
-    __syncthreads();
+    if (__syncthreads_or(failed)) {
+        if (threadIdx.x == 0) *px.abort = 2 + (int)(parity ^ 1u);
+        return false;
+    }
     const uint32_t bar = tc::saddr(px.bar);
     if (threadIdx.x == 0) {
         tc::fence_after();
@@ -112,12 +117,7 @@ __device__ __forceinline__ bool tc_run(const PixTc &px, const TcGemm &G, uint32_
         }
         tc::commit(bar);
     }
-    const bool ok = tc::wait_parity(bar, parity);
-    const bool bad = __syncthreads_or(!ok);
-    if (bad) {
-        if (threadIdx.x == 0) *px.abort = 2 + (int)parity;
-        return false;
-    }
+    failed = !tc::wait_parity(bar, parity);
     tc::fence_after();
     return true;
 }
@@ -188,23 +188,15 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
     const float be = r02 * (1.0f + E - 2.0f * e1) * Pq;
     const float ga = r02 * 4.0f * e2 * Pq;
     const float sqrt2 = 1.41421356237309515f;
-    float2 *xs = px.xs + 32 * grp, *ys = px.ys + 64 * grp;
-    if (tg < 32) {
-        float sx = 0.f, cx = 0.f;
-        if (tg < H) sincospi_sfu(-2.0f * th[4] * (float)tg * gc.invN, &sx, &cx);
-        xs[tg] = make_float2(cx, sx);
-    } else if (tg < 96) {
-        const int vi = tg - 32;
-        float sy = 0.f, cy = 0.f;
-        if (vi < N) sincospi_sfu(-2.0f * th[5] * (float)(vi - c) * gc.invN, &sy, &cy);
-        ys[vi] = make_float2(F * cy, F * sy);
-    }
-    __syncthreads();
     float *bh = px.bop, *bl = px.bop + tc::kBopFloats;
     constexpr int kLb = tc::kLboB / 4;
+    const int ks = (N + 7) >> 3;          // k-steps of 8 covering the side
+    const int n8 = 8 * ks;                // columns or rows of one chain over iy (or ix)
+    const int h8 = 8 * ((H + 7) >> 3);    // and over u
     // (a) the model's half spectrum Mt into the chain's table D slots, and M = Mt /
-    // scale_u as the operand of (1): rows (chain, u < 32), K (re, vi | im, vi); thread
-    // tg of the group takes column vi = tg mod 64 and the rows u = tg / 64 + 2 i
+    // scale_u as the operand of (1): rows (chain, u < h8), K (re, vi | im, vi); thread
+    // tg of the group takes column vi = tg mod 64 and the rows u = tg / 64 + 2 i.  The row
+    // phases X(u) are formed a lane each and passed by shuffles
     {
         const int vi = tg & 63, u0 = tg >> 6;
         const bool col = vi < N;
@@ -212,11 +204,14 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
         if (col) slot_offsets(npad, vi >> 5, vi & 31, ox, oy, ot);
         const float ky = (float)(vi - c) * gc.dk;
         const float cst = fmaf(be * ky, ky, 1.0f), gky = ga * ky;
-        const float2 Y = ys[vi];
+        float Xs, Xc, sy, cy;
+        sincospi_sfu(-2.0f * th[4] * (float)lane * gc.invN, &Xs, &Xc);
+        sincospi_sfu(-2.0f * th[5] * (float)(vi - c) * gc.invN, &sy, &cy);
+        const float2 Y = make_float2(F * cy, F * sy);
         const float sN = (float)N, sN2 = (float)N * 0.70710678118654752f;
 #pragma unroll 4
-        for (int i = 0; i < 16; ++i) {
-            const int u = u0 + 2 * i;
+        for (int u = u0; u < h8; u += 2) {
+            const float2 X = make_float2(__shfl_sync(BS_FULL_MASK, Xc, u), __shfl_sync(BS_FULL_MASK, Xs, u));
             float Mr = 0.f, Mi = 0.f;
             if (col && u < H) {
                 float *row = tab + (size_t)u * rowf;
@@ -224,7 +219,6 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
                 const float s = fmaf(fmaf(al, kx, gky), kx, cst);
                 const float rs = rsqrtf(s);
                 const float A = row[ot] * rs * rs * rs;
-                const float2 X = xs[u];
                 const float mr = A * (X.x * Y.x - X.y * Y.y), mi = A * (X.x * Y.y + X.y * Y.x);
                 row[ox] = mr;
                 row[oy] = mi;
@@ -232,98 +226,125 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
                 Mr = mr * inv_scale;
                 Mi = mi * inv_scale;
             }
-            tc::split_store(bh, bl, tc::op_index(32 * grp + u, vi, 128, kLb), Mr);
-            tc::split_store(bh, bl, tc::op_index(32 * grp + u, 64 + vi, 128, kLb), Mi);
+            tc::split_store(bh, bl, tc::op_index(h8 * grp + u, vi, 128, kLb), Mr);
+            tc::split_store(bh, bl, tc::op_index(h8 * grp + u, 64 + vi, 128, kLb), Mi);
         }
     }
     const uint32_t bop = tc::saddr(px.bop);
-    const int ks = (N + 7) >> 3;   // k-steps of 8 covering the side
     const uint32_t tl = *px.tmem + ((uint32_t)(32 * (warp & 3)) << 16);
     constexpr uint32_t aflo = tc::kColAFlo - tc::kColAF, a2lo = tc::kColA2lo - tc::kColA2;
+    bool failed = false;
     // (1) G = M E for both chains: rows (re, iy | im, iy), columns (chain, u)
-    if (!tc_run(px, TcGemm{tc::kColAF, 64u, aflo, bop, 16u * 144, 32u * 144, tc::idesc(128, 64), 2, ks}, 0))
+    if (!tc_run(px, TcGemm{tc::kColAF, 64u, aflo, bop, 16u * 144, 32u * 144, tc::idesc(128, 2 * h8), 2, ks}, 0, failed))
         return pix_nan(g);
     // (1) -> operand of (2): row (chain, iy), K (re, u | im, u), G as it is (the weights
-    // are in the constant); this thread's lane (p, iy), its chain's 32 columns
+    // are in the constant); this thread's lane (p, iy), its chain's h8 columns
     {
         float v[32];
-        tc::ld32(tl + 32 * grp, v);
+        tc::ld8n(tl + h8 * grp, h8 >> 3, v);
         const int p = L >> 6, iy = L & 63;
-        const int e0 = tc::op_index(64 * grp + iy, p * 32, 64, kLb);
+        if (iy < n8) {
+            const int e0 = tc::op_index(n8 * grp + iy, p * 32, 64, kLb);
 #pragma unroll
-        for (int m = 0; m < 8; ++m)
-            tc::split_store4(bh, bl, e0 + m * kLb, v[4 * m], v[4 * m + 1], v[4 * m + 2], v[4 * m + 3]);
+            for (int m = 0; m < 8; ++m)
+                if (4 * m < h8)
+                    tc::split_store4(bh, bl, e0 + m * kLb, v[4 * m], v[4 * m + 1], v[4 * m + 2], v[4 * m + 3]);
+        }
     }
-    // (2) m = W G: rows ix, columns (chain, iy)
-    if (!tc_run(px, TcGemm{tc::kColA2, 32u, a2lo, bop, 8u * 144, 16u * 144, tc::idesc(128, 128), 2,
+    // (2) m = W G: rows ix (twice), columns (chain, iy)
+    if (!tc_run(px, TcGemm{tc::kColA2, 32u, a2lo, bop, 8u * 144, 16u * 144, tc::idesc(128, 2 * n8), 2,
                            (H + 7) >> 3},
-                1))
+                1, failed))
         return pix_nan(g);
-    // the residual, chi^2 (compensated FP32 per thread, FP64 across threads) and the
-    // operand of (3): rows (chain, iy), K ix; lanes ix < 64 of the group's warps 0 and
-    // 1, the chain's 64 columns iy
-    double chi = 0.0;
-    if ((warp & 3) < 2) {
-        const int ix = L;
+    // the residual and the operand of (3): rows (chain, iy), K ix; the group's warps 0 and 1
+    // (lanes ix) take the first 32 rows iy, warps 2 and 3 (lanes 64 + ix) the others, 16 at a
+    // time.  chi^2 (compensated FP32 per thread over iy in order, FP64 across threads) stays with
+    // warps 0 and 1, which read the other rows again for it
+    {
+        const int ix = L & 63, half = L >> 6;
         float c_hi = 0.f, c_lo = 0.f;
+        auto chi_term = [&](float t) {
+            float t_hi, t_lo;
+            two_sum(c_hi, t, t_hi, t_lo);
+            c_hi = t_hi;
+            c_lo += t_lo;
+        };
         const int eb = (ix >> 2) * kLb + (ix & 3);
+        const bool ll = want_ll && half == 0;
+#pragma unroll 1
+        for (int y0 = 32 * half; y0 < 32 * half + 32 && y0 < n8; y0 += 16) {
+            float m[16];
+            tc::ld16(tl + n8 * grp + y0, m);
+            float p[16];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float m[32];
-            tc::ld32(tl + 64 * grp + 32 * h, m);
-#pragma unroll
-            for (int t = 0; t < 32; ++t) {
-                const int iy = 32 * h + t;
+            for (int t = 0; t < 16; ++t) {
+                const int iy = y0 + t;
                 float r = 0.f;
+                p[t] = 0.f;
                 if (ix < N && iy < N) {
                     const int e = iy * N + ix;
                     const float res = px.dimg[e] - m[t];
                     r = px.wimg[e] * res;
-                    if (want_ll) {
-                        float t_hi, t_lo;
-                        two_sum(c_hi, r * res, t_hi, t_lo);
-                        c_hi = t_hi;
-                        c_lo += t_lo;
-                    }
+                    p[t] = r * res;
                 }
-                const int rr = 64 * grp + iy;
-                tc::split_store(bh, bl, eb + (rr >> 3) * 16 * kLb + ((rr & 7) << 2), r);
+                const int rr = n8 * grp + iy;
+                if (iy < n8) tc::split_store(bh, bl, eb + (rr >> 3) * 16 * kLb + ((rr & 7) << 2), r);
+            }
+            if (ll) {
+#pragma unroll
+                for (int t = 0; t < 16; ++t)
+                    if (ix < N && y0 + t < N) chi_term(p[t]);
             }
         }
-        chi = (double)c_hi + (double)c_lo;
-    }
-    if (want_ll) {
-        const double cw = warp_sum_d(chi);
-        if (lane == 0) px.chi[warp] = cw;
+        if (ll) {
+#pragma unroll 1
+            for (int y0 = 32; y0 < n8; y0 += 16) {
+                float m[16];
+                tc::ld16(tl + n8 * grp + y0, m);
+#pragma unroll
+                for (int t = 0; t < 16; ++t) {
+                    if (ix < N && y0 + t < N) {
+                        const int e = (y0 + t) * N + ix;
+                        const float res = px.dimg[e] - m[t];
+                        chi_term(px.wimg[e] * res * res);
+                    }
+                }
+            }
+        }
+        if (want_ll) {
+            const double cw = warp_sum_d((double)c_hi + (double)c_lo);
+            if (lane == 0) px.chi[warp] = cw;
+        }
     }
     // (3) conj Q = [C; S] r: rows (re, a | im, a), columns (chain, iy)
-    if (!tc_run(px, TcGemm{tc::kColAF, 0u, aflo, bop, 0u, 16u * 144, tc::idesc(128, 128), 1, ks}, 0))
+    if (!tc_run(px, TcGemm{tc::kColAF, 0u, aflo, bop, 0u, 16u * 144, tc::idesc(128, 2 * n8), 1, ks}, 0, failed))
         return pix_nan(g);
-    // (3) -> operand of (4): row (chain, u = a - c < 32), K (re, iy | im, iy); this
-    // thread's lane (q, a), its chain's 64 columns iy
+    // (3) -> operand of (4): row (chain, u = a - c < h8), K (re, iy | im, iy); this
+    // thread's lane (q, a), its chain's n8 columns iy
     {
         const int q = L >> 6, u = (L & 63) - c;
+#pragma unroll 1
+        for (int y0 = 0; y0 < n8; y0 += 16) {
+            float v[16];
+            tc::ld16(tl + n8 * grp + y0, v);
+            if (u >= 0 && u < h8) {
+                const int e0 = tc::op_index(h8 * grp + u, q * 64 + y0, 128, kLb);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float v[32];
-            tc::ld32(tl + 64 * grp + 32 * h, v);
-            if (u >= 0 && u < 32) {
-                const int e0 = tc::op_index(32 * grp + u, q * 64 + 32 * h, 128, kLb);
-#pragma unroll
-                for (int m = 0; m < 8; ++m)
-                    tc::split_store4(bh, bl, e0 + m * kLb, v[4 * m], v[4 * m + 1], v[4 * m + 2], v[4 * m + 3]);
+                for (int m = 0; m < 4; ++m)
+                    if (y0 + 4 * m < n8)
+                        tc::split_store4(bh, bl, e0 + m * kLb, v[4 * m], v[4 * m + 1], v[4 * m + 2], v[4 * m + 3]);
             }
         }
     }
     // (4) conj R = E conj Q: rows (re, vi | im, vi), columns (chain, u)
-    if (!tc_run(px, TcGemm{tc::kColAF, 64u, aflo, bop, 16u * 144, 32u * 144, tc::idesc(128, 64), 2, ks}, 1))
+    if (!tc_run(px, TcGemm{tc::kColAF, 64u, aflo, bop, 16u * 144, 32u * 144, tc::idesc(128, 2 * h8), 2, ks}, 1, failed))
         return pix_nan(g);
     // D' = Mt + scale_u R in the chain's table D slots; this thread's lane (p, vi), its
-    // chain's 32 columns u
+    // chain's columns u
     {
         const int p = L >> 6, vi = L & 63;
         float v[32];
-        tc::ld32(tl + 32 * grp, v);
+        tc::ld8n(tl + h8 * grp, h8 >> 3, v);
         if (vi < N) {
             int ox, oy, ot;
             slot_offsets(npad, vi >> 5, vi & 31, ox, oy, ot);
@@ -338,7 +359,10 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
             }
         }
     }
-    __syncthreads();
+    if (__syncthreads_or(failed)) {
+        if (threadIdx.x == 0) *px.abort = 2 + 1;
+        return pix_nan(g);
+    }
     // the gradient from the half-plane pass on the chain's effective spectrum, its rows
     // over the group's four warps
     pix_grad<NC>(P, gc, tab, sm.kxr, px, xph, vcol, th, g);

@@ -131,22 +131,37 @@ __device__ __forceinline__ bool wait_parity(uint32_t bar, uint32_t parity)
     }
 }
 
-// 32 consecutive TMEM columns of this thread's lane (the warp's 32 lanes).
-__device__ __forceinline__ void ld32(uint32_t taddr, float (&v)[32])
+// n8 (at most 4) times 8 consecutive TMEM columns of this thread's lane (the warp's 32 lanes).
+__device__ __forceinline__ void ld8n(uint32_t taddr, int n8, float (&v)[32])
 {
     uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) r[8 * i + j] = 0u;
+        if (i < n8)
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                         : "=r"(r[8 * i]), "=r"(r[8 * i + 1]), "=r"(r[8 * i + 2]), "=r"(r[8 * i + 3]),
+                           "=r"(r[8 * i + 4]), "=r"(r[8 * i + 5]), "=r"(r[8 * i + 6]), "=r"(r[8 * i + 7])
+                         : "r"(taddr + 8 * i));
+    }
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// 16 consecutive TMEM columns of this thread's lane.
+__device__ __forceinline__ void ld16(uint32_t taddr, float (&v)[16])
+{
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // Four consecutive K-elements (one core-matrix row) as high and low TF32 parts.
@@ -200,8 +215,6 @@ struct PixTc {
     uint32_t *tmem;   // TMEM base of the CTA (512 columns)
     int *abort;       // 2 + the pending parity once a wait gave up, else 0
     int *done;        // [2] a chain group has no more evaluations
-    float2 *xs;       // [2][32] per chain: exp(-2 pi i u dx / N)
-    float2 *ys;       // [2][64] per chain: F exp(-2 pi i v dy / N), v = vi - c
     float *gsum;      // [2][4][6] per chain and warp of its group: the six gradient sums
     float *bop;       // [2][kBopFloats] the data operand of the current transform, high then low
     float *tab1;      // [h_max][3 npad] the second chain's table (the first's is the staged one)
@@ -212,11 +225,10 @@ struct PixTc {
 __host__ __device__ __forceinline__ int pix_tc_img_floats(int max_side) { return (max_side * max_side + 3) & ~3; }
 
 // Floats of the region: 16 (chi) + 2 (barrier) + 1 (TMEM address) + 1 (abort) + 2
-// (done) + 2 (pad) + 128 (xs) + 256 (ys) + 48 (gradient sums) + operand + table + two
-// images.
+// (done) + 2 (pad) + 48 (gradient sums) + operand + table + two images.
 __host__ __device__ __forceinline__ size_t pix_tc_bytes(int max_side, int h_max, int npad)
 {
-    return ((size_t)456 + 2 * tc::kBopFloats + (size_t)h_max * 3 * npad + 2 * (size_t)pix_tc_img_floats(max_side)) *
+    return ((size_t)72 + 2 * tc::kBopFloats + (size_t)h_max * 3 * npad + 2 * (size_t)pix_tc_img_floats(max_side)) *
            sizeof(float);
 }
 
@@ -230,10 +242,8 @@ __device__ __forceinline__ PixTc pix_tc_view(float2 *kxr, int h_max, int npad, i
     v.tmem = reinterpret_cast<uint32_t *>(base + 18);
     v.abort = reinterpret_cast<int *>(base + 19);
     v.done = reinterpret_cast<int *>(base + 20);
-    v.xs = reinterpret_cast<float2 *>(base + 24);
-    v.ys = reinterpret_cast<float2 *>(base + 152);
-    v.gsum = base + 408;
-    v.bop = base + 456;
+    v.gsum = base + 24;
+    v.bop = base + 72;
     v.tab1 = v.bop + 2 * tc::kBopFloats;
     v.dimg = v.tab1 + (size_t)h_max * 3 * npad;
     v.wimg = v.dimg + pix_tc_img_floats(max_side);
