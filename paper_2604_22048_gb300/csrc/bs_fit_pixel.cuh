@@ -134,16 +134,15 @@ __device__ __forceinline__ double pix_nan(float g[6])
 // the group sums the terms of its rows u in [r j, r (j + 1)), r even (the pass reads
 // rows in pairs); the four warp sums meet in shared memory, where every thread of the
 // group adds them in warp order and forms the gradient (the sums and the gradient of
-// eval_logpost, exponential profile, no chi^2).
+// eval_logpost, exponential profile, no chi^2).  m: the model's shape at th.
 template <int NC>
-__device__ void pix_grad(const FitParams &P, const GalCtx &gc, const float *tab, const float2 *kxr, const PixTc &px,
+__device__ __forceinline__ void pix_grad(const FitParams &P, const GalCtx &gc, const Shape &m, const float *tab, const float2 *kxr, const PixTc &px,
                          float4 *xph, const float vcol[NC], const float th[6], float g[6])
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int grp = warp >> 2, wj = warp & 3;
     const int per = 2 * ((gc.H + 7) >> 3);
     const int u0 = min(gc.H, wj * per), u1 = min(gc.H, u0 + per);
-    const Shape m = model_shape<0>(P, th);
     float sums[6], chi_hi = 0.f, chi_lo = 0.f;
     spectral_sums<NC, false, 0>(P, gc, m, tab, kxr, xph, vcol, th, u0, u1, sums, chi_hi, chi_lo);
     float *gs = px.gsum + grp * 24;
@@ -171,22 +170,15 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
     const int L = 32 * (warp & 3) + lane;             // this thread's TMEM lane
     const int tg = tid & 127;                         // thread within the group
     const PixTc px = pix_tc_view(sm.kxr, P.h_max, P.npad, P.max_side);
-    const int N = gc.N, H = gc.H, c = gc.c, npad = P.npad;
-    const int rowf = row_floats(npad);
+    const int N = gc.N, H = gc.H, c = gc.c;
+    constexpr int npad = 32 * NC, rowf = 96 * NC;
     float *tab = grp ? px.tab1 : sm.tab;
+    const Shape ms = model_shape<0>(P, th);
+    const float F = ms.F, E = ms.E, al = ms.al, be = ms.be, ga = ms.ga;
     __syncthreads();   // the previous evaluation's readers of the tables and buffers are done
     if (all_done) *all_done = px.done[0] && px.done[1];
     if (px.done[0] && px.done[1]) return 0.0;
     if (*px.abort) return pix_nan(g);
-    const float F = exp10f(th[0]);
-    const float r0 = exp10f(th[1]) * (1.0f / kHlrOverR0);
-    const float r02 = r0 * r0;
-    const float e1 = th[2], e2 = th[3];
-    const float E = e1 * e1 + e2 * e2;
-    const float Pq = 1.0f / (1.0f - E);
-    const float al = r02 * (1.0f + E + 2.0f * e1) * Pq;
-    const float be = r02 * (1.0f + E - 2.0f * e1) * Pq;
-    const float ga = r02 * 4.0f * e2 * Pq;
     const float sqrt2 = 1.41421356237309515f;
     float *bh = px.bop, *bl = px.bop + tc::kBopFloats;
     constexpr int kLb = tc::kLboB / 4;
@@ -209,25 +201,32 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
         sincospi_sfu(-2.0f * th[5] * (float)(vi - c) * gc.invN, &sy, &cy);
         const float2 Y = make_float2(F * cy, F * sy);
         const float sN = (float)N, sN2 = (float)N * 0.70710678118654752f;
-#pragma unroll 4
-        for (int u = u0; u < h8; u += 2) {
-            const float2 X = make_float2(__shfl_sync(BS_FULL_MASK, Xc, u), __shfl_sync(BS_FULL_MASK, Xs, u));
-            float Mr = 0.f, Mi = 0.f;
-            if (col && u < H) {
-                float *row = tab + (size_t)u * rowf;
-                const float kx = sm.kxr[u].x;
-                const float s = fmaf(fmaf(al, kx, gky), kx, cst);
-                const float rs = rsqrtf(s);
-                const float A = row[ot] * rs * rs * rs;
-                const float mr = A * (X.x * Y.x - X.y * Y.y), mi = A * (X.x * Y.y + X.y * Y.x);
-                row[ox] = mr;
-                row[oy] = mi;
-                const float inv_scale = u == 0 ? sN : sN2;
-                Mr = mr * inv_scale;
-                Mi = mi * inv_scale;
+        // operand element (h8 grp + u, vi) of eight-row group ug, u = ug + u0 + 2 j
+        const int eo = (vi >> 2) * kLb + (vi & 3) + u0 * 4;
+#pragma unroll 1
+        for (int ug = 0; ug < h8; ug += 8) {
+            const int e0 = eo + ((h8 * grp + ug) >> 3) * 32 * kLb;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int u = ug + u0 + 2 * j;
+                const float2 X = make_float2(__shfl_sync(BS_FULL_MASK, Xc, u), __shfl_sync(BS_FULL_MASK, Xs, u));
+                float Mr = 0.f, Mi = 0.f;
+                if (col && u < H) {
+                    float *row = tab + u * rowf;
+                    const float kx = sm.kxr[u].x;
+                    const float s = fmaf(fmaf(al, kx, gky), kx, cst);
+                    const float rs = rsqrtf(s);
+                    const float A = row[ot] * rs * rs * rs;
+                    const float mr = A * (X.x * Y.x - X.y * Y.y), mi = A * (X.x * Y.y + X.y * Y.x);
+                    row[ox] = mr;
+                    row[oy] = mi;
+                    const float inv_scale = u == 0 ? sN : sN2;
+                    Mr = mr * inv_scale;
+                    Mi = mi * inv_scale;
+                }
+                tc::split_store(bh, bl, e0 + 8 * j, Mr);
+                tc::split_store(bh, bl, e0 + 8 * j + 16 * kLb, Mi);   // K index 64 + vi
             }
-            tc::split_store(bh, bl, tc::op_index(h8 * grp + u, vi, 128, kLb), Mr);
-            tc::split_store(bh, bl, tc::op_index(h8 * grp + u, 64 + vi, 128, kLb), Mi);
         }
     }
     const uint32_t bop = tc::saddr(px.bop);
@@ -257,64 +256,47 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
                 1, failed))
         return pix_nan(g);
     // the residual and the operand of (3): rows (chain, iy), K ix; the group's warps 0 and 1
-    // (lanes ix) take the first 32 rows iy, warps 2 and 3 (lanes 64 + ix) the others, 16 at a
-    // time.  chi^2 (compensated FP32 per thread over iy in order, FP64 across threads) stays with
-    // warps 0 and 1, which read the other rows again for it
+    // (lanes ix) take the first half of the eight-row groups, warps 2 and 3 (lanes 64 + ix) the rest
     {
-        const int ix = L & 63, half = L >> 6;
-        float c_hi = 0.f, c_lo = 0.f;
-        auto chi_term = [&](float t) {
-            float t_hi, t_lo;
-            two_sum(c_hi, t, t_hi, t_lo);
-            c_hi = t_hi;
-            c_lo += t_lo;
-        };
-        const int eb = (ix >> 2) * kLb + (ix & 3);
-        const bool ll = want_ll && half == 0;
-#pragma unroll 1
-        for (int y0 = 32 * half; y0 < 32 * half + 32 && y0 < n8; y0 += 16) {
-            float m[16];
-            tc::ld16(tl + n8 * grp + y0, m);
-            float p[16];
+        const int ix = L & 63;
+        const int g0 = (L >> 6) ? (ks + 1) >> 1 : 0, ng = (L >> 6) ? ks >> 1 : (ks + 1) >> 1;
+        float m[32];
+        tc::ld8n(tl + n8 * grp + 8 * g0, ng, m);
+        const float *dp = px.dimg + 8 * g0 * N + ix, *wp = px.wimg + 8 * g0 * N + ix;
+        const int e0 = (ix >> 2) * kLb + (ix & 3) + (ks * grp + g0) * 16 * kLb;
 #pragma unroll
-            for (int t = 0; t < 16; ++t) {
-                const int iy = y0 + t;
+        for (int t = 0; t < 32; ++t) {
+            if (t < 8 * ng) {
                 float r = 0.f;
-                p[t] = 0.f;
-                if (ix < N && iy < N) {
-                    const int e = iy * N + ix;
-                    const float res = px.dimg[e] - m[t];
-                    r = px.wimg[e] * res;
-                    p[t] = r * res;
-                }
-                const int rr = n8 * grp + iy;
-                if (iy < n8) tc::split_store(bh, bl, eb + (rr >> 3) * 16 * kLb + ((rr & 7) << 2), r);
-            }
-            if (ll) {
-#pragma unroll
-                for (int t = 0; t < 16; ++t)
-                    if (ix < N && y0 + t < N) chi_term(p[t]);
+                if (ix < N && 8 * g0 + t < N) r = wp[t * N] * (dp[t * N] - m[t]);
+                tc::split_store(bh, bl, e0 + (t >> 3) * 16 * kLb + ((t & 7) << 2), r);
             }
         }
-        if (ll) {
+    }
+    // chi^2 (warps 0 and 1 of the group, all rows again: one evaluation of a trajectory):
+    // compensated FP32 per thread over iy in order, FP64 across threads
+    if (want_ll) {
+        float c_hi = 0.f, c_lo = 0.f;
+        if (L < 64) {
 #pragma unroll 1
-            for (int y0 = 32; y0 < n8; y0 += 16) {
-                float m[16];
-                tc::ld16(tl + n8 * grp + y0, m);
+            for (int g8 = 0; g8 < ks; ++g8) {
+                float m[32];
+                tc::ld8n(tl + n8 * grp + 8 * g8, 1, m);
 #pragma unroll
-                for (int t = 0; t < 16; ++t) {
-                    if (ix < N && y0 + t < N) {
-                        const int e = (y0 + t) * N + ix;
+                for (int t = 0; t < 8; ++t) {
+                    if (L < N && 8 * g8 + t < N) {
+                        const int e = (8 * g8 + t) * N + L;
                         const float res = px.dimg[e] - m[t];
-                        chi_term(px.wimg[e] * res * res);
+                        float t_hi, t_lo;
+                        two_sum(c_hi, px.wimg[e] * res * res, t_hi, t_lo);
+                        c_hi = t_hi;
+                        c_lo += t_lo;
                     }
                 }
             }
         }
-        if (want_ll) {
-            const double cw = warp_sum_d((double)c_hi + (double)c_lo);
-            if (lane == 0) px.chi[warp] = cw;
-        }
+        const double cw = warp_sum_d((double)c_hi + (double)c_lo);
+        if (lane == 0) px.chi[warp] = cw;
     }
     // (3) conj Q = [C; S] r: rows (re, a | im, a), columns (chain, iy)
     if (!tc_run(px, TcGemm{tc::kColAF, 0u, aflo, bop, 0u, 16u * 144, tc::idesc(128, 2 * n8), 1, ks}, 0, failed))
@@ -365,7 +347,7 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
     }
     // the gradient from the half-plane pass on the chain's effective spectrum, its rows
     // over the group's four warps
-    pix_grad<NC>(P, gc, tab, sm.kxr, px, xph, vcol, th, g);
+    pix_grad<NC>(P, gc, ms, tab, sm.kxr, px, xph, vcol, th, g);
     if (!want_ll) return 0.0;
     const double chi2 = px.chi[4 * grp] + px.chi[4 * grp + 1];
     const float lprior = P.prior_const - 0.5f * (th[4] * th[4] + th[5] * th[5]) * P.inv_sxy2 +

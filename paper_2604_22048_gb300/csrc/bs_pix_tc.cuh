@@ -112,22 +112,24 @@ __device__ __forceinline__ uint64_t now_ns()
     return t;
 }
 
-// Wait for the phase of the given parity to complete; false after kWaitNs.  Each
-// try_wait may suspend the warp in hardware for up to 20 us until the phase
-// completes; the limit is checked between tries.
+// Wait for the phase of the given parity to complete; false after kWaitNs.  The products
+// take about a microsecond and the waiting warps have nothing else to do, so the tries carry no
+// suspend-time hint; the clock for the limit is read only once a try has failed.
 __device__ __forceinline__ bool wait_parity(uint32_t bar, uint32_t parity)
 {
-    const uint64_t t0 = now_ns();
+    uint64_t t0 = 0;
     for (;;) {
         uint32_t ok;
         asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(ok)
-            : "r"(bar), "r"(parity), "r"(20000u)
+            : "r"(bar), "r"(parity)
             : "memory");
         if (ok) return true;
-        if (now_ns() - t0 > kWaitNs) return false;
+        const uint64_t t = now_ns();
+        if (t0 == 0) t0 = t;
+        if (t - t0 > kWaitNs) return false;
     }
 }
 
