@@ -380,8 +380,8 @@ __device__ void pix_drain(const FitParams &P, const GalCtx &gc, const SmemView &
 // instance PROF 4).  The gradient is the half-plane pass on the effective spectrum
 // D' = M + DFT(y) (scaled as the table).
 //
-// One CTA of 16 warps runs a galaxy's chains (at most 4), one evaluation of every chain at
-// a time: the first warp of each chain (its leader) runs the chain's logic, and all
+// One CTA of 16 warps runs a galaxy's chains (at most 4, or a share of them where there are SMs to
+// spare: dense_chains_per_cta), one evaluation of every chain at a time: the first warp of each chain (its leader) runs the chain's logic, and all
 // warps meet in dense_round, where one read of P serves every chain.  The transforms'
 // rows are split over the warps of the chain (16 / n_chains), the product's columns over
 // all 16 warps; every output is summed by one lane in a fixed order, so a chain's draws
@@ -461,7 +461,8 @@ __device__ void dense_setup(const FitParams &P, const GalCtx &gc, const SmemView
 
 // y = P r of every chain slot (all warps): the precision is symmetric, so y_a = sum_b
 // P[b][a] r_b, and a warp takes 32 columns a at a time, each row b of them one coalesced
-// load used for the four slots.
+// load used for all slots (pairs of them in packed arithmetic).
+template <int PAIRS>
 __device__ __forceinline__ void dense_product(const FitParams &P, const GalCtx &gc, const DenseView &dv, int gal,
                                               int n_slots)
 {
@@ -472,7 +473,13 @@ __device__ __forceinline__ void dense_product(const FitParams &P, const GalCtx &
     for (int a0 = 32 * warp; a0 < n; a0 += 32 * nwarp) {
         const int a = a0 + lane;
         const float *col = Pg + min(a, n - 1);
-        float2 y01 = make_float2(0.f, 0.f), y23 = make_float2(0.f, 0.f);
+        float2 y[PAIRS];
+#pragma unroll
+        for (int c = 0; c < PAIRS; ++c) y[c] = make_float2(0.f, 0.f);
+        auto term = [&](float p, const float4 &r) {
+            y[0] = fma2(f2(p), make_float2(r.x, r.y), y[0]);
+            if constexpr (PAIRS > 1) y[1] = fma2(f2(p), make_float2(r.z, r.w), y[1]);
+        };
         const float4 *r = dv.rb;
         int b0 = 0;
         for (; b0 + kAhead <= n; b0 += kAhead) {
@@ -481,11 +488,7 @@ __device__ __forceinline__ void dense_product(const FitParams &P, const GalCtx &
             for (int t = 0; t < kAhead; ++t) p[t] = __ldg(col + t * n);
             col += kAhead * n;
 #pragma unroll
-            for (int t = 0; t < kAhead; ++t) {
-                const float4 rv = r[t];
-                y01 = fma2(f2(p[t]), make_float2(rv.x, rv.y), y01);
-                y23 = fma2(f2(p[t]), make_float2(rv.z, rv.w), y23);
-            }
+            for (int t = 0; t < kAhead; ++t) term(p[t], r[t]);
             r += kAhead;
         }
         {
@@ -493,19 +496,13 @@ __device__ __forceinline__ void dense_product(const FitParams &P, const GalCtx &
 #pragma unroll
             for (int t = 0; t < kAhead; ++t) p[t] = b0 + t < n ? __ldg(col + t * n) : 0.f;
 #pragma unroll
-            for (int t = 0; t < kAhead; ++t) {
-                if (b0 + t < n) {
-                    const float4 rv = r[t];
-                    y01 = fma2(f2(p[t]), make_float2(rv.x, rv.y), y01);
-                    y23 = fma2(f2(p[t]), make_float2(rv.z, rv.w), y23);
-                }
-            }
+            for (int t = 0; t < kAhead; ++t)
+                if (b0 + t < n) term(p[t], r[t]);
         }
         if (a < n) {
-            const float y[4] = {y01.x, y01.y, y23.x, y23.y};
 #pragma unroll
-            for (int c = 0; c < kDenseChains; ++c)
-                if (c < n_slots) dv.yb(c)[a] = y[c];
+            for (int c = 0; c < 2 * PAIRS; ++c)
+                if (c < n_slots) dv.yb(c)[a] = (c & 1) ? y[c >> 1].y : y[c >> 1].x;
         }
     }
 }
@@ -745,7 +742,8 @@ __device__ bool dense_round(const FitParams &P, const GalCtx &gc, const SmemView
         else dense_residual<4>(P, gc, dv, gal, s, k, nk);
     }
     __syncthreads();
-    dense_product(P, gc, dv, gal, n_slots);
+    if (n_slots <= 2) dense_product<1>(P, gc, dv, gal, n_slots);
+    else dense_product<2>(P, gc, dv, gal, n_slots);
     __syncthreads();
     if (in) {
         if (ub <= 2) dense_back<2>(gc, dv, s, k, nk);
