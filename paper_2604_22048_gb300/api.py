@@ -50,13 +50,15 @@ def psf_table(kind, fwhm, beta=3.0, device="cuda"):
 def pack_stamps(sides, align=4):
     """Offsets of stamps packed back to back, each start rounded up to `align`
     elements.  Returns (offsets int64 array, total elements)."""
-    sides = np.asarray(sides, dtype=np.int64)
-    sizes = sides * sides
-    sizes = (sizes + align - 1) // align * align
-    offs = np.zeros(len(sides), dtype=np.int64)
-    if len(sides) > 1:
-        offs[1:] = np.cumsum(sizes)[:-1]
-    return offs, int(sizes.sum())
+    sizes = np.array(sides, dtype=np.int64)
+    sizes *= sizes
+    sizes += align - 1
+    sizes //= align
+    sizes *= align
+    ends = np.empty(len(sizes) + 1, dtype=np.int64)
+    ends[0] = 0
+    np.cumsum(sizes, out=ends[1:])
+    return ends[:-1], int(ends[-1])
 
 
 def render(theta, side, psf, *, shear=None, offsets=None, total=None, pixel_scale=PIXEL_SCALE,
@@ -66,15 +68,19 @@ def render(theta, side, psf, *, shear=None, offsets=None, total=None, pixel_scal
     (flat stamps, offsets)."""
     _need_cuda(theta, side, shear)
     n = theta.shape[0]
+    table, n_psf = psf
+    theta = theta.contiguous()
+    lib, stream = F.lib(), _stream()
+    # everything that does not need the sides is done above: the copy waits for the stream, and
+    # what follows it is time the GPU stands idle
     sides_h = side.cpu().numpy()
     if offsets is None:
         offs_h, total = pack_stamps(sides_h)
         offsets = torch.from_numpy(offs_h).to(theta.device)
     out = torch.zeros(total, dtype=torch.float32, device=theta.device)
     ms = int(max_side or sides_h.max())
-    table, n_psf = psf
-    F.check(F.lib().bs_render(n, _p(theta.contiguous()), _p(shear), _p(offsets), _p(side), ms,
-                              _p(table), n_psf, pixel_scale, _p(out), _stream()))
+    F.check(lib.bs_render(n, _p(theta), _p(shear), _p(offsets), _p(side), ms,
+                          _p(table), n_psf, pixel_scale, _p(out), stream))
     return out, offsets
 
 
@@ -129,7 +135,7 @@ class FitPlan:
         a.data = _p(data)
         a.offsets = _p(offsets)
         a.side = _p(side)
-        a.max_side = int(max_side or int(side.max().item()))
+        largest = None if max_side else side.max()   # read at the end
         a.psf = _p(table)
         a.n_psf = n_psf
         a.noise_sigma = _p(noise_sigma)
@@ -187,6 +193,8 @@ class FitPlan:
         o.warmup_accept_stat = _p(self.warm_stat)
         o.warmup_step_size = _p(self.warm_step)
         self.out = o
+        # the read waits for the stream: what a fit needs besides is prepared by then
+        a.max_side = int(max_side) if max_side else int(largest.item())
         self.ws_bytes = F.lib().bs_fit_workspace_bytes(C.byref(a))
         self.ws = torch.empty(self.ws_bytes, dtype=torch.uint8, device=dev)
 
@@ -406,7 +414,7 @@ def logpost_points(data, offsets, side, psf, noise_sigma, gal_index, theta, *, m
     a.data = _p(data)
     a.offsets = _p(offsets)
     a.side = _p(side)
-    a.max_side = int(max_side or int(side.max().item()))
+    largest = None if max_side else side.max()
     a.psf = _p(table)
     a.n_psf = n_psf
     a.noise_sigma = _p(noise_sigma)
@@ -422,8 +430,11 @@ def logpost_points(data, offsets, side, psf, noise_sigma, gal_index, theta, *, m
     n = theta.shape[0]
     lp = torch.empty(n, dtype=torch.float64, device=theta.device)
     g = torch.empty((n, 6), dtype=torch.float32, device=theta.device)
-    F.check(F.lib().bs_logpost_points(C.byref(a), n, _p(gal_index), _p(theta.contiguous()), _p(lp),
-                                      _p(g), _stream()))
+    theta = theta.contiguous()
+    lib, args = F.lib(), (n, _p(gal_index), _p(theta), _p(lp), _p(g), _stream())
+    # the read waits for the stream; nothing but the launch is left after it
+    a.max_side = int(max_side) if max_side else int(largest.item())
+    F.check(lib.bs_logpost_points(C.byref(a), *args))
     return lp, g
 
 
@@ -765,10 +776,10 @@ class ShearLogLike(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, params, plan: ShearPlan):
-        g1, g2, alpha = [float(x) for x in params.detach().cpu().double()]
-        out = plan.loglike(g1, g2, alpha, host=True)
-        ctx.save_for_backward(torch.tensor(out[1:], dtype=torch.float64))
-        return torch.tensor(out[0], dtype=torch.float64)
+        g1, g2, alpha = params.detach().cpu().double().tolist()
+        out = torch.from_numpy(plan.loglike(g1, g2, alpha, host=True))
+        ctx.save_for_backward(out[1:].clone())
+        return out[0].clone()
 
     @staticmethod
     def backward(ctx, gout):
