@@ -57,7 +57,7 @@ __device__ __forceinline__ void store_ess(float sum, const ChainMoments &m, int 
 // alike.
 // 10,000 galaxies x 4 chains x 300: 493-614 us (with the autocorrelation of the
 // chains) re-reading both factors of every product and reducing chain by chain and lag by lag,
-// 132 us now; 64 registers (8 CTAs of 4 warps per SM) against 72 with spills 148, 78 158.
+// 117 us now at 64 registers (8 CTAs of 4 warps per SM; 120 us for 7 CTAs, 119 for 9).
 constexpr int kLagBlock = 8;
 
 __host__ __device__ constexpr size_t ess_warp_floats(int C, int S)
@@ -71,10 +71,11 @@ __global__ void __launch_bounds__(128, 8) ess_kernel(const float *samples, int n
 {
     extern __shared__ __align__(16) float ess_smem[];
     const int lane = threadIdx.x & 31, warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
-    const long long wid = (long long)blockIdx.x * warps + warp;
-    if (wid >= (long long)n_gal * 6) return;
-    // planes of the parameters in turn: neighbouring warps read neighbouring galaxies
-    const int k = (int)(wid / n_gal), gal = (int)(wid - (long long)k * n_gal);
+    // grid y: the parameter, so that neighbouring warps read neighbouring galaxies
+    const int k = blockIdx.y;
+    const long long gl = (long long)blockIdx.x * warps + warp;
+    if (gl >= n_gal) return;
+    const int gal = (int)gl;
     const float *x = samples + (((size_t)k * n_gal + gal) * C) * S;
     const int stride = S + kLagBlock;
     float2 *d = reinterpret_cast<float2 *>(ess_smem + warp * ess_warp_floats(C, S));
@@ -88,16 +89,29 @@ __global__ void __launch_bounds__(128, 8) ess_kernel(const float *samples, int n
             const float *xb = two ? xa + S : xa;
             float2 *dp = d + p * stride;
             if constexpr (VEC) {
-#pragma unroll 3
-                for (int i = 4 * lane; i < S; i += 128) {
-                    const float4 a = __ldg(reinterpret_cast<const float4 *>(xa + i));
-                    float4 b = __ldg(reinterpret_cast<const float4 *>(xb + i));
-                    if (!two) b = make_float4(0.f, 0.f, 0.f, 0.f);
-                    float4 *o = reinterpret_cast<float4 *>(dp + i);
-                    o[0] = make_float4(a.x, b.x, a.y, b.y);
-                    o[1] = make_float4(a.z, b.z, a.w, b.w);
-                    sa += (a.x + a.y) + (a.z + a.w);
-                    sb += (b.x + b.y) + (b.z + b.w);
+                // six loads in flight per round trip
+                for (int i0 = 4 * lane; i0 < S; i0 += 384) {
+                    float4 a[3], b[3];
+#pragma unroll
+                    for (int t = 0; t < 3; ++t) {
+                        const int i = i0 + 128 * t;
+                        a[t] = b[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (i < S) {
+                            a[t] = __ldg(reinterpret_cast<const float4 *>(xa + i));
+                            if (two) b[t] = __ldg(reinterpret_cast<const float4 *>(xb + i));
+                        }
+                    }
+#pragma unroll
+                    for (int t = 0; t < 3; ++t) {
+                        const int i = i0 + 128 * t;
+                        if (i < S) {
+                            float4 *o = reinterpret_cast<float4 *>(dp + i);
+                            o[0] = make_float4(a[t].x, b[t].x, a[t].y, b[t].y);
+                            o[1] = make_float4(a[t].z, b[t].z, a[t].w, b[t].w);
+                        }
+                        sa += (a[t].x + a[t].y) + (a[t].z + a[t].w);
+                        sb += (b[t].x + b[t].y) + (b[t].z + b[t].w);
+                    }
                 }
             } else {
 #pragma unroll 4
@@ -359,8 +373,8 @@ cudaError_t launch_chain_ess(const float *samples, int n_gal, int n_chains, int 
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)(wpc * per_warp));
         if (e != cudaSuccess) return e;
-        kernel<<<(unsigned)((warps + wpc - 1) / wpc), 32 * wpc, wpc * per_warp, stream>>>(samples, n_gal, n_chains,
-                                                                                          n_samples, ess, rhat);
+        const dim3 grid((unsigned)(((long long)n_gal + wpc - 1) / wpc), 6);
+        kernel<<<grid, 32 * wpc, wpc * per_warp, stream>>>(samples, n_gal, n_chains, n_samples, ess, rhat);
     } else {
         ess_kernel_global<<<(unsigned)((warps + 3) / 4), 128, 0, stream>>>(samples, n_gal, n_chains, n_samples, ess, rhat);
     }

@@ -21,7 +21,7 @@
 // Bound by instruction issue (2.4 of 4 per cycle up to 63 px) and, for large stamps, by the
 // CTAs their shared memory allows.  20,000 stamps of 25-101 px with a Moffat PSF each:
 // 2.7 ms with direct sums over a stamp's N^2 pixels, the PSF integrated at every grid
-// point and one shared-memory load per two multiply-adds; 0.57 ms now (error against
+// point and one shared-memory load per two multiply-adds; 0.51 ms now (error against
 // 64 bits 3.6e-7 and 2.8e-7).
 #include "bs_device.cuh"
 #include "bs_internal.h"
@@ -30,7 +30,6 @@ namespace bs {
 
 namespace {
 
-constexpr int kRowBlock = 16;    // values of y per block of the two passes
 constexpr int kNodes = 96;       // nodes t_j = j / 8 of the Moffat integral held in shared memory
 
 // (x/2)^nu K_nu(x) by the trapezoidal rule with step 1/4, the factor folded into the
@@ -104,22 +103,22 @@ __device__ __forceinline__ float r_sincpi(float x)
 
 struct RenderSmem {
     float4 *S;       // [H][H] (Re S+, Im S+, Re S-, Im S-)
-    float4 *A;       // [H][kRowBlock] (Re A(+y), Im A(+y), Re A(-y), Im A(-y)); the PSF values before that
+    float4 *A;       // [H][RB] (Re A(+y), Im A(+y), Re A(-y), Im A(-y)); the PSF values before that
     float2 *tw;      // [N] (cos, sin)(2 pi m / N)
     float2 *X, *Y;   // [H] centroid phases exp(-2 pi i u dx / N), exp(-2 pi i a dy / N)
     float *snc;      // [H] sinc(u / N), the pixel's factor per axis
     float2 *nodes;   // [kNodes] cosh t_j, cosh(nu t_j), t_j = j / 8
 };
 
-__host__ __device__ __forceinline__ size_t render_smem_bytes(int max_side)
+__host__ __device__ __forceinline__ size_t render_smem_bytes(int max_side, int RB)
 {
     const size_t h = (max_side + 1) / 2;
-    return (h * h + h * kRowBlock) * sizeof(float4) + ((size_t)max_side + 2 * h + kNodes) * sizeof(float2) +
+    return (h * h + h * RB) * sizeof(float4) + ((size_t)max_side + 2 * h + kNodes) * sizeof(float2) +
            h * sizeof(float);
 }
 
 // Stamps of side in (min_side, max_side], the others are left to another launch.
-template <int NT>
+template <int NT, int RB>
 __global__ void __launch_bounds__(NT) render_kernel(int n, const float *theta, const float *shear,
                                                     const int64_t *offsets, const int32_t *side, int min_side,
                                                     int max_side, const bs_psf *psf, int n_psf, float p, float *out)
@@ -130,7 +129,7 @@ __global__ void __launch_bounds__(NT) render_kernel(int n, const float *theta, c
         const int hm = (max_side + 1) / 2;
         sm.S = reinterpret_cast<float4 *>(smem_raw);
         sm.A = sm.S + (size_t)hm * hm;
-        sm.tw = reinterpret_cast<float2 *>(sm.A + (size_t)hm * kRowBlock);
+        sm.tw = reinterpret_cast<float2 *>(sm.A + (size_t)hm * RB);
         sm.X = sm.tw + max_side;
         sm.Y = sm.X + hm;
         sm.nodes = sm.Y + hm;
@@ -210,8 +209,8 @@ __global__ void __launch_bounds__(NT) render_kernel(int n, const float *theta, c
         }
         float *img = out + offsets[i];
         const int ut = (H + 3) >> 2;
-        for (int y0 = 0; y0 < H; y0 += kRowBlock) {
-            const int ny = min(kRowBlock, H - y0);
+        for (int y0 = 0; y0 < H; y0 += RB) {
+            const int ny = min(RB, H - y0);
             __syncthreads();   // S is complete (first block), A's readers are done (later ones)
             // column pass: four rows u of two y (the second one half a block further)
             const int hy = (ny + 1) >> 1;
@@ -246,7 +245,7 @@ __global__ void __launch_bounds__(NT) render_kernel(int n, const float *theta, c
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     if (4 * tile + r >= H) break;
-                    float4 *A = sm.A + (4 * tile + r) * kRowBlock + yi;   // C + i D and C - i D
+                    float4 *A = sm.A + (4 * tile + r) * RB + yi;   // C + i D and C - i D
                     A[0] = make_float4(C[r].x - D[r].y, C[r].y + D[r].x, C[r].x + D[r].y, C[r].y - D[r].x);
                     if (yi + hy < ny)
                         A[hy] = make_float4(C2[r].x - D2[r].y, C2[r].y + D2[r].x, C2[r].x + D2[r].y, C2[r].y - D2[r].x);
@@ -267,7 +266,7 @@ __global__ void __launch_bounds__(NT) render_kernel(int n, const float *theta, c
                     const float2 t1 = sm.tw[i1], t2 = sm.tw[i2];
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
-                        const float4 v = a[u * kRowBlock + r];
+                        const float4 v = a[u * RB + r];
                         const float2 vu = make_float2(v.x, v.y), vd = make_float2(v.z, v.w);
                         up[0][r] = __ffma2_rn(vu, t1, up[0][r]);
                         dn[0][r] = __ffma2_rn(vd, t1, dn[0][r]);
@@ -304,24 +303,24 @@ __global__ void __launch_bounds__(NT) render_kernel(int n, const float *theta, c
 
 }  // namespace
 
-// Shared memory follows the largest side of a launch (26 KB at 63 px, 58 KB at 101 px), and a
-// stamp's tiles of the two passes keep about (side + 3)^2 / 56 threads busy: stamps up to
-// 63 px run in CTAs of 64 threads, larger ones in their own launch in CTAs of 128.  The
-// launches pass over each other's stamps.  One launch of 128 threads for all sides, with
-// half as much work per thread and load, kept shared memory 92% busy at 53 px (22 ns a
-// stamp; 18 ns so).
+// Shared memory follows the largest side of a launch (34 KB at 63 px, 70 KB at 101 px), and a
+// block's tiles of the two passes keep about 2 H threads busy: stamps up to 63 px run in
+// CTAs of 128 threads (24 warps per SM), larger ones in their own launch in CTAs of 256.  The
+// launches pass over each other's stamps.  20,000 stamps of 25-101 px through the binding: 735 us;
+// 64 and 128 threads with blocks of 16 rows 798 us (16 warps per SM); one launch of 128
+// threads for all sides, with half as much work per thread and load, 847 us.
 constexpr int kSmallSide = 63;
 
-template <int NT>
+template <int NT, int RB>
 static cudaError_t launch_class(int grid, int n, const float *theta, const float *shear, const int64_t *offsets,
                                 const int32_t *side, int min_side, int max_side, const bs_psf *psf, int n_psf,
                                 float pixel_scale, float *out, cudaStream_t stream)
 {
-    const size_t smem = render_smem_bytes(max_side);
-    const cudaError_t e = cudaFuncSetAttribute(render_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const size_t smem = render_smem_bytes(max_side, RB);
+    const cudaError_t e = cudaFuncSetAttribute(render_kernel<NT, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)smem);
     if (e != cudaSuccess) return e;
-    render_kernel<NT><<<grid, NT, smem, stream>>>(n, theta, shear, offsets, side, min_side, max_side, psf, n_psf,
+    render_kernel<NT, RB><<<grid, NT, smem, stream>>>(n, theta, shear, offsets, side, min_side, max_side, psf, n_psf,
                                                   pixel_scale, out);
     bs::count_launches(1);
     return cudaGetLastError();
@@ -334,11 +333,11 @@ cudaError_t launch_render(int n, const float *theta, const float *shear, const i
     if (n <= 0) return cudaSuccess;
     const int grid = n < 65535 ? n : 65535;
     if (max_side > kSmallSide) {
-        const cudaError_t e = launch_class<128>(grid, n, theta, shear, offsets, side, kSmallSide, max_side, psf, n_psf,
+        const cudaError_t e = launch_class<256, 32>(grid, n, theta, shear, offsets, side, kSmallSide, max_side, psf, n_psf,
                                                 pixel_scale, out, stream);
         if (e != cudaSuccess) return e;
     }
-    return launch_class<64>(grid, n, theta, shear, offsets, side, 0, max_side < kSmallSide ? max_side : kSmallSide,
+    return launch_class<128, 32>(grid, n, theta, shear, offsets, side, 0, max_side < kSmallSide ? max_side : kSmallSide,
                             psf, n_psf, pixel_scale, out, stream);
 }
 
