@@ -12,14 +12,13 @@
 //   m(y, +-x) = P -+ Q, the weights w_u / N^2 (w_0 = 1, w_u = 2) folded into M:
 //     two pixels for 2 multiply-adds per (u, y, x).
 // The column pass thus costs a quarter and the row pass half of the direct sums.  Rows go
-// through shared memory in blocks of 16 values of y (32 rows), so that A takes H x 16
-// entries instead of H x N and more CTAs fit an SM; a thread sums four rows u of one y
-// (column pass) or eight rows of one x (row pass), so that a twiddle and its index serve
-// several packed FP32x2 multiply-adds.
+// through shared memory in blocks of RB values of y (2 RB rows), so that A takes H x RB
+// entries instead of H x N and more CTAs fit an SM; a thread sums four rows u of two y
+// (column pass) or eight rows of two x (row pass), so that a load serves several packed
+// FP32x2 multiply-adds.
 // The PSF depends on |k| alone: it is formed for the H (H + 1) / 2 pairs (u, a <= u) and
 // read for (u, +-a) and (a, +-u).
-// Bound by instruction issue (2.4 of 4 per cycle up to 63 px) and, for large stamps, by the
-// CTAs their shared memory allows.  20,000 stamps of 25-101 px with a Moffat PSF each:
+// Bound by instruction issue and by the CTAs that shared memory allows (24 warps per SM).  20,000 stamps of 25-101 px with a Moffat PSF each:
 // 2.7 ms with direct sums over a stamp's N^2 pixels, the PSF integrated at every grid
 // point and one shared-memory load per two multiply-adds; 0.51 ms now (error against
 // 64 bits 3.6e-7 and 2.8e-7).
