@@ -76,7 +76,7 @@ __device__ void pix_tc_setup(const FitParams &P, const GalCtx &gc, const SmemVie
     tc::fence_after();
 }
 
-// One 3xTF32 product into TMEM columns [0, N) (all threads; thread 0 issues and
+// One 3xTF32 product into TMEM columns [0, N) (all threads; one lane of the first warp issues and
 // commits, everyone waits for the given parity).  K runs over n_q halves of nk steps
 // of 8: step (q, k) reads A at TMEM column a + q a_q + 8 k (its low part a_lo columns
 // further) and B at b + q b_q + 288 k bytes (the data operand: leading offset 144 B,
@@ -96,9 +96,14 @@ __device__ __forceinline__ bool tc_run(const PixTc &px, const TcGemm &G, uint32_
         return false;
     }
     const uint32_t bar = tc::saddr(px.bar);
-    if (threadIdx.x == 0) {
+    // The first warp as a whole runs the loop and one elected lane issues, so that the
+    // descriptors stay in uniform registers: under a test of the thread index each of them was moved
+    // there again for every MMA, about 50 cycles an MMA against 21 (400 galaxies of 41 px:
+    // 101.0 -> 90.3 ms; unrolling the loop by four gave nothing on either form).
+    if (__shfl_sync(BS_FULL_MASK, threadIdx.x >> 5, 0) == 0) {
         tc::fence_after();
-        const uint32_t tmem = *px.tmem;
+        const uint32_t elected = tc::elect_one();
+        const uint32_t tmem = __shfl_sync(BS_FULL_MASK, *px.tmem, 0);
         const uint32_t b_lo = tc::kBopFloats * 4;
         for (int q = 0; q < G.n_q; ++q) {
             // a k-step advances the B descriptor's start-address field (bytes / 16, the
@@ -106,16 +111,17 @@ __device__ __forceinline__ bool tc_run(const PixTc &px, const TcGemm &G, uint32_
             uint32_t a = tmem + G.a + q * G.a_q;
             const uint32_t b0 = G.b + q * G.b_q;
             uint64_t bh = tc::sdesc(b0, tc::kLboB, G.sbo_b), bl = tc::sdesc(b0 + b_lo, tc::kLboB, G.sbo_b);
+#pragma unroll 1
             for (int k = 0; k < G.nk; ++k) {
-                tc::mma_ta(tmem, a, bl, G.id, (q | k) ? 1u : 0u);
-                tc::mma_ta(tmem, a + G.a_lo, bh, G.id, 1u);
-                tc::mma_ta(tmem, a, bh, G.id, 1u);
+                tc::mma_ta(elected, tmem, a, bl, G.id, (q | k) ? 1u : 0u);
+                tc::mma_ta(elected, tmem, a + G.a_lo, bh, G.id, 1u);
+                tc::mma_ta(elected, tmem, a, bh, G.id, 1u);
                 a += 8;
                 bh += 288 / 16;
                 bl += 288 / 16;
             }
         }
-        tc::commit(bar);
+        tc::commit(elected, bar);
     }
     failed = !tc::wait_parity(bar, parity);
     tc::fence_after();

@@ -34,7 +34,7 @@
 // at each one; every product carries both chains' data (B rows (chain, u) or (chain,
 // iy)), so each barrier and MMA round trip serves two evaluations.  Thread t reads TMEM
 // lane 32 (w mod 4) + (t mod 32) and its chain's columns (w / 4), the group's warps
-// split the spectral gradient pass by rows, and thread 0 issues the MMAs.  A chain that
+// split the spectral gradient pass by rows, and one lane of the first warp issues the MMAs.  A chain that
 // has finished, or has no evaluation at a step, joins with a skip flag until both are
 // done.  Each evaluation commits four MMA groups to one mbarrier, so the parities it
 // waits on are 0, 1, 0, 1 in every evaluation.  A wait gives up after two seconds: the
@@ -94,10 +94,13 @@ __device__ __forceinline__ void split_store(float *hi, float *lo, int i, float x
     lo[i] = tf32_rn(x - h);
 }
 
-__device__ __forceinline__ void commit(uint32_t bar)
+__device__ __forceinline__ void commit(uint32_t elected, uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                 : "memory");
+    asm volatile(
+        "{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar),
+        "r"(elected)
+        : "memory");
 }
 
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -190,12 +193,22 @@ constexpr int kColA2 = 384;                    // the complex-to-real constant, 
 constexpr int kColA2lo = 448;
 constexpr int kThreads = 256;                  // eight warps: lane quadrant w % 4, chain w / 4
 
-__device__ __forceinline__ void mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t id, uint32_t accumulate)
+// One lane of a converged warp: 1 there, 0 in the others.
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e;
+}
+
+// Executed by the whole warp with the same operands; the elected lane issues.
+__device__ __forceinline__ void mma_ta(uint32_t elected, uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t id,
+                                       uint32_t accumulate)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(b), "r"(id), "r"(accumulate));
+        "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b), "r"(id), "r"(accumulate), "r"(elected));
 }
 
 // Eight consecutive TMEM columns of this thread's lane.
