@@ -207,7 +207,7 @@ typedef struct {
                                      then renders the model image and transforms
                                      the weighted residual back (four dense
                                      DFT-matrix products on the tensor cores,
-                                     3xTF32, two chains per CTA).  Requires the
+                                     3xTF32, two or four chains per CTA).  Requires the
                                      exponential profile, one exposure, no
                                      noise_corr and max_side <= 63. */
     const float *pixel_prec;      /* NULL, or device float: a general pixel

@@ -994,6 +994,9 @@ __device__ __forceinline__ double eval_logpost(const FitParams &P, const GalCtx 
     return -0.5 * (chi2 + s_chi2_off) * (double)gc.inv_b + (double)lprior;
 }
 
+// Chains per CTA of the pixel-weight kernels (instances PROF 3 and 5; 0: another path).
+__host__ __device__ constexpr int pix_chains(int prof) { return prof == 3 ? 2 : prof == 5 ? 4 : 0; }
+
 #include "bs_fit_pixel.cuh"
 
 __device__ __forceinline__ float pick6(const float (&v)[6], int i)
@@ -1044,9 +1047,9 @@ __device__ __forceinline__ bool trajectory(const FitParams &P, const GalCtx &gc,
         for (int k = 0; k < 6; ++k) x[k] = __shfl_sync(BS_FULL_MASK, tp, k);
         if (!in_support(P, x)) return false;
         double v;
-        if constexpr (PROF == 3) {
+        if constexpr (pix_chains(PROF) > 0) {
             float gg[6];
-            v = eval_pix<NC>(P, gc, sm, gal, xph_c, vcol, x, gg, l == nst - 1, nullptr);
+            v = eval_pix<NC, pix_chains(PROF)>(P, gc, sm, gal, xph_c, vcol, x, gg, l == nst - 1, nullptr);
             gp = pick6(gg, pi);
         } else if constexpr (PROF == 4) {
             dense_round<NC>(P, gc, sm, gal, cta_chains(P), true, slot, vcol, x, gp, l == nst - 1, v);
@@ -1077,8 +1080,6 @@ struct ChainScalars {
 struct ChainLanes {
     float th[8], thl[8], g[8], wmean[8], wm2[8];
 };
-__shared__ ChainScalars s_chain_scal[kMaxChains];
-__shared__ ChainLanes s_chain_lanes[kMaxChains];
 
 // Chain `chain` of galaxy gal, run by the warp of the CTA's `slot`.
 template <int NC, int PROF>
@@ -1089,8 +1090,11 @@ __device__ void run_chain(const FitParams &P, const GalCtx &gc, const SmemView &
     const int pi = lane < 6 ? lane : 5;     // parameter of this lane (lanes 6.. shadow parameter 5)
     const bool own = lane < 6;
     // the pixel path's groups of four warps run one chain each: their first warp writes
-    const bool wr = PROF != 3 || (threadIdx.x & 127) < 32;
+    const bool wr = pix_chains(PROF) == 0 || (threadIdx.x & 127) < 32;
     const int C = P.n_chains, W = P.n_warmup, S = P.n_samples, L = P.n_leapfrog;
+    constexpr int kSlots = 4 * pix_chains(PROF) > kMaxChains ? 4 * pix_chains(PROF) : kMaxChains;
+    __shared__ ChainScalars s_chain_scal[kSlots];
+    __shared__ ChainLanes s_chain_lanes[kSlots];
     ChainScalars &cs = s_chain_scal[threadIdx.x >> 5];
     ChainLanes &cl = s_chain_lanes[threadIdx.x >> 5];
     const uint64_t gid = P.gal_id ? P.gal_id[gal] : (uint64_t)gal;
@@ -1329,11 +1333,12 @@ __device__ __forceinline__ void fit_loop(const FitParams &P)
     __shared__ int s_gal, s_grp;
     const int cc = cta_chains(P);              // chains of this CTA
     const int groups = cta_groups(P);          // CTAs a galaxy's chains are split over
-    // the pixel path: two chains per CTA, each run by a group of four warps (a phase
+    // the pixel path: two or four chains per CTA, each run by a group of four warps (a phase
     // table per group)
-    const SmemView sm = smem_view(smem_raw, P.h_max, P.npad, P.max_side, PROF == 3 ? 2 : cc);
+    constexpr int PG = pix_chains(PROF);
+    const SmemView sm = smem_view(smem_raw, P.h_max, P.npad, P.max_side, PG > 0 ? PG : cc);
     const int warp = threadIdx.x >> 5;
-    if constexpr (PROF == 3) pix_tc_begin(pix_tc_view(sm.kxr, P.h_max, P.npad, P.max_side));
+    if constexpr (PG > 0) pix_tc_begin(pix_tc_view<PG>(sm.kxr, P.h_max, P.npad, P.max_side));
     bool first = true;
     for (;;) {
         if (threadIdx.x == 0) {
@@ -1368,17 +1373,17 @@ __device__ __forceinline__ void fit_loop(const FitParams &P)
             if (P.done) publish_galaxy(P, gal);
             continue;
         }
-        if constexpr (PROF == 3) {
-            const PixTc px = pix_tc_view(sm.kxr, P.h_max, P.npad, P.max_side);
-            if (threadIdx.x == 0) px.done[0] = px.done[1] = 0;
-            pix_tc_setup(P, gc, sm, px, gal);
-            const int grp = warp >> 2, chain = 2 * s_grp + grp;
+        if constexpr (PG > 0) {
+            const PixTc px = pix_tc_view<PG>(sm.kxr, P.h_max, P.npad, P.max_side);
+            if (threadIdx.x < PG) px.done[threadIdx.x] = 0;
+            pix_tc_setup<PG>(P, gc, sm, px, gal);
+            const int grp = warp >> 2, chain = PG * s_grp + grp;
             float vcol[NC];
 #pragma unroll
             for (int j = 0; j < NC; ++j) vcol[j] = (float)((threadIdx.x & 31) + 32 * j - gc.c);
             float4 *xph = sm.xph + (size_t)grp * phase_stride(P.h_max);
             if (chain < P.n_chains) run_chain<NC, PROF>(P, gc, sm, gal, chain, grp);
-            pix_drain<NC>(P, gc, sm, gal, xph, vcol);
+            pix_drain<NC, PG>(P, gc, sm, gal, xph, vcol);
             __syncthreads();
             if (threadIdx.x == 0 && *px.abort && P.status) P.status[gal] = 4;
         } else {
@@ -1393,7 +1398,7 @@ __device__ __forceinline__ void fit_loop(const FitParams &P)
         __syncthreads();
         if (P.done) publish_galaxy(P, gal);
     }
-    if constexpr (PROF == 3) pix_tc_end(pix_tc_view(sm.kxr, P.h_max, P.npad, P.max_side));
+    if constexpr (PG > 0) pix_tc_end(pix_tc_view<PG>(sm.kxr, P.h_max, P.npad, P.max_side));
 }
 
 // Register budgets of the kernel instances (the launch bounds give ptxas the
@@ -1406,10 +1411,14 @@ template <int NC, int PROF>
 __global__ void __launch_bounds__(128, 5) fit_kernel_r96(const FitParams P) { fit_loop<NC, PROF>(P); }
 template <int NC, int PROF>
 __global__ void __launch_bounds__(256, 3) fit_kernel_r80(const FitParams P) { fit_loop<NC, PROF>(P); }
-// The pixel path: two chains per CTA of eight warps; its tensor memory (the transforms'
-// constants and accumulator: all 512 columns) allows one CTA per SM.
-template <int NC>
-__global__ void __launch_bounds__(tc::kThreads, 1) fit_kernel_pix(const FitParams P) { fit_loop<NC, 3>(P); }
+// The pixel path: two chains per CTA of eight warps (PROF 3) or four per CTA of sixteen (PROF 5); its
+// tensor memory (the transforms' constants and accumulator: all 512 columns) allows one CTA
+// per SM.
+template <int NC, int PROF>
+__global__ void __launch_bounds__(tc::Geo<pix_chains(PROF)>::kThreads, 1) fit_kernel_pix(const FitParams P)
+{
+    fit_loop<NC, PROF>(P);
+}
 
 // The dense covariance: one CTA of 16 warps per galaxy, its chains in step (dense_round).
 template <int NC>
@@ -1518,13 +1527,13 @@ __global__ void __launch_bounds__(32 * kDenseWarps, 1) logpost_points_dense_kern
 // The pixel path's points: one CTA of eight warps per point; the first group of four
 // warps evaluates it, the second joins with a skip flag.
 template <int NC>
-__global__ void __launch_bounds__(tc::kThreads, 1) logpost_points_pix_kernel(const FitParams P, int n_points,
+__global__ void __launch_bounds__(tc::Geo<2>::kThreads, 1) logpost_points_pix_kernel(const FitParams P, int n_points,
                                                                             const int32_t *gal_index, const float *theta,
                                                                             double *logp, float *grad)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SmemView sm = smem_view(smem_raw, P.h_max, P.npad, P.max_side, 2);
-    const PixTc px = pix_tc_view(sm.kxr, P.h_max, P.npad, P.max_side);
+    const PixTc px = pix_tc_view<2>(sm.kxr, P.h_max, P.npad, P.max_side);
     pix_tc_begin(px);
     const int grp = threadIdx.x >> 7, lane = threadIdx.x & 31;
     for (int i = blockIdx.x; i < n_points; i += gridDim.x) {
@@ -1538,7 +1547,7 @@ __global__ void __launch_bounds__(tc::kThreads, 1) logpost_points_pix_kernel(con
             continue;
         }
         if (threadIdx.x == 0) px.done[0] = px.done[1] = 0;
-        pix_tc_setup(P, gc, sm, px, gal);
+        pix_tc_setup<2>(P, gc, sm, px, gal);
         float vcol[NC];
 #pragma unroll
         for (int j = 0; j < NC; ++j) vcol[j] = (float)(lane + 32 * j - gc.c);
@@ -1550,7 +1559,7 @@ __global__ void __launch_bounds__(tc::kThreads, 1) logpost_points_pix_kernel(con
             for (int k = 0; k < 6; ++k) t[k] = th[k];
             double v = -INFINITY;
             if (in_support(P, t)) {
-                v = eval_pix<NC>(P, gc, sm, gal, xph, vcol, t, g, true, nullptr);
+                v = eval_pix<NC, 2>(P, gc, sm, gal, xph, vcol, t, g, true, nullptr);
             } else {
 #pragma unroll
                 for (int k = 0; k < 6; ++k) g[k] = NAN;
@@ -1558,7 +1567,7 @@ __global__ void __launch_bounds__(tc::kThreads, 1) logpost_points_pix_kernel(con
             if (threadIdx.x == 0 && logp) logp[i] = v;
             if (grad && threadIdx.x < 6) grad[(size_t)i * 6 + threadIdx.x] = pick6(g, threadIdx.x);
         }
-        pix_drain<NC>(P, gc, sm, gal, xph, vcol);
+        pix_drain<NC, 2>(P, gc, sm, gal, xph, vcol);
         __syncthreads();
     }
     pix_tc_end(px);

@@ -9,14 +9,16 @@
 // Re[conj(R_k) dM_k / dtheta] / (sigma^2 N^2) with R = DFT(w (d - m)), so the half-plane
 // pass of eval_logpost gives it when its data spectrum is replaced by the effective
 // D' = M + R (scaled as the table).  The transforms run on the tensor cores (the layout
-// and operand split are described with PixTc); one CTA of eight warps evaluates two chains.
+// and operand split are described with PixTc); one CTA evaluates two or four chains (G).
 
 // Per galaxy (all threads): the A operands of the four products for this side into
 // tensor memory (warp w writes lanes 32 (w mod 4) .. + 31, the high parts for w < 4 and
-// the low parts otherwise), the second chain's copy of the table, and the stamp and
+// the low parts otherwise), the further chains' copies of the table, and the stamp and
 // its weights in shared memory.
+template <int G>
 __device__ void pix_tc_setup(const FitParams &P, const GalCtx &gc, const SmemView &sm, const PixTc &px, int gal)
 {
+    using Q = tc::Geo<G>;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int N = gc.N, c = gc.c, H = gc.H;
     const int row = 32 * (warp & 3) + lane;      // the TMEM lane this thread writes
@@ -25,11 +27,11 @@ __device__ void pix_tc_setup(const FitParams &P, const GalCtx &gc, const SmemVie
     auto part = [&](float x) { const float h = tc::tf32_rn(x); return lo ? tc::tf32_rn(x - h) : h; };
     // [[C, -S], [S, C]]: row r = (p, a), column k = (q, b): p = q gives C, else -S (p = 0) or S
     const int p = row >> 6, a = row & 63;
-    for (int k0 = 0; k0 < 128; k0 += 8) {
+    for (int k0 = 0; k0 < 2 * Q::KV && warp < 8; k0 += 8) {
         float v[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const int k = k0 + j, q = k >> 6, b = k & 63;
+            const int k = k0 + j, q = k >= Q::KV, b = k - q * Q::KV;
             float co = 0.f, sn = 0.f;
             if (a < N && b < N) {
                 int m = ((a - c) * (b - c)) % N;   // exact reduction of the phase index
@@ -38,17 +40,17 @@ __device__ void pix_tc_setup(const FitParams &P, const GalCtx &gc, const SmemVie
             }
             v[j] = part(p == q ? co : (p == 0 ? -sn : sn));
         }
-        tc::st8(tl + (lo ? tc::kColAFlo : tc::kColAF) + k0, v);
+        tc::st8(tl + (lo ? Q::kColAFlo : Q::kColAF) + k0, v);
     }
     // the complex-to-real constant: rows ix < 64, K (re, u | im, u):
     // (w_u / N^2) (cos, -sin)(2 pi u (ix - c) / N); rows 64 + ix again, so that the model image
     // comes out in both halves of the accumulator's lanes
     const float wn = 1.0f / ((float)N * (float)N);
-    for (int k0 = 0; k0 < 64; k0 += 8) {
+    for (int k0 = 0; k0 < 2 * Q::KU && warp < 8; k0 += 8) {
         float v[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const int k = k0 + j, q = k >> 5, u = k & 31;
+            const int k = k0 + j, q = k >= Q::KU, u = k - q * Q::KU;
             float co = 0.f, sn = 0.f;
             if (a < N && u < H) {
                 int m = (u * (a - c)) % N;
@@ -60,11 +62,15 @@ __device__ void pix_tc_setup(const FitParams &P, const GalCtx &gc, const SmemVie
             }
             v[j] = part(q ? -sn : co);
         }
-        tc::st8(tl + (lo ? tc::kColA2lo : tc::kColA2) + k0, v);
+        tc::st8(tl + (lo ? Q::kColA2lo : Q::kColA2) + k0, v);
     }
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     const int nrow = gc.H * row_floats(P.npad);
-    for (int i = tid; i < nrow; i += blockDim.x) px.tab1[i] = sm.tab[i];
+    for (int i = tid; i < nrow; i += blockDim.x) {
+        const float t = sm.tab[i];
+#pragma unroll
+        for (int g = 0; g < G - 1; ++g) px.tab1[(size_t)g * P.h_max * row_floats(P.npad) + i] = t;
+    }
     const int64_t off = P.offsets[gal];
     const int n = N * N;
     for (int i = tid; i < n; i += blockDim.x) {
@@ -87,6 +93,7 @@ struct TcGemm {
     uint32_t a, a_q, a_lo, b, b_q, sbo_b, id;
     int n_q, nk;
 };
+template <int CG>
 __device__ __forceinline__ bool tc_run(const PixTc &px, const TcGemm &G, uint32_t parity, bool &failed)
 {
     tc::fence_async_smem();
@@ -104,7 +111,7 @@ __device__ __forceinline__ bool tc_run(const PixTc &px, const TcGemm &G, uint32_
         tc::fence_after();
         const uint32_t elected = tc::elect_one();
         const uint32_t tmem = __shfl_sync(BS_FULL_MASK, *px.tmem, 0);
-        const uint32_t b_lo = tc::kBopFloats * 4;
+        const uint32_t b_lo = tc::Geo<CG>::kBopFloats * 4;
         for (int q = 0; q < G.n_q; ++q) {
             // a k-step advances the B descriptor's start-address field (bytes / 16, the
             // low 14 bits; every address stays below 256 KB, so the field does not carry)
@@ -162,31 +169,35 @@ __device__ __forceinline__ void pix_grad(const FitParams &P, const GalCtx &gc, c
     spectral_grad<0>(P, gc, m, sums, th, g);
 }
 
-// One evaluation of both chains of the CTA (all threads; each group passes its own
+// One evaluation of the G chains of the CTA (all threads; each group passes its own
 // chain's th; a group with skip set passes any finite th and ignores the results).
 // Returns the log posterior of the caller's chain if want_ll (the caller's group's
-// flag), else 0; *all_done is set when both groups have raised their done flags (the
+// flag), else 0; *all_done is set when all groups have raised their done flags (the
 // evaluation then does nothing).
-template <int NC>
+template <int NC, int G>
 __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView &sm, int gal, float4 *xph,
                            const float vcol[NC], const float th[6], float g[6], bool want_ll, bool *all_done)
 {
+    using Q = tc::Geo<G>;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int grp = warp >> 2;                        // the chain of this thread's group
     const int L = 32 * (warp & 3) + lane;             // this thread's TMEM lane
     const int tg = tid & 127;                         // thread within the group
-    const PixTc px = pix_tc_view(sm.kxr, P.h_max, P.npad, P.max_side);
+    const PixTc px = pix_tc_view<G>(sm.kxr, P.h_max, P.npad, P.max_side);
     const int N = gc.N, H = gc.H, c = gc.c;
     constexpr int npad = 32 * NC, rowf = 96 * NC;
-    float *tab = grp ? px.tab1 : sm.tab;
+    float *tab = grp ? px.tab1 + (size_t)(grp - 1) * P.h_max * rowf : sm.tab;
     const Shape ms = model_shape<0>(P, th);
     const float F = ms.F, E = ms.E, al = ms.al, be = ms.be, ga = ms.ga;
     __syncthreads();   // the previous evaluation's readers of the tables and buffers are done
-    if (all_done) *all_done = px.done[0] && px.done[1];
-    if (px.done[0] && px.done[1]) return 0.0;
+    bool done = true;
+#pragma unroll
+    for (int q = 0; q < G; ++q) done = done && px.done[q];
+    if (all_done) *all_done = done;
+    if (done) return 0.0;
     if (*px.abort) return pix_nan(g);
     const float sqrt2 = 1.41421356237309515f;
-    float *bh = px.bop, *bl = px.bop + tc::kBopFloats;
+    float *bh = px.bop, *bl = px.bop + Q::kBopFloats;
     constexpr int kLb = tc::kLboB / 4;
     const int ks = (N + 7) >> 3;          // k-steps of 8 covering the side
     const int n8 = 8 * ks;                // columns or rows of one chain over iy (or ix)
@@ -211,7 +222,7 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
         const int eo = (vi >> 2) * kLb + (vi & 3) + u0 * 4;
 #pragma unroll 1
         for (int ug = 0; ug < h8; ug += 8) {
-            const int e0 = eo + ((h8 * grp + ug) >> 3) * 32 * kLb;
+            const int e0 = eo + ((h8 * grp + ug) >> 3) * (Q::KV / 2) * kLb;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int u = ug + u0 + 2 * j;
@@ -230,17 +241,22 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
                     Mr = mr * inv_scale;
                     Mi = mi * inv_scale;
                 }
-                tc::split_store(bh, bl, e0 + 8 * j, Mr);
-                tc::split_store(bh, bl, e0 + 8 * j + 16 * kLb, Mi);   // K index 64 + vi
+                if (Q::KV == 64 || vi < Q::KV) {
+                    tc::split_store(bh, bl, e0 + 8 * j, Mr);
+                    tc::split_store(bh, bl, e0 + 8 * j + (Q::KV / 4) * kLb, Mi);   // K index KV + vi
+                }
             }
         }
     }
     const uint32_t bop = tc::saddr(px.bop);
     const uint32_t tl = *px.tmem + ((uint32_t)(32 * (warp & 3)) << 16);
-    constexpr uint32_t aflo = tc::kColAFlo - tc::kColAF, a2lo = tc::kColA2lo - tc::kColA2;
+    constexpr uint32_t aflo = Q::kColAFlo - Q::kColAF, a2lo = Q::kColA2lo - Q::kColA2;
+    constexpr uint32_t core = tc::kLboB;                            // bytes of a core matrix
+    constexpr uint32_t sbo_v2 = Q::KV / 2 * core, sbo_v = Q::KV / 4 * core, sbo_u2 = Q::KU / 2 * core;
     bool failed = false;
-    // (1) G = M E for both chains: rows (re, iy | im, iy), columns (chain, u)
-    if (!tc_run(px, TcGemm{tc::kColAF, 64u, aflo, bop, 16u * 144, 32u * 144, tc::idesc(128, 2 * h8), 2, ks}, 0, failed))
+    // (1) G = M E for all chains: rows (re, iy | im, iy), columns (chain, u)
+    if (!tc_run<G>(px, TcGemm{Q::kColAF, Q::KV, aflo, bop, Q::KV / 4 * core, sbo_v2, tc::idesc(128, G * h8), 2, ks}, 0,
+                   failed))
         return pix_nan(g);
     // (1) -> operand of (2): row (chain, iy), K (re, u | im, u), G as it is (the weights
     // are in the constant); this thread's lane (p, iy), its chain's h8 columns
@@ -249,7 +265,7 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
         tc::ld8n(tl + h8 * grp, h8 >> 3, v);
         const int p = L >> 6, iy = L & 63;
         if (iy < n8) {
-            const int e0 = tc::op_index(n8 * grp + iy, p * 32, 64, kLb);
+            const int e0 = tc::op_index(n8 * grp + iy, p * Q::KU, 2 * Q::KU, kLb);
 #pragma unroll
             for (int m = 0; m < 8; ++m)
                 if (4 * m < h8)
@@ -257,9 +273,9 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
         }
     }
     // (2) m = W G: rows ix (twice), columns (chain, iy)
-    if (!tc_run(px, TcGemm{tc::kColA2, 32u, a2lo, bop, 8u * 144, 16u * 144, tc::idesc(128, 2 * n8), 2,
-                           (H + 7) >> 3},
-                1, failed))
+    if (!tc_run<G>(px, TcGemm{Q::kColA2, Q::KU, a2lo, bop, Q::KU / 4 * core, sbo_u2, tc::idesc(128, G * n8), 2,
+                              (H + 7) >> 3},
+                   1, failed))
         return pix_nan(g);
     // the residual and the operand of (3): rows (chain, iy), K ix; the group's warps 0 and 1
     // (lanes ix) take the first half of the eight-row groups, warps 2 and 3 (lanes 64 + ix) the rest
@@ -269,13 +285,14 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
         float m[32];
         tc::ld8n(tl + n8 * grp + 8 * g0, ng, m);
         const float *dp = px.dimg + 8 * g0 * N + ix, *wp = px.wimg + 8 * g0 * N + ix;
-        const int e0 = (ix >> 2) * kLb + (ix & 3) + (ks * grp + g0) * 16 * kLb;
+        const int e0 = (ix >> 2) * kLb + (ix & 3) + (ks * grp + g0) * (Q::KV / 4) * kLb;
 #pragma unroll
         for (int t = 0; t < 32; ++t) {
             if (t < 8 * ng) {
                 float r = 0.f;
                 if (ix < N && 8 * g0 + t < N) r = wp[t * N] * (dp[t * N] - m[t]);
-                tc::split_store(bh, bl, e0 + (t >> 3) * 16 * kLb + ((t & 7) << 2), r);
+                if (Q::KV == 64 || ix < Q::KV)
+                    tc::split_store(bh, bl, e0 + (t >> 3) * (Q::KV / 4) * kLb + ((t & 7) << 2), r);
             }
         }
     }
@@ -305,7 +322,7 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
         if (lane == 0) px.chi[warp] = cw;
     }
     // (3) conj Q = [C; S] r: rows (re, a | im, a), columns (chain, iy)
-    if (!tc_run(px, TcGemm{tc::kColAF, 0u, aflo, bop, 0u, 16u * 144, tc::idesc(128, 2 * n8), 1, ks}, 0, failed))
+    if (!tc_run<G>(px, TcGemm{Q::kColAF, 0u, aflo, bop, 0u, sbo_v, tc::idesc(128, G * n8), 1, ks}, 0, failed))
         return pix_nan(g);
     // (3) -> operand of (4): row (chain, u = a - c < h8), K (re, iy | im, iy); this
     // thread's lane (q, a), its chain's n8 columns iy
@@ -316,7 +333,7 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
             float v[16];
             tc::ld16(tl + n8 * grp + y0, v);
             if (u >= 0 && u < h8) {
-                const int e0 = tc::op_index(h8 * grp + u, q * 64 + y0, 128, kLb);
+                const int e0 = tc::op_index(h8 * grp + u, q * Q::KV + y0, 2 * Q::KV, kLb);
 #pragma unroll
                 for (int m = 0; m < 4; ++m)
                     if (y0 + 4 * m < n8)
@@ -325,7 +342,8 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
         }
     }
     // (4) conj R = E conj Q: rows (re, vi | im, vi), columns (chain, u)
-    if (!tc_run(px, TcGemm{tc::kColAF, 64u, aflo, bop, 16u * 144, 32u * 144, tc::idesc(128, 2 * h8), 2, ks}, 1, failed))
+    if (!tc_run<G>(px, TcGemm{Q::kColAF, Q::KV, aflo, bop, Q::KV / 4 * core, sbo_v2, tc::idesc(128, G * h8), 2, ks}, 1,
+                   failed))
         return pix_nan(g);
     // D' = Mt + scale_u R in the chain's table D slots; this thread's lane (p, vi), its
     // chain's columns u
@@ -363,17 +381,17 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
 
 // A group whose chain has no further evaluations (all threads of the group): raise
 // its done flag, then join the other group's evaluations until both are done.
-template <int NC>
+template <int NC, int G>
 __device__ void pix_drain(const FitParams &P, const GalCtx &gc, const SmemView &sm, int gal, float4 *xph,
                           const float vcol[NC])
 {
-    const PixTc px = pix_tc_view(sm.kxr, P.h_max, P.npad, P.max_side);
+    const PixTc px = pix_tc_view<G>(sm.kxr, P.h_max, P.npad, P.max_side);
     if ((threadIdx.x & 127) == 0) px.done[threadIdx.x >> 7] = 1;
     const float th[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // any finite point: the results are not used
     float g[6];
     for (;;) {
         bool all = false;
-        eval_pix<NC>(P, gc, sm, gal, xph, vcol, th, g, false, &all);
+        eval_pix<NC, G>(P, gc, sm, gal, xph, vcol, th, g, false, &all);
         if (all) break;
     }
 }

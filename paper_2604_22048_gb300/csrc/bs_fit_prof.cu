@@ -23,20 +23,22 @@ FitKernel prof_kernel(int max_side)
     }
 }
 
-// Per-pixel weights (profile 3), exponential: stamps of at most 63 px, two chains
-// per CTA of eight warps, the transforms on the tensor cores.
-FitKernel pix_kernel(int max_side)
-{
-    return max_side <= 31 ? fit_kernel_pix<1> : fit_kernel_pix<2>;
-}
+// Per-pixel weights (profile 3), exponential: stamps of at most 63 px, two or four chains
+// per CTA, the transforms on the tensor cores.
+bool pix_quad(int max_side, int n_chains) { return n_chains == 4 && max_side <= kPixQuadSide; }
 
-constexpr int kPixThreads = tc::kThreads;
+FitKernel pix_kernel(int max_side, bool quad)
+{
+    if (quad) return max_side <= 31 ? fit_kernel_pix<1, 5> : fit_kernel_pix<2, 5>;
+    return max_side <= 31 ? fit_kernel_pix<1, 3> : fit_kernel_pix<2, 3>;
+}
+static_assert(tc::Geo<4>::KV == kPixQuadSide + 1, "the four-chain layout's largest side");
 
 bool is_pix(int profile) { return profile == 3; }
 
-FitKernel kernel_for(int profile, int max_side)
+FitKernel kernel_for(int profile, int max_side, int n_chains)
 {
-    if (profile == 3) return pix_kernel(max_side);
+    if (profile == 3) return pix_kernel(max_side, pix_quad(max_side, n_chains));
     if (profile == 4) return fit_kernel_dense<1>;   // a dense covariance: at most 31 px
     return profile == BS_PROFILE_SPERGEL ? prof_kernel<1>(max_side) : prof_kernel<2>(max_side);
 }
@@ -66,7 +68,8 @@ size_t smem_for(int profile, int max_side, int n_chains)
 {
     if (is_pix(profile)) {
         const int h = (max_side + 1) / 2, npad = 32 * ((max_side + 31) / 32);
-        return fit_smem_bytes(max_side, 2) + 16 + pix_tc_bytes(max_side, h, npad);
+        return pix_quad(max_side, n_chains) ? fit_smem_bytes(max_side, 4) + 16 + pix_tc_bytes<4>(max_side, h, npad)
+                                            : fit_smem_bytes(max_side, 2) + 16 + pix_tc_bytes<2>(max_side, h, npad);
     }
     size_t b = fit_smem_bytes(max_side, n_chains);
     if (profile == 4) {
@@ -76,9 +79,9 @@ size_t smem_for(int profile, int max_side, int n_chains)
     return b;
 }
 
-int threads_for(int profile, int n_chains)
+int threads_for(int profile, int n_chains, int max_side)
 {
-    return is_pix(profile) ? kPixThreads : profile == 4 ? 32 * kDenseWarps : 32 * n_chains;
+    return is_pix(profile) ? 128 * (pix_quad(max_side, n_chains) ? 4 : 2) : profile == 4 ? 32 * kDenseWarps : 32 * n_chains;
 }
 
 // K_mu(x) = int_0^inf exp(-x cosh t) cosh(mu t) dt by the trapezoidal rule
@@ -119,9 +122,9 @@ int fit_blocks_per_sm_profile(int profile, int n_chains, int max_side)
 {
     int nb = 0;
     const size_t smem = smem_for(profile, max_side, n_chains);
-    FitKernel k = kernel_for(profile, max_side);
+    FitKernel k = kernel_for(profile, max_side, n_chains);
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, threads_for(profile, n_chains), smem) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, threads_for(profile, n_chains, max_side), smem) != cudaSuccess)
         return 1;
     return nb > 0 ? nb : 1;
 }
@@ -130,10 +133,10 @@ cudaError_t launch_fit_profile(const FitParams &p, int grid, cudaStream_t stream
 {
     const int cc = cta_chains(p);
     const size_t smem = smem_for(p.profile, p.max_side, cc);
-    FitKernel k = kernel_for(p.profile, p.max_side);
+    FitKernel k = kernel_for(p.profile, p.max_side, cc);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<grid, threads_for(p.profile, cc), smem, stream>>>(p);
+    k<<<grid, threads_for(p.profile, cc, p.max_side), smem, stream>>>(p);
     bs::count_launches(1);
     return cudaGetLastError();
 }
@@ -141,15 +144,15 @@ cudaError_t launch_fit_profile(const FitParams &p, int grid, cudaStream_t stream
 cudaError_t launch_logpost_points_profile(const FitParams &p, int n_points, const int32_t *gal_index,
                                           const float *theta, double *logp, float *grad, cudaStream_t stream)
 {
-    const size_t smem = smem_for(p.profile, p.max_side, kPointWarps);
+    const size_t smem = smem_for(p.profile, p.max_side, is_pix(p.profile) ? 2 : kPointWarps);
     PointsKernel k = points_for(p.profile, p.max_side);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (is_pix(p.profile)) {
         const int grid = n_points < 4096 ? n_points : 4096;
-        k<<<grid, kPixThreads, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
+        k<<<grid, tc::Geo<2>::kThreads, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
     } else {
-        k<<<n_points, threads_for(p.profile, kPointWarps), smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
+        k<<<n_points, threads_for(p.profile, kPointWarps, p.max_side), smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
     }
     bs::count_launches(1);
     return cudaGetLastError();

@@ -10,6 +10,7 @@ namespace bs {
 
 constexpr int kMaxChains = 8;
 constexpr int kMaxWindows = 24;
+constexpr int kPixQuadSide = 47;    // largest stamp of the pixel-weight path with four chains per CTA
 constexpr int kDenseMaxSide = 31;   // largest stamp with a general pixel covariance
 
 // Everything one fit launch needs, filled by the C-ABI layer.
@@ -80,11 +81,11 @@ struct FitParams {
 
 // Chains (warps) of one CTA of a fit launch.
 __host__ __device__ inline int cta_chains(const FitParams &p) { return p.cpc > 0 ? p.cpc : p.n_chains; }
-// CTAs a galaxy's chains are split over (the pixel-weight path: pairs of chains, the
-// last one alone for an odd count).
+// CTAs a galaxy's chains are split over (the pixel-weight path: two or four chains each, the
+// last one what is left).
 __host__ __device__ inline int cta_groups(const FitParams &p)
 {
-    return p.profile == 3 ? (p.n_chains + 1) / 2 : p.n_chains / cta_chains(p);
+    return (p.n_chains + cta_chains(p) - 1) / cta_chains(p);
 }
 
 // Shared memory bytes per CTA for a given max stamp side and chains per galaxy.

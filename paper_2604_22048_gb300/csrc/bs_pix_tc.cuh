@@ -28,14 +28,14 @@
 // (3xTF32): the operand rounding of plain TF32 would miss the log-likelihood
 // tolerance by a factor of several.
 //
-// One CTA of eight warps runs two chains in lockstep: warps 0-3 the first, 4-7 the
-// second (each group's warps run the same chain logic and make the same decisions,
-// from the same numbers).  Every step of a chain is one evaluation, so the two meet
-// at each one; every product carries both chains' data (B rows (chain, u) or (chain,
-// iy)), so each barrier and MMA round trip serves two evaluations.  Thread t reads TMEM
+// One CTA runs two chains (or four, where the layout of sides up to 47 px fits: Geo) in lockstep:
+// warps 0-3 the first, 4-7 the second, ... (each group's warps run the same chain logic and
+// make the same decisions, from the same numbers).  Every step of a chain is one
+// evaluation, so the chains meet at each one; every product carries all chains' data (B rows
+// (chain, u) or (chain, iy)), so each barrier and MMA round trip serves them all.  Thread t reads TMEM
 // lane 32 (w mod 4) + (t mod 32) and its chain's columns (w / 4), the group's warps
 // split the spectral gradient pass by rows, and one lane of the first warp issues the MMAs.  A chain that
-// has finished, or has no evaluation at a step, joins with a skip flag until both are
+// has finished, or has no evaluation at a step, joins with a skip flag until all are
 // done.  Each evaluation commits four MMA groups to one mbarrier, so the parities it
 // waits on are 0, 1, 0, 1 in every evaluation.  A wait gives up after two seconds: the
 // CTA then marks its galaxy (status 4), issues no further MMA, and its evaluations
@@ -50,7 +50,6 @@ namespace tc {
 
 constexpr int kLboB = 144;                     // data operands: 16-byte pad per core matrix (column
                                                // stores of a warp fall in 32 distinct banks)
-constexpr int kBopFloats = 16 * 16 * (kLboB / 4);   // one data operand: 128 rows x 64 K or 64 x 128
 constexpr uint64_t kWaitNs = 2000000000ull;    // limit of one MMA wait
 
 // Element (row, k) of an operand of kt K-elements per row (no swizzle, K-major):
@@ -185,13 +184,27 @@ __device__ __forceinline__ void split_store4(float *hi, float *lo, int i, float 
     *reinterpret_cast<float4 *>(lo + i) = l;
 }
 
-// TMEM columns of the CTA: the accumulator, then the A operands (high, low).
 constexpr int kTmemCols = 512;
-constexpr int kColAF = 128;                    // [[C, -S], [S, C]], 128 columns: K (re, v | im, v)
-constexpr int kColAFlo = 256;
-constexpr int kColA2 = 384;                    // the complex-to-real constant, 64 columns: K (re, u | im, u)
-constexpr int kColA2lo = 448;
-constexpr int kThreads = 256;                  // eight warps: lane quadrant w % 4, chain w / 4
+
+// A CTA of G chains (2 or 4): four warps per chain (lane quadrant w % 4, chain w / 4), sides
+// up to KV - 1.  TMEM columns: the accumulator, then the A operands (high, low).
+template <int G>
+struct Geo {
+    static constexpr int kThreads = 128 * G;
+    static constexpr int KV = G == 2 ? 64 : 48;     // K elements over v, ix or iy
+    static constexpr int KU = KV / 2;               // and over u
+    // one data operand: G KU rows x 2 KV K, or G KV rows x 2 KU or KV
+    static constexpr int kBopFloats = G * KU * KV / 16 * (kLboB / 4);
+    static constexpr int kColAF = G * KV;           // [[C, -S], [S, C]], 2 KV columns: K (re, v | im, v)
+    static constexpr int kColAFlo = kColAF + 2 * KV;
+    static constexpr int kColA2 = kColAFlo + 2 * KV;    // the complex-to-real constant, 2 KU columns: K (re, u | im, u)
+    static constexpr int kColA2lo = kColA2 + 2 * KU;
+    // floats of the shared region before the data operand: chi (8 G), barrier (2), TMEM address, abort,
+    // done flags (G), from kGsum the gradient sums (24 G)
+    static constexpr int kGsum = (9 * G + 4 + 3) & ~3;
+    static constexpr int kBop = kGsum + 24 * G;
+    static_assert(kColA2lo + 2 * KU <= kTmemCols && G * KV <= 256 && kBop % 4 == 0, "tensor memory");
+};
 
 // One lane of a converged warp: 1 there, 0 in the others.
 __device__ __forceinline__ uint32_t elect_one()
@@ -225,42 +238,44 @@ __device__ __forceinline__ void st8(uint32_t taddr, const float (&v)[8])
 
 // Shared memory of the tensor-core pixel path, after the (kx, kx^2) table.
 struct PixTc {
-    double *chi;      // [8] per-warp partial chi^2 of the evaluation
+    double *chi;      // [4 G] per-warp partial chi^2 of the evaluation
     uint64_t *bar;    // MMA completion barrier
     uint32_t *tmem;   // TMEM base of the CTA (512 columns)
     int *abort;       // 2 + the pending parity once a wait gave up, else 0
-    int *done;        // [2] a chain group has no more evaluations
-    float *gsum;      // [2][4][6] per chain and warp of its group: the six gradient sums
+    int *done;        // [G] a chain group has no more evaluations
+    float *gsum;      // [G][4][6] per chain and warp of its group: the six gradient sums
     float *bop;       // [2][kBopFloats] the data operand of the current transform, high then low
-    float *tab1;      // [h_max][3 npad] the second chain's table (the first's is the staged one)
+    float *tab1;      // [G - 1][h_max][3 npad] the further chains' tables (the first's is the staged one)
     float *dimg;      // [max_side^2] the stamp
     float *wimg;      // [max_side^2] the weights
 };
 
 __host__ __device__ __forceinline__ int pix_tc_img_floats(int max_side) { return (max_side * max_side + 3) & ~3; }
 
-// Floats of the region: 16 (chi) + 2 (barrier) + 1 (TMEM address) + 1 (abort) + 2
-// (done) + 2 (pad) + 48 (gradient sums) + operand + table + two images.
+template <int G>
 __host__ __device__ __forceinline__ size_t pix_tc_bytes(int max_side, int h_max, int npad)
 {
-    return ((size_t)72 + 2 * tc::kBopFloats + (size_t)h_max * 3 * npad + 2 * (size_t)pix_tc_img_floats(max_side)) *
+    using Q = tc::Geo<G>;
+    return ((size_t)Q::kBop + 2 * Q::kBopFloats + (size_t)(G - 1) * h_max * 3 * npad + 2 * (size_t)pix_tc_img_floats(max_side)) *
            sizeof(float);
 }
 
 // The region starts after the (kx, kx^2) table (h_max + 1 float2), 16-byte aligned.
+template <int G>
 __device__ __forceinline__ PixTc pix_tc_view(float2 *kxr, int h_max, int npad, int max_side)
 {
     float *base = reinterpret_cast<float *>(kxr + ((h_max + 2) & ~1));
+    using Q = tc::Geo<G>;
     PixTc v;
     v.chi = reinterpret_cast<double *>(base);
-    v.bar = reinterpret_cast<uint64_t *>(base + 16);
-    v.tmem = reinterpret_cast<uint32_t *>(base + 18);
-    v.abort = reinterpret_cast<int *>(base + 19);
-    v.done = reinterpret_cast<int *>(base + 20);
-    v.gsum = base + 24;
-    v.bop = base + 72;
-    v.tab1 = v.bop + 2 * tc::kBopFloats;
-    v.dimg = v.tab1 + (size_t)h_max * 3 * npad;
+    v.bar = reinterpret_cast<uint64_t *>(base + 8 * G);
+    v.tmem = reinterpret_cast<uint32_t *>(base + 8 * G + 2);
+    v.abort = reinterpret_cast<int *>(base + 8 * G + 3);
+    v.done = reinterpret_cast<int *>(base + 8 * G + 4);
+    v.gsum = base + Q::kGsum;
+    v.bop = base + Q::kBop;
+    v.tab1 = v.bop + 2 * Q::kBopFloats;
+    v.dimg = v.tab1 + (size_t)(G - 1) * h_max * 3 * npad;
     v.wimg = v.dimg + pix_tc_img_floats(max_side);
     return v;
 }
