@@ -308,10 +308,10 @@ static int dense_chains_per_cta(int n_gal, int n_chains, int sms)
 }
 
 // Chains per CTA of a pixel-weight fit, one CTA per SM.  A wave of four-chain CTAs takes 1.64 (31 px)
-// to 1.87 (41 px) times a wave of two-chain CTAs (the products and barriers are shared by
-// more chains), so four are taken where they make the waves shorter by more than that, as a
-// last wave that is not full can prevent; 400 galaxies of 41 px, 4 chains: 90.3 ms in six waves of
-// two, 84.3 ms in three waves of four.
+// to 1.82 (47 px) times a wave of two-chain CTAs (the products and barriers are shared by
+// more chains: 152 galaxies of 41 px, 4 chains x 70 iterations, 8.98 ms against two waves of
+// 5.11), so four are taken where they make the waves fewer by more than that, as a last wave
+// that is not full can prevent.
 static int pixel_chains_per_cta(int n_gal, int n_chains, int max_side, int sms)
 {
     if (max_side > bs::kPixQuadSide || n_chains < 3) return 2;

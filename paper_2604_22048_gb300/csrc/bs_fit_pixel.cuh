@@ -209,8 +209,8 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
     {
         const int vi = tg & 63, u0 = tg >> 6;
         const bool col = vi < N;
-        int ox = 0, oy = 0, ot = 0;
-        if (col) slot_offsets(npad, vi >> 5, vi & 31, ox, oy, ot);
+        int ox, oy, ot;
+        slot_offsets(npad, col ? vi >> 5 : 0, col ? vi & 31 : 0, ox, oy, ot);
         const float ky = (float)(vi - c) * gc.dk;
         const float cst = fmaf(be * ky, ky, 1.0f), gky = ga * ky;
         float Xs, Xc, sy, cy;
@@ -223,24 +223,30 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
 #pragma unroll 1
         for (int ug = 0; ug < h8; ug += 8) {
             const int e0 = eo + ((h8 * grp + ug) >> 3) * (Q::KV / 2) * kLb;
+            // every load of the four rows before the first store, which the compiler cannot move them over
+            float T[4], kx[4];
+            float2 X[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int u = ug + u0 + 2 * j, uc = min(u, H - 1);
+                T[j] = tab[uc * rowf + ot];
+                kx[j] = sm.kxr[uc].x;
+                X[j] = make_float2(__shfl_sync(BS_FULL_MASK, Xc, u), __shfl_sync(BS_FULL_MASK, Xs, u));
+            }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int u = ug + u0 + 2 * j;
-                const float2 X = make_float2(__shfl_sync(BS_FULL_MASK, Xc, u), __shfl_sync(BS_FULL_MASK, Xs, u));
-                float Mr = 0.f, Mi = 0.f;
-                if (col && u < H) {
-                    float *row = tab + u * rowf;
-                    const float kx = sm.kxr[u].x;
-                    const float s = fmaf(fmaf(al, kx, gky), kx, cst);
-                    const float rs = rsqrtf(s);
-                    const float A = row[ot] * rs * rs * rs;
-                    const float mr = A * (X.x * Y.x - X.y * Y.y), mi = A * (X.x * Y.y + X.y * Y.x);
-                    row[ox] = mr;
-                    row[oy] = mi;
-                    const float inv_scale = u == 0 ? sN : sN2;
-                    Mr = mr * inv_scale;
-                    Mi = mi * inv_scale;
+                const float s = fmaf(fmaf(al, kx[j], gky), kx[j], cst);
+                const float rs = rsqrtf(s);
+                const float A = T[j] * rs * rs * rs;
+                const float mr = A * (X[j].x * Y.x - X[j].y * Y.y), mi = A * (X[j].x * Y.y + X[j].y * Y.x);
+                const float inv_scale = u == 0 ? sN : sN2;
+                const bool in = col && u < H;
+                if (in) {
+                    tab[u * rowf + ox] = mr;
+                    tab[u * rowf + oy] = mi;
                 }
+                const float Mr = in ? mr * inv_scale : 0.f, Mi = in ? mi * inv_scale : 0.f;
                 if (Q::KV == 64 || vi < Q::KV) {
                     tc::split_store(bh, bl, e0 + 8 * j, Mr);
                     tc::split_store(bh, bl, e0 + 8 * j + (Q::KV / 4) * kLb, Mi);   // K index KV + vi
@@ -282,18 +288,31 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
     {
         const int ix = L & 63;
         const int g0 = (L >> 6) ? (ks + 1) >> 1 : 0, ng = (L >> 6) ? ks >> 1 : (ks + 1) >> 1;
-        float m[32];
-        tc::ld8n(tl + n8 * grp + 8 * g0, ng, m);
         const float *dp = px.dimg + 8 * g0 * N + ix, *wp = px.wimg + 8 * g0 * N + ix;
-        const int e0 = (ix >> 2) * kLb + (ix & 3) + (ks * grp + g0) * (Q::KV / 4) * kLb;
+        int e0 = (ix >> 2) * kLb + (ix & 3) + (ks * grp + g0) * (Q::KV / 4) * kLb;
+        // eight rows at a time, their loads before the first store.  Here and in the other steps between
+        // products the warps waited for chains of shared-memory loads, each behind the last
+        // element's stores, which the compiler must not move it over: a round of two chains at 41 px
+        // took 17,800 cycles, 15,200 with the loads of a few elements ahead (four chains 10.6 -> 9.0
+        // ms a launch of one wave; fully unrolled groups took 12.2 ms for want of registers)
+#pragma unroll 1
+        for (int q = 0; q < ng; ++q) {
+            float m[32], d[8], w[8];
+            tc::ld8n(tl + n8 * grp + 8 * (g0 + q), 1, m);
+            const int left = ix < N ? N - 8 * (g0 + q) : 0;
 #pragma unroll
-        for (int t = 0; t < 32; ++t) {
-            if (t < 8 * ng) {
-                float r = 0.f;
-                if (ix < N && 8 * g0 + t < N) r = wp[t * N] * (dp[t * N] - m[t]);
-                if (Q::KV == 64 || ix < Q::KV)
-                    tc::split_store(bh, bl, e0 + (t >> 3) * (Q::KV / 4) * kLb + ((t & 7) << 2), r);
+            for (int t = 0; t < 8; ++t) {
+                d[t] = t < left ? dp[t * N] : 0.f;
+                w[t] = t < left ? wp[t * N] : 0.f;
             }
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const float r = t < left ? w[t] * (d[t] - m[t]) : 0.f;
+                if (Q::KV == 64 || ix < Q::KV) tc::split_store(bh, bl, e0 + (t << 2), r);
+            }
+            dp += 8 * N;
+            wp += 8 * N;
+            e0 += Q::KV / 4 * kLb;
         }
     }
     // chi^2 (warps 0 and 1 of the group, all rows again: one evaluation of a trajectory):
@@ -305,13 +324,19 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
             for (int g8 = 0; g8 < ks; ++g8) {
                 float m[32];
                 tc::ld8n(tl + n8 * grp + 8 * g8, 1, m);
+                float x[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    const bool in = L < N && 8 * g8 + t < N;
+                    const int e = in ? (8 * g8 + t) * N + L : 0;
+                    const float res = px.dimg[e] - m[t];
+                    x[t] = px.wimg[e] * res * res;
+                }
 #pragma unroll
                 for (int t = 0; t < 8; ++t) {
                     if (L < N && 8 * g8 + t < N) {
-                        const int e = (8 * g8 + t) * N + L;
-                        const float res = px.dimg[e] - m[t];
                         float t_hi, t_lo;
-                        two_sum(c_hi, px.wimg[e] * res * res, t_hi, t_lo);
+                        two_sum(c_hi, x[t], t_hi, t_lo);
                         c_hi = t_hi;
                         c_lo += t_lo;
                     }
@@ -357,10 +382,16 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
             const int os = p ? oy : ox;
             const float sg = p ? -gc.invN : gc.invN;
 #pragma unroll
-            for (int u = 0; u < 32; ++u) {
-                if (u < H) {
-                    float *slot = tab + (size_t)u * rowf + os;
-                    *slot = fmaf((u ? sqrt2 : 1.0f) * sg, v[u], *slot);
+            for (int u0 = 0; u0 < 32; u0 += 8) {
+                if (u0 < H) {
+                    float o[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (u0 + j < H) o[j] = tab[(u0 + j) * rowf + os];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (u0 + j < H)
+                            tab[(u0 + j) * rowf + os] = fmaf((u0 + j ? sqrt2 : 1.0f) * sg, v[u0 + j], o[j]);
                 }
             }
         }
