@@ -294,7 +294,7 @@ __device__ double eval_pix(const FitParams &P, const GalCtx &gc, const SmemView 
         // products the warps waited for chains of shared-memory loads, each behind the last
         // element's stores, which the compiler must not move it over: a round of two chains at 41 px
         // took 17,800 cycles, 15,200 with the loads of a few elements ahead (four chains 10.6 -> 9.0
-        // ms a launch of one wave; fully unrolled groups took 12.2 ms for want of registers)
+        // ms a launch of one wave; with the groups unrolled 12.2 ms, for want of registers)
 #pragma unroll 1
         for (int q = 0; q < ng; ++q) {
             float m[32], d[8], w[8];
@@ -444,7 +444,9 @@ __device__ void pix_drain(const FitParams &P, const GalCtx &gc, const SmemView &
 // from L2): 32 rows of loads are in flight per warp.
 // 64 galaxies of 21 px, 4 chains x (100 + 100), L <= 8: 332 ms with a warp per chain that
 // evaluated on its own (the product waiting for each row of P, transforms on 11 to 21 of 32
-// lanes), 23.8 ms now, the same draws bit for bit; issue 1.7 per cycle on the 64 SMs in use.
+// lanes), 23.8 ms on 64 SMs with all chains of a galaxy in one CTA, 18.2 ms with two per CTA on
+// 128, the same draws bit for bit.  The L1 holds part of P between rounds: its first rows kept
+// in shared memory instead came out the same or slower (21 px 18.3 -> 19.4 ms, 13 px 8.56 -> 8.56).
 //
 // After the shared region, in floats: the twiddles exp(+2 pi i m / N) (max_side float2),
 // the chains' requests, the residual images of the four chain slots interleaved (max_side^2

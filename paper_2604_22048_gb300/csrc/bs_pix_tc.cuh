@@ -21,8 +21,8 @@
 //        imaginary output is -Q_i: conj Q);
 //   (4)  conj R = transform (1) of conj Q.
 // These A operands live in tensor memory (lane = row, column = K index), high and
-// low TF32 parts: 384 of the CTA's 512 columns, the accumulator the other 128.  Each
-// transform is a tcgen05.mma of kind::tf32 (M = 128, N = 64 or 128, K = 8 per
+// low TF32 parts, beside the accumulator (Geo).  Each transform is a tcgen05.mma of
+// kind::tf32 (M = 128, N the rows of all chains rounded up to 8 each, K = 8 per
 // instruction; B, the data, in shared memory without swizzle) in three terms,
 // A_hi B_hi + A_hi B_lo + A_lo B_hi with x = hi + lo split by round-to-nearest TF32
 // (3xTF32): the operand rounding of plain TF32 would miss the log-likelihood
