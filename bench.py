@@ -211,13 +211,13 @@ def flops_per_eval(N):
 # to that file the traffic is reported as null until the next capture.
 CAPTURED_TRAFFIC = {
     # one galaxy of the plain workload (53x53, 4 chains x (200 + 300) draws), from a one-pass
-    # capture of the full 10,000-galaxy launch: (133,567,488 + 292,933,632) B / 10,000
+    # capture of the full 10,000-galaxy launch: (135,008,768 + 293,555,968) B / 10,000
     "fit": ("paper_2604_22048_gb300/csrc/bs_fit_impl.cuh",
-            "e9f67fed04fb016f403a11a2e5d9ea4f97cb15a9d1a18d7f51d4a859bae988e2", 42650.1,
+            "303672ef0b44afd67b5e4b2b7498b86e6d0e16a4a25a910ae55fcb27166eda58", 42856.5,
             {"side": 53, "chains": 4, "n_warmup": 200, "n_samples": 300}),
-    # one interim sample of the shear workload: (483,096,576 + 3,097,088) B / (200,000 x 300)
+    # one interim sample of the shear workload: (483,382,528 + 457,472) B / (200,000 x 300)
     "shear": ("paper_2604_22048_gb300/csrc/bs_shear.cu",
-              "5e102b705e1ea3da5d060dc3ac880c763355d9247f1fc83031b22cb8fe2683d7", 8.1032, {}),
+              "65381469d210009cd3a12dbab856cfd3bb88604758825b9a003dd9fdee3e818a", 8.0640, {}),
 }
 
 
