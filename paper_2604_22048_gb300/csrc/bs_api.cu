@@ -235,13 +235,25 @@ static bs_status fill_fit_params(const bs_fit_args *a, bs::FitParams &p, const c
                         "%s: chains_per_cta needs the exponential profile, one exposure and white noise", who);
         p.cpc = a->chains_per_cta;
     }
-    if (p.profile == 3) p.cpc = 2;   // the pixel-weight path: two chains per CTA (bs_fit_galaxies may take four)
+    if (p.profile == 3) p.cpc = 2;   // the pixel-weight path: two chains per CTA (fits and plans may take four)
     return BS_OK;
 }
 
 }  // extern "C"
 
 namespace bs {
+
+// Chains per CTA of a pixel-weight fit, one CTA per SM.  A wave of four-chain CTAs takes 1.64 (31 px)
+// to 1.82 (47 px) times a wave of two-chain CTAs (the products and barriers are shared by
+// more chains: 152 galaxies of 41 px, 4 chains x 70 iterations, 8.98 ms against two waves of
+// 5.11), so four are taken where they make the waves fewer by more than that, as a last wave
+// that is not full can prevent.
+int pixel_chains_per_cta(int n_gal, int n_chains, int max_side, int sms)
+{
+    if (max_side > kPixQuadSide || n_chains < 3) return 2;
+    auto waves = [&](int cc) { return ((long long)n_gal * ((n_chains + cc - 1) / cc) + sms - 1) / sms; };
+    return 19 * waves(4) < 10 * waves(2) ? 4 : 2;
+}
 
 // Validate a fit request and fill every launch parameter except the
 // scheduling fields (work list, counter).
@@ -307,18 +319,6 @@ static int dense_chains_per_cta(int n_gal, int n_chains, int sms)
     return cc;
 }
 
-// Chains per CTA of a pixel-weight fit, one CTA per SM.  A wave of four-chain CTAs takes 1.64 (31 px)
-// to 1.82 (47 px) times a wave of two-chain CTAs (the products and barriers are shared by
-// more chains: 152 galaxies of 41 px, 4 chains x 70 iterations, 8.98 ms against two waves of
-// 5.11), so four are taken where they make the waves fewer by more than that, as a last wave
-// that is not full can prevent.
-static int pixel_chains_per_cta(int n_gal, int n_chains, int max_side, int sms)
-{
-    if (max_side > bs::kPixQuadSide || n_chains < 3) return 2;
-    auto waves = [&](int cc) { return ((long long)n_gal * ((n_chains + cc - 1) / cc) + sms - 1) / sms; };
-    return 19 * waves(4) < 10 * waves(2) ? 4 : 2;
-}
-
 bs_status bs_fit_galaxies(const bs_fit_args *a, const bs_fit_out *o, void *workspace,
                           size_t workspace_bytes, void *stream)
 {
@@ -342,7 +342,7 @@ bs_status bs_fit_galaxies(const bs_fit_args *a, const bs_fit_out *o, void *works
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (p.profile == 4) p.cpc = dense_chains_per_cta(a->n_gal, p.n_chains, sms);
-    if (p.profile == 3) p.cpc = pixel_chains_per_cta(a->n_gal, p.n_chains, p.max_side, sms);
+    if (p.profile == 3) p.cpc = bs::pixel_chains_per_cta(a->n_gal, p.n_chains, p.max_side, sms);
     const int per_sm = bs::fit_blocks_per_sm(bs::cta_chains(p), a->max_side, p.regs, p.profile);
     long long grid = (long long)sms * per_sm;
     const long long items = (long long)a->n_gal * bs::cta_groups(p);

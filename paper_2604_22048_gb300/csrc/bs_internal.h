@@ -88,6 +88,8 @@ __host__ __device__ inline int cta_groups(const FitParams &p)
     return (p.n_chains + cta_chains(p) - 1) / cta_chains(p);
 }
 
+int pixel_chains_per_cta(int n_gal, int n_chains, int max_side, int sms);
+
 // Shared memory bytes per CTA for a given max stamp side and chains per galaxy.
 size_t fit_smem_bytes(int max_side, int n_chains);
 // Launch helpers implemented in the .cu files.

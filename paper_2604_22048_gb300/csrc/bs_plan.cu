@@ -122,7 +122,9 @@ cudaError_t autotune(bs_fit_plan_s *pl, int sms)
         for (int r : kRegVariants) waves = std::max(waves, bs::fit_blocks_per_sm(L.p.n_chains, L.p.max_side, r, L.p.profile));
         const int n_trial = std::min(L.p.n_work, 2 * sms * waves);
         float best = 0.f;
-        int best_regs = 128, best_cpc = 0;
+        // all of a galaxy's chains; the pixel-weight path's two or four are not the tuner's to choose
+        const int all = L.p.profile == 3 ? L.p.cpc : 0;
+        int best_regs = 128, best_cpc = all;
         // Candidates: the 128-, 96- and 80-register instances, with all of a
         // galaxy's chains in one CTA or half of them (two CTAs per galaxy,
         // each staging it).  All give the same chains bit for bit (the library
@@ -131,19 +133,19 @@ cudaError_t autotune(bs_fit_plan_s *pl, int sms)
         for (int v = 0; v < 3 && e == cudaSuccess; ++v) {
             if (kRegVariants[v] == 96 && L.p.n_chains > 4) continue;   // that instance takes <= 128 threads
             float ms = 0.f;
-            L.p.cpc = 0;
+            L.p.cpc = all;
             e = time_variant(L, kRegVariants[v], n_trial, sms, st, e0, e1, ms);
             L.trial_ms[v] = ms;
             if (e == cudaSuccess && (v == 0 || ms < best)) {
                 best = ms;
                 best_regs = kRegVariants[v];
-                best_cpc = 0;
+                best_cpc = all;
             }
             if (e == cudaSuccess && half_layout_ok(L.p)) {
                 L.p.cpc = L.p.n_chains / 2;
                 e = time_variant(L, kRegVariants[v], n_trial, sms, st, e0, e1, ms);
                 L.trial_half[v] = ms;
-                L.p.cpc = 0;
+                L.p.cpc = all;
                 if (e == cudaSuccess && ms < best) {
                     best = ms;
                     best_regs = kRegVariants[v];
@@ -250,6 +252,7 @@ bs_status plan_create(const bs_fit_args *a, const bs_fit_out *o, const int32_t *
         L.slot_class = c + 1;
         L.trial_ms[0] = L.trial_ms[1] = L.trial_ms[2] = 0.f;
         L.trial_half[0] = L.trial_half[1] = L.trial_half[2] = 0.f;
+        if (L.p.profile == 3) L.p.cpc = bs::pixel_chains_per_cta(count[c], a->n_chains, maxs[c], sms);
         const int per_sm = bs::fit_blocks_per_sm(a->n_chains, maxs[c], L.p.regs, L.p.profile);
         L.grid = std::min(count[c], sms * per_sm);
         pl->launches.push_back(L);
