@@ -776,7 +776,9 @@ class ShearLogLike(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, params, plan: ShearPlan):
-        g1, g2, alpha = params.detach().cpu().double().tolist()
+        x = params.detach().cpu().double()
+        # a vector, or anything whose three rows are numbers (a column)
+        g1, g2, alpha = x.tolist() if x.dim() == 1 else [float(v) for v in x]
         out = torch.from_numpy(plan.loglike(g1, g2, alpha, host=True))
         ctx.save_for_backward(out[1:].clone())
         return out[0].clone()
