@@ -381,8 +381,9 @@ cudaError_t launch_chain_ess(const float *samples, int n_gal, int n_chains, int 
         const int wpc = per_warp > kEssSmemCta / 2 ? 1 : per_warp > kEssSmemCta / 4 ? 2 : 4;
         const bool vec = n_samples % 4 == 0 && (reinterpret_cast<uintptr_t>(samples) & 15) == 0;
         auto kernel = vec ? ess_kernel<true> : ess_kernel<false>;
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)(wpc * per_warp));
+        // the same limit from every call: one that followed the size of the call could be lowered by
+        // another host thread between here and the launch
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEssSmemMax);
         if (e != cudaSuccess) return e;
         const dim3 grid((unsigned)(((long long)n_gal + wpc - 1) / wpc), 6);
         kernel<<<grid, 32 * wpc, wpc * per_warp, stream>>>(samples, n_gal, n_chains, n_samples, ess, rhat);

@@ -36,6 +36,15 @@ PointsKernel points_kernel_for(int max_side) { BS_FIT_NC_SWITCH(logpost_points_k
 
 #undef BS_FIT_NC_SWITCH
 
+// A kernel's limit of dynamic shared memory: that of the largest stamp and chain count, the same
+// from every host thread (a limit that followed each call could be lowered by another thread between the
+// setting and the launch; the occupancy follows what a launch asks for, not the limit).
+cudaError_t allow_smem(const void *kernel)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)fit_smem_bytes(BS_MAX_SIDE, kMaxChains));
+}
+
 }  // namespace
 
 size_t fit_smem_bytes(int max_side, int n_chains)
@@ -52,7 +61,7 @@ int fit_blocks_per_sm(int n_chains, int max_side, int regs, int profile)
     int nb = 0;
     const size_t smem = fit_smem_bytes(max_side, n_chains);
     FitKernel k = fit_kernel_for(max_side, regs, n_chains);
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem((const void *)k);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, 32 * n_chains, smem) != cudaSuccess)
         return 1;
     return nb > 0 ? nb : 1;
@@ -64,7 +73,7 @@ cudaError_t launch_fit(const FitParams &p, int grid, cudaStream_t stream)
     const int cc = cta_chains(p);
     const size_t smem = fit_smem_bytes(p.max_side, cc);
     FitKernel k = fit_kernel_for(p.max_side, p.regs, cc);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void *)k);
     if (e != cudaSuccess) return e;
     k<<<grid, 32 * cc, smem, stream>>>(p);
     bs::count_launches(1);
@@ -78,7 +87,7 @@ cudaError_t launch_logpost_points(const FitParams &p, int n_points, const int32_
     if (p.profile != 0) return launch_logpost_points_profile(p, n_points, gal_index, theta, logp, grad, stream);
     const size_t smem = fit_smem_bytes(p.max_side, kPointWarps);
     PointsKernel k = points_kernel_for(p.max_side);
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem((const void *)k);
     if (e != cudaSuccess) return e;
     k<<<n_points, 32 * kPointWarps, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
     bs::count_launches(1);

@@ -79,6 +79,16 @@ size_t smem_for(int profile, int max_side, int n_chains)
     return b;
 }
 
+// A kernel's limit of dynamic shared memory: that of the largest stamp and chain count it takes, the
+// same from every host thread (as for the white-noise kernels).
+cudaError_t allow_smem(const void *kernel, int profile, int max_side, int n_chains)
+{
+    const size_t most = is_pix(profile)  ? smem_for(profile, pix_quad(max_side, n_chains) ? kPixQuadSide : 63, n_chains)
+                        : profile == 4 ? smem_for(profile, kDenseMaxSide, kDenseChains)
+                                       : smem_for(profile, BS_MAX_SIDE, kMaxChains);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 int threads_for(int profile, int n_chains, int max_side)
 {
     return is_pix(profile) ? 128 * (pix_quad(max_side, n_chains) ? 4 : 2) : profile == 4 ? 32 * kDenseWarps : 32 * n_chains;
@@ -123,7 +133,7 @@ int fit_blocks_per_sm_profile(int profile, int n_chains, int max_side)
     int nb = 0;
     const size_t smem = smem_for(profile, max_side, n_chains);
     FitKernel k = kernel_for(profile, max_side, n_chains);
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem((const void *)k, profile, max_side, n_chains);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, threads_for(profile, n_chains, max_side), smem) != cudaSuccess)
         return 1;
     return nb > 0 ? nb : 1;
@@ -134,7 +144,7 @@ cudaError_t launch_fit_profile(const FitParams &p, int grid, cudaStream_t stream
     const int cc = cta_chains(p);
     const size_t smem = smem_for(p.profile, p.max_side, cc);
     FitKernel k = kernel_for(p.profile, p.max_side, cc);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void *)k, p.profile, p.max_side, cc);
     if (e != cudaSuccess) return e;
     k<<<grid, threads_for(p.profile, cc, p.max_side), smem, stream>>>(p);
     bs::count_launches(1);
@@ -146,7 +156,7 @@ cudaError_t launch_logpost_points_profile(const FitParams &p, int n_points, cons
 {
     const size_t smem = smem_for(p.profile, p.max_side, is_pix(p.profile) ? 2 : kPointWarps);
     PointsKernel k = points_for(p.profile, p.max_side);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void *)k, p.profile, p.max_side, 2);
     if (e != cudaSuccess) return e;
     if (is_pix(p.profile)) {
         const int grid = n_points < 4096 ? n_points : 4096;

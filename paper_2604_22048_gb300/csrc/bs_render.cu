@@ -316,8 +316,9 @@ static cudaError_t launch_class(int grid, int n, const float *theta, const float
                                 float pixel_scale, float *out, cudaStream_t stream)
 {
     const size_t smem = render_smem_bytes(max_side, RB);
+    // the limit is that of the largest stamp, the same from every host thread
     const cudaError_t e = cudaFuncSetAttribute(render_kernel<NT, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
+                                               (int)render_smem_bytes(BS_MAX_SIDE, RB));
     if (e != cudaSuccess) return e;
     render_kernel<NT, RB><<<grid, NT, smem, stream>>>(n, theta, shear, offsets, side, min_side, max_side, psf, n_psf,
                                                   pixel_scale, out);
