@@ -451,7 +451,7 @@ bs_status bs_shear_loglike(const bs_shear_data *d, double g1, double g2, double 
     bs_status st = bs::shear_prepare(d, g1, g2, alpha, L, add, alpha_scale, "bs_shear_loglike");
     if (st != BS_OK) return st;
     if (!out) return fail(BS_ERR_INVALID_ARG, "bs_shear_loglike: NULL out");
-    const int grid = bs::shear_grid_blocks(), used = bs::shear_grid_for(d->n_gal, d->b != nullptr);
+    const int grid = bs::shear_grid_blocks(), used = bs::shear_grid_for(L);
     const size_t need = (size_t)(grid * 4 + 4) * sizeof(double);
     if (!workspace || workspace_bytes < need)
         return fail(BS_ERR_OUT_OF_MEMORY, "bs_shear_loglike: workspace of %zu bytes needed", need);

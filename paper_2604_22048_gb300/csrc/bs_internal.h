@@ -146,9 +146,9 @@ struct ShearFullLaunch {
 constexpr int kShearFullOut = 9;   // value, d/d(g1, g2, sigma_e, mu_f, sigma_f, a_f, mu_s, sigma_s)
 
 // CTAs of a one-point pass that fill the GPU (the size of the workspace), and of a pass
-// over n_gal galaxies: no more than one per 32 of them.
+// over s.n_gal galaxies: no more than one per 32 of them.
 int shear_grid_blocks();
-int shear_grid_for(long long n_gal, bool has_b);
+int shear_grid_for(const ShearLaunch &s);
 double shear_weight_total(const bs_shear_data *d);
 // Several (g1, g2, alpha) points per pass over the samples (no b).
 constexpr int kMultiPoints = 4;

@@ -77,7 +77,7 @@ extern "C" bs_status bs_shear_loglike_noalloc(const bs_shear_data *data, double 
                              "bs_shear_loglike_noalloc: this device needs %d partial slots, the static "
                              "scratch holds %d; use bs_shear_loglike with a workspace",
                              grid, kNoAllocBlocks);
-    const int used = bs::shear_grid_for(data->n_gal, data->b != nullptr);
+    const int used = bs::shear_grid_for(L);
     double *scratch = nullptr;
     st = scratch_for_current_device(&scratch);
     if (st != BS_OK) return st;

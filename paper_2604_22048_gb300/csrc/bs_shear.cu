@@ -27,6 +27,7 @@
 // accumulated in FP64 and written as per-block partials; a one-block kernel
 // sums the partials in a fixed order (deterministic) and adds the
 // per-galaxy constants.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(kShearThreads, 3) shear_kernel(const __grid_co
     const unsigned gmask = 0xFFu << (lane & ~(kGroup - 1));
     const long long group = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kGroup;
     const long long ngroups = (long long)gridDim.x * blockDim.x / kGroup;
-    const ShearConst &c = s.c;
+    const ShearConst c = s.c;      // (a copy: read through a reference the constants cost 116 bytes of spills, not 52)
     const int K = s.K;
     double acc = 0.0;
 
@@ -1091,35 +1092,46 @@ int resident_grid(GridCache &cache, K kernel, size_t smem)
     return sms * nb;
 }
 
-GridCache g_grid_one, g_grid_b, g_grid_full, g_grid_multi;
+GridCache g_grid_one, g_grid_b, g_grid_scalar, g_grid_scalar_b, g_grid_full, g_grid_multi;
+
+// Whether a one-point pass streams its samples in tiles.
+bool shear_vec(const ShearLaunch &s)
+{
+    return (s.K % 4 == 0) && ((reinterpret_cast<uintptr_t>(s.e1) & 15) == 0) &&
+           ((reinterpret_cast<uintptr_t>(s.e2) & 15) == 0) &&
+           (s.b == nullptr || (reinterpret_cast<uintptr_t>(s.b) & 15) == 0);
+}
+
+// Each pass is sized by its own kernel: with offsets the tile kernel holds 2 CTAs per SM, the scalar
+// one 3 (100,000 x 250 with b: 68-70 us, 78-95 us with 2 per SM).
+int shear_grid_resident(bool has_b, bool vec)
+{
+    if (vec)
+        return has_b ? resident_grid(g_grid_b, shear_kernel_tma<BS_EPRIOR_TRUNC_GAUSS, true>, tma_smem_bytes(true))
+                     : resident_grid(g_grid_one, shear_kernel_tma<BS_EPRIOR_TRUNC_GAUSS, false>, tma_smem_bytes(false));
+    return has_b ? resident_grid(g_grid_scalar_b, shear_kernel<BS_EPRIOR_TRUNC_GAUSS, true>, 0)
+                 : resident_grid(g_grid_scalar, shear_kernel<BS_EPRIOR_TRUNC_GAUSS, false>, 0);
+}
 
 }  // namespace
 
-static int shear_grid_resident(bool has_b)
-{
-    return has_b ? resident_grid(g_grid_b, shear_kernel_tma<BS_EPRIOR_TRUNC_GAUSS, true>, tma_smem_bytes(true))
-                 : resident_grid(g_grid_one, shear_kernel_tma<BS_EPRIOR_TRUNC_GAUSS, false>, tma_smem_bytes(false));
-}
-
 int shear_grid_blocks()
 {
-    const int a = shear_grid_resident(false), b = shear_grid_resident(true);
-    return a > b ? a : b;
+    int most = 0;
+    for (int i = 0; i < 4; ++i) most = std::max(most, shear_grid_resident(i & 1, i & 2));
+    return most;
 }
 
-int shear_grid_for(long long n_gal, bool has_b)
+int shear_grid_for(const ShearLaunch &s)
 {
-    const int full = shear_grid_resident(has_b);
-    const long long want = (n_gal + 31) / 32;
+    const int full = shear_grid_resident(s.b != nullptr, shear_vec(s));
+    const long long want = (s.n_gal + 31) / 32;
     return want < 1 ? 1 : want < full ? (int)want : full;
 }
 
 cudaError_t launch_shear(const ShearLaunch &s, int grid, cudaStream_t stream)
 {
-    const bool vec = (s.K % 4 == 0) && ((reinterpret_cast<uintptr_t>(s.e1) & 15) == 0) &&
-                     ((reinterpret_cast<uintptr_t>(s.e2) & 15) == 0) &&
-                     (s.b == nullptr || (reinterpret_cast<uintptr_t>(s.b) & 15) == 0);
-    const bool hb = s.b != nullptr;
+    const bool vec = shear_vec(s), hb = s.b != nullptr;
     if (s.family == BS_EPRIOR_BA14)
         return hb ? launch_fb<BS_EPRIOR_BA14, true>(s, grid, vec, stream)
                   : launch_fb<BS_EPRIOR_BA14, false>(s, grid, vec, stream);
