@@ -187,7 +187,6 @@ __device__ __forceinline__ void load_chunk(const ShearLaunch &s, long long base,
 // Online log-sum-exp state of one lane (both halves share the reference).
 struct Lse {
     float m;                 // the reference log2 weight
-    float mx;                // largest log2 weight seen (the tile kernels: eval_quad)
     float2 sw, t1, t2, tq;   // t_i: sum of weight rU p eps'_i
     float2 tr;               // sum of weight rU r
 };
@@ -288,27 +287,56 @@ __device__ __forceinline__ void eval_chunk(const ShearConst &c, const Chunk &ch,
     for (int h = 0; h < 2; ++h) add_pair(L, ew[h], e1[h], e2[h], ru[h], pp[h], rr[h], qq[h]);
 }
 
-// Four samples of a galaxy after its first four, against the reference as it stands: no test and
-// no branch, so that consecutive quads and points overlap.  eval_chunk's rescaling (a log
-// weight above the reference by more than 32) is left to the galaxy's end, where the largest log
-// weight seen tells whether it was ever due (lse_jumped) and the lane's samples are then taken
-// again by eval_chunk (replay_lane).  Posterior samples of one galaxy span far less.
-template <int FAMILY, bool HAS_B>
+// Four samples of a galaxy at one of several points, without a branch, so that consecutive quads and
+// points overlap and the time does not depend on the data: the reference moves to the quad's largest
+// log weight where that lies above it by more than 32, as in eval_chunk, and the sums are scaled by
+// the weight between the two, which is 1 in most quads.  Four points of 50,000 x 300: 107-113 us at any
+// alpha; with eval_chunk 107 us at alpha = 0.2 and 123-132 at 0.005, with a lane's samples taken again at
+// the galaxy's end where a weight had jumped 101-104 and 305-315.
+template <int FAMILY>
 __device__ __forceinline__ void eval_quad(const ShearConst &c, const Chunk &ch, Lse &L)
 {
-    const float2 nm = f2(-L.m);
+    float2 x[2], fw[2], ru[2], pp[2], rr[2], qq[2];
     const float2 e1[2] = {make_float2(ch.e1.x, ch.e1.y), make_float2(ch.e1.z, ch.e1.w)};
     const float2 e2[2] = {make_float2(ch.e2.x, ch.e2.y), make_float2(ch.e2.z, ch.e2.w)};
-    const float2 bb[2] = {make_float2(ch.b.x, ch.b.y), make_float2(ch.b.z, ch.b.w)};
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        pair_terms<FAMILY, false>(c, e1[h], e2[h], f2(0.f), x[h], fw[h], ru[h], pp[h], rr[h], qq[h]);
+    const float mloc = fmaxf(fmaxf(x[0].x, x[0].y), fmaxf(x[1].x, x[1].y));
+    const float m = mloc - L.m > 32.0f ? mloc : L.m;
+    const float2 sc = f2(ex2_ftz(L.m - m)), nm = f2(-m);
+    L.m = m;
+    L.sw = mul2(L.sw, sc);
+    L.t1 = mul2(L.t1, sc);
+    L.t2 = mul2(L.t2, sc);
+    L.tq = mul2(L.tq, sc);
+    L.tr = mul2(L.tr, sc);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) add_pair(L, pair_weight(x[h], nm, fw[h]), e1[h], e2[h], ru[h], pp[h], rr[h], qq[h]);
+}
+
+// Four samples of a galaxy against the reference 0 (L.m = 0), for points whose exponents are bounded: an
+// ellipticity in the unit disk has 0 <= Q < 1, so that x lies in (-a2, c0), and with a2 <= kMaxFall
+// (alpha >= 0.095) and c0 <= kMaxRise no weight leaves the range of a float and no reference is needed.
+// Four points of 50,000 x 300: 96-101 us.
+constexpr float kMaxFall = 80.0f, kMaxRise = 32.0f;
+template <int FAMILY>
+__device__ __forceinline__ void eval_bounded(const ShearConst &c, const Chunk &ch, Lse &L)
+{
+    const float2 e1[2] = {make_float2(ch.e1.x, ch.e1.y), make_float2(ch.e1.z, ch.e1.w)};
+    const float2 e2[2] = {make_float2(ch.e2.x, ch.e2.y), make_float2(ch.e2.z, ch.e2.w)};
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         float2 x, fw, ru, pp, rr, qq;
-        pair_terms<FAMILY, HAS_B>(c, e1[h], e2[h], bb[h], x, fw, ru, pp, rr, qq);
-        L.mx = fmaxf(L.mx, fmaxf(x.x, x.y));
-        add_pair(L, pair_weight(x, nm, fw), e1[h], e2[h], ru, pp, rr, qq);
+        pair_terms<FAMILY, false>(c, e1[h], e2[h], f2(0.f), x, fw, ru, pp, rr, qq);
+        add_pair(L, mul2(make_float2(ex2_ftz(x.x), ex2_ftz(x.y)), fw), e1[h], e2[h], ru, pp, rr, qq);
     }
 }
-__device__ __forceinline__ bool lse_jumped(const Lse &L) { return L.mx - L.m > 32.0f; }
+
+// A galaxy's sum of weights outside these did leave that range: samples on or outside the unit circle, which
+// the BA14 weight does not exclude (the truncated Gaussian gives them none), or a shear near 1.
+// Its samples are then taken again with a reference (replay_galaxy).
+constexpr float kLeast = 0x1p-100f, kMost = 0x1p100f;
 
 // Merge the lanes of a galaxy's group and add the galaxy's terms, times the galaxy's weight
 // w[n] (1 when w is NULL; a zero weight drops the galaxy), to the accumulators of the
@@ -316,7 +344,7 @@ __device__ __forceinline__ bool lse_jumped(const Lse &L) { return L.mx - L.m > 3
 // derivative sums, each lane one of them: the FP64 pipe takes 16 cycles an operation for the
 // whole SM, so the four go through it side by side.  (g1, g2) is the shear of the evaluation.
 template <int G = kGroup>
-__device__ __forceinline__ void finish_galaxy(const Lse &L, float g1, float g2, unsigned gmask, int sub,
+__device__ __forceinline__ float finish_galaxy(const Lse &L, float g1, float g2, unsigned gmask, int sub,
                                               const float *w, long long n, double &acc)
 {
     float m = L.m;
@@ -338,9 +366,9 @@ __device__ __forceinline__ void finish_galaxy(const Lse &L, float g1, float g2, 
         tq = tq * ca + oq * cb;
         m = mn;
     }
-    if (sub >= 4) return;
+    if (sub >= 4) return sw;
     const float wf = w ? __ldg(w + n) : 1.0f;
-    if (wf == 0.0f) return;
+    if (wf == 0.0f) return sw;
     if (sw > 0.f) {
         const float inv = 1.0f / sw;
         const float d = sub == 1 ? -2.0f * t1 * inv : sub == 2 ? -2.0f * t2 * inv : tq * inv;
@@ -358,19 +386,18 @@ __device__ __forceinline__ void finish_galaxy(const Lse &L, float g1, float g2, 
     } else if (sub == 0) {
         acc = -INFINITY;
     }
+    return sw;
 }
 
 __device__ __forceinline__ void lse_reset(Lse &L)
 {
     L.m = -1e30f;
-    L.mx = -INFINITY;
     L.sw = L.t1 = L.t2 = L.tq = L.tr = f2(0.f);
 }
 
-// One lane's samples of galaxy n (tile kernels' assignment: 12 of every 48) by eval_chunk, from
-// the start.
-template <int FAMILY, bool HAS_B>
-__device__ __noinline__ Lse replay_lane(const ShearLaunch &s, const ShearConst &c, long long n, int sub);
+// Galaxy n (BA14) at point p by the group's lanes, each its samples of the tile kernels' assignment (12 of
+// every 48) by eval_chunk; this lane's term as finish_galaxy adds it.
+__device__ __noinline__ double replay_galaxy(const ShearMultiLaunch &m, int p, long long n, int sub, unsigned gmask);
 
 // Block reduction of the lanes' FP64 accumulators (quantity = lane of the group of G, the
 // first four) into this block's partials.
@@ -432,7 +459,7 @@ constexpr int kQuads = kChunk / 4;
 
 // ---- Tensor-memory-accelerator tiles (K a multiple of 4, 16-byte aligned rows): a CTA streams
 // tiles of kTileG consecutive galaxies x kTileK samples of e1 and e2 (and b) with 2-D
-// cp.async.bulk.tensor loads into a ring of two or three stages; one thread issues the
+// cp.async.bulk.tensor loads into a ring of three stages; one thread issues the
 // loads of a stage and arms the stage's mbarrier with their byte count, and the
 // others wait on it.  Thread t serves galaxy t / 4 of the tile and its samples
 // [12 (t mod 4), + 12) of each chunk.  Galaxies past n_gal and samples past K arrive zero-filled and
@@ -440,20 +467,20 @@ constexpr int kQuads = kChunk / 4;
 // partials, so that the pass's value is NaN.
 constexpr int kTileG = kShearThreads / kAGroup;   // 64 galaxies per tile
 constexpr int kTileK = kChunk * kAGroup;          // 48 samples per chunk
-// stages of a ring of NV arrays: 72 KB either way, so that 3 CTAs fit an SM
-__host__ __device__ constexpr int tma_stages(int nv) { return nv == 3 ? 2 : 3; }
-// Launch bounds for 2 CTAs per SM, of whose 128 registers the compiler takes 78: 3 CTAs are resident
-// and nothing is rebuilt or spilled.  10^6 x 300 (no b): 446 us so (5.4 TB/s), 472 us bounded
+constexpr int kTmaStages = 3;
+// Launch bounds for 2 CTAs per SM, of whose 128 registers the compiler takes 78: without b 3 CTAs are
+// resident and nothing is rebuilt or spilled.  10^6 x 300: 446 us so (5.4 TB/s), 472 us bounded
 // for 3 CTAs, 476 us before the constants were held, 539 us with 4 stages (2 CTAs fit).
-// With b, 3.6 GB: 612 us; 712 us through per-lane cp.async copies, whose kernel this
-// replaced.  What is left is the memory: the warps' waits find their tile late, and
-// deeper rings per warp or L2 prefetches of whole tiles made the pass slower (516-690 us).
+// With b, 3.6 GB, 2 CTAs fit: 580-590 us; 610 us with two stages, which let 3 in; 709 us through
+// per-lane cp.async copies, whose kernel this replaced.  What is left is the memory: the
+// warps' waits find their tile late, and deeper rings per warp or L2 prefetches of whole tiles made
+// the pass without b slower (516-690 us).
 constexpr int kTmaBlocks = 2;
 constexpr int kTileFloats = kTileG * kTileK;      // one array's box, 12 KB
 
 __host__ __device__ constexpr size_t tma_smem_bytes(bool has_b)
 {
-    return (size_t)tma_stages(has_b ? 3 : 2) * (has_b ? 3 : 2) * kTileFloats * sizeof(float) + 128;   // + alignment of the ring
+    return (size_t)kTmaStages * (has_b ? 3 : 2) * kTileFloats * sizeof(float) + 128;   // + alignment of the ring
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -489,7 +516,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 // stage's previous item has been released.  Every wait gives up after two seconds.
 template <int NV>
 struct TmaRing {
-    static constexpr int kStages = tma_stages(NV);
+    static constexpr int kStages = kTmaStages;
     float *ring;
     uint64_t *full, *empty;
     int cpg, n_items;
@@ -601,7 +628,7 @@ __global__ void __launch_bounds__(kShearThreads, kTmaBlocks)
                      const __grid_constant__ CUtensorMap m2, const __grid_constant__ CUtensorMap m3)
 {
     extern __shared__ __align__(128) unsigned char tma_raw[];
-    constexpr int NV = HAS_B ? 3 : 2, NS = tma_stages(NV);
+    constexpr int NV = HAS_B ? 3 : 2, NS = kTmaStages;
     __shared__ __align__(8) uint64_t full[NS], empty[NS];
     __shared__ int s_fail;
     const int tid = threadIdx.x;
@@ -618,15 +645,6 @@ __global__ void __launch_bounds__(kShearThreads, kTmaBlocks)
     double acc = 0.0;
     Lse L;
     lse_reset(L);
-    // With b the pass waits for memory (2 CTAs per SM, 570 us at 10^6 x 300; 612 us with
-    // eval_chunk at 3); without, it is eval_chunk's fewer registers that pay (446 us at 3 CTAs,
-    // 461 us with eval_quad at 3, 476 us at 2).
-    auto one_quad = [&](const Chunk &ch) {
-        if constexpr (HAS_B)
-            eval_quad<FAMILY, HAS_B>(c, ch, L);
-        else
-            eval_chunk<FAMILY, HAS_B>(c, ch, L);
-    };
     bool failed = false;
     int chunk = 0;
     long long tile = blockIdx.x;
@@ -642,21 +660,15 @@ __global__ void __launch_bounds__(kShearThreads, kTmaBlocks)
             if (chunk == 0) {
                 if (nq > 0) eval_first<FAMILY, HAS_B>(c, tma_quad(R, item, 0), L);
             } else if (nq > 0) {
-                one_quad(tma_quad(R, item, 0));
+                eval_chunk<FAMILY, HAS_B>(c, tma_quad(R, item, 0), L);
             }
 #pragma unroll
             for (int h = 1; h < kQuads; ++h)
-                if (h < nq) one_quad(tma_quad(R, item, h));
+                if (h < nq) eval_chunk<FAMILY, HAS_B>(c, tma_quad(R, item, h), L);
         }
         R.release(item);
         if (++chunk == R.cpg) {
-            if (n < s.n_gal) {
-                if constexpr (HAS_B) {
-                    if (lse_jumped(L)) L = replay_lane<FAMILY, HAS_B>(s, s.c, n, sub);
-                    __syncwarp(gmask);
-                }
-                finish_galaxy<kAGroup>(L, s.g1, s.g2, gmask, sub, s.w, n, acc);
-            }
+            if (n < s.n_gal) finish_galaxy<kAGroup>(L, s.g1, s.g2, gmask, sub, s.w, n, acc);
             lse_reset(L);
             chunk = 0;
             tile += gridDim.x;
@@ -667,19 +679,22 @@ __global__ void __launch_bounds__(kShearThreads, kTmaBlocks)
     block_partials<kAGroup>(s, s_fail ? NAN : acc);
 }
 
-template <int FAMILY, bool HAS_B>
-__device__ __noinline__ Lse replay_lane(const ShearLaunch &s, const ShearConst &c, long long n, int sub)
+__device__ __noinline__ double replay_galaxy(const ShearMultiLaunch &m, int p, long long n, int sub, unsigned gmask)
 {
+    const ShearLaunch &s = m.s;
     Lse L;
     lse_reset(L);
     const long long base = n * (long long)s.K;
     for (int k0 = kChunk * sub; k0 < s.K; k0 += kTileK)
         for (int k = k0; k < k0 + kChunk && k < s.K; k += 4) {
             Chunk ch;
-            load_chunk<HAS_B>(s, base, k, s.K, ch);
-            eval_chunk<FAMILY, HAS_B>(c, ch, L);
+            load_chunk<false>(s, base, k, s.K, ch);
+            eval_chunk<BS_EPRIOR_BA14, false>(m.c[p], ch, L);
         }
-    return L;
+    __syncwarp(gmask);
+    double t = 0.0;
+    finish_galaxy<kAGroup>(L, m.g1[p], m.g2[p], gmask, sub, s.w, n, t);
+    return t;
 }
 
 // The tensor-map encoder of the driver, looked up once through the runtime
@@ -1171,15 +1186,16 @@ int shear_multi_grid_blocks() { return resident_grid(g_grid_multi, shear_kernel_
 // state; a galaxy's 4 lanes put their FP64 totals per point in their own shared-memory
 // slot, summed over the block in a fixed order.  On a wait that gives up, the block's
 // partials are NaN.
-// FULL: all kMultiPoints points are asked for (no test between them).
-template <int FAMILY, bool FULL>
+// FULL: all kMultiPoints points are asked for (no test between them).  BOUNDED: eval_bounded's bounds
+// hold for every point.
+template <int FAMILY, bool FULL, bool BOUNDED>
 __global__ void __launch_bounds__(kShearThreads, 2)
     shear_kernel_tma_multi(const __grid_constant__ ShearMultiLaunch m, const __grid_constant__ CUtensorMap m1,
                            const __grid_constant__ CUtensorMap m2)
 {
     constexpr int NP = kMultiPoints;
     extern __shared__ __align__(128) unsigned char tma_raw[];
-    __shared__ __align__(8) uint64_t full[tma_stages(2)], empty[tma_stages(2)];
+    __shared__ __align__(8) uint64_t full[kTmaStages], empty[kTmaStages];
     __shared__ double acc[kTileG][NP][4];
     __shared__ int s_fail;
     const ShearLaunch &s = m.s;
@@ -1195,10 +1211,16 @@ __global__ void __launch_bounds__(kShearThreads, 2)
     TmaRing<2> R;
     R.init(tma_raw, full, empty, s.n_gal, K);   // (its barrier also orders the resets above)
     if (tid == 0)
-        for (int t = 0; t < tma_stages(2) - 1; ++t) R.issue(&m1, &m2, nullptr);
+        for (int t = 0; t < kTmaStages - 1; ++t) R.issue(&m1, &m2, nullptr);
     Lse L[NP];
+    auto reset = [&]() {
 #pragma unroll
-    for (int p = 0; p < NP; ++p) lse_reset(L[p]);
+        for (int p = 0; p < NP; ++p) {
+            lse_reset(L[p]);
+            if (kChunk * sub < K) L[p].m = BOUNDED ? 0.0f : m.m0[p];   // a lane without samples has no reference
+        }
+    };
+    reset();
     bool failed = false;
     int chunk = 0;
     long long tile = blockIdx.x;
@@ -1215,14 +1237,14 @@ __global__ void __launch_bounds__(kShearThreads, 2)
             for (int h = 0; h < kQuads; ++h) {
                 if (h < nq) {
                     const Chunk ch = tma_quad(R, item, h);
-                    if (h == 0 && chunk == 0) {
 #pragma unroll
-                        for (int p = 0; p < NP; ++p)
-                            if (FULL || p < m.n_points) eval_first<FAMILY, false>(m.c[p], ch, L[p]);
-                    } else {
-#pragma unroll
-                        for (int p = 0; p < NP; ++p)
-                            if (FULL || p < m.n_points) eval_quad<FAMILY, false>(m.c[p], ch, L[p]);
+                    for (int p = 0; p < NP; ++p) {
+                        if (FULL || p < m.n_points) {
+                            if constexpr (BOUNDED)
+                                eval_bounded<FAMILY>(m.c[p], ch, L[p]);
+                            else
+                                eval_quad<FAMILY>(m.c[p], ch, L[p]);
+                        }
                     }
                 }
             }
@@ -1234,15 +1256,15 @@ __global__ void __launch_bounds__(kShearThreads, 2)
                 for (int p = 0; p < NP; ++p) {
                     if (p < m.n_points) {
                         double t = 0.0;
-                        if (lse_jumped(L[p])) L[p] = replay_lane<FAMILY, false>(s, m.c[p], n, sub);
-                        __syncwarp(gmask);
-                        finish_galaxy<kAGroup>(L[p], m.g1[p], m.g2[p], gmask, sub, s.w, n, t);
+                        const float sw = finish_galaxy<kAGroup>(L[p], m.g1[p], m.g2[p], gmask, sub, s.w, n, t);
+                        if constexpr (FAMILY == BS_EPRIOR_BA14)
+                            if ((BOUNDED || m.m0[p] == 0.0f) && !(sw > kLeast && sw < kMost))
+                                t = replay_galaxy(m, p, n, sub, gmask);
                         acc[gl][p][sub] += t;
                     }
                 }
             }
-#pragma unroll
-            for (int p = 0; p < NP; ++p) lse_reset(L[p]);
+            reset();
             chunk = 0;
             tile += gridDim.x;
         }
@@ -1258,6 +1280,20 @@ __global__ void __launch_bounds__(kShearThreads, 2)
     }
 }
 
+namespace {
+
+using MultiKernel = void (*)(const ShearMultiLaunch, const CUtensorMap, const CUtensorMap);
+template <int FAMILY>
+MultiKernel tma_multi_kernel(bool full, bool bounded)
+{
+    if (bounded) return full ? shear_kernel_tma_multi<FAMILY, true, true> : shear_kernel_tma_multi<FAMILY, false, true>;
+    return full ? shear_kernel_tma_multi<FAMILY, true, false> : shear_kernel_tma_multi<FAMILY, false, false>;
+}
+
+}  // namespace
+
+float multi_reference(const ShearLaunch &s) { return s.a2 <= kMaxFall && s.c0 <= kMaxRise ? 0.0f : -1e30f; }
+
 cudaError_t launch_shear_multi(const ShearMultiLaunch &m, int grid, cudaStream_t stream)
 {
     const ShearLaunch &s = m.s;
@@ -1265,11 +1301,10 @@ cudaError_t launch_shear_multi(const ShearMultiLaunch &m, int grid, cudaStream_t
                      ((reinterpret_cast<uintptr_t>(s.e2) & 15) == 0) && s.b == nullptr;
     CUtensorMap m1, m2;
     if (vec && make_sample_map(m1, s.e1, s.n_gal, s.K) && make_sample_map(m2, s.e2, s.n_gal, s.K)) {
-        const bool full = m.n_points == kMultiPoints;
-        auto k = s.family == BS_EPRIOR_BA14
-                     ? (full ? shear_kernel_tma_multi<BS_EPRIOR_BA14, true> : shear_kernel_tma_multi<BS_EPRIOR_BA14, false>)
-                     : (full ? shear_kernel_tma_multi<BS_EPRIOR_TRUNC_GAUSS, true>
-                             : shear_kernel_tma_multi<BS_EPRIOR_TRUNC_GAUSS, false>);
+        bool bounded = true;
+        for (int p = 0; p < m.n_points; ++p) bounded = bounded && m.m0[p] == 0.0f;
+        auto k = s.family == BS_EPRIOR_BA14 ? tma_multi_kernel<BS_EPRIOR_BA14>(m.n_points == kMultiPoints, bounded)
+                                            : tma_multi_kernel<BS_EPRIOR_TRUNC_GAUSS>(m.n_points == kMultiPoints, bounded);
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)tma_smem_bytes(false));
         if (e != cudaSuccess) return e;
