@@ -85,11 +85,12 @@ cudaError_t launch_logpost_points(const FitParams &p, int n_points, const int32_
                                   cudaStream_t stream)
 {
     if (p.profile != 0) return launch_logpost_points_profile(p, n_points, gal_index, theta, logp, grad, stream);
-    const size_t smem = fit_smem_bytes(p.max_side, kPointWarps);
+    const int warps = point_warps(p);
+    const size_t smem = fit_smem_bytes(p.max_side, warps);
     PointsKernel k = points_kernel_for(p.max_side);
     const cudaError_t e = allow_smem((const void *)k);
     if (e != cudaSuccess) return e;
-    k<<<n_points, 32 * kPointWarps, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
+    k<<<n_points, 32 * warps, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
     bs::count_launches(1);
     return cudaGetLastError();
 }

@@ -1447,45 +1447,56 @@ __device__ void point_eval(const FitParams &P, const GalCtx &gc, const SmemView 
     if (grad && lane < 6) grad[lane] = gl;
 }
 
-// Points: a CTA stages a galaxy with all its warps and each warp then evaluates a point
-// of it.  Point i's CTA serves the run of points of the same galaxy from i to the end of
-// i's aligned block of kPointWarps points; a CTA whose point continues such a run has
-// nothing to do.  The staging (12 H N^2 flop against the evaluation's 33 H N) is
-// what the call costs.
-constexpr int kPointWarps = 4;
+// Points: a CTA stages a galaxy with all its warps, which then evaluate its points in turn.
+// Point i's CTA serves the run of points of the same galaxy from i to the end of i's aligned block
+// of kPointRun points; a CTA whose point continues such a run has nothing to do.  The
+// staging (12 H N^2 flop against the evaluation's 33 H N) is what the call costs.
+constexpr int kPointRun = 4;
+
+// Warps of a CTA: four share the rows and columns of the one-exposure staging.  The folded staging
+// (several exposures, or a noise correlation) takes a row of the spectrum at a time, a thread per
+// image row and then per column, with a barrier after each: it keeps as many warps busy as the
+// side has threads for.  2,000 points, one per galaxy: 25 px, three exposures, 361 us with four warps, 225
+// with one; 41 px, three, 1.39 ms with four, 1.12 with two; 53 px, three, 2.97 ms with two, 2.36 with four.
+inline int point_warps(const FitParams &P)
+{
+    if (P.n_exp == 1 && !P.noise_corr) return kPointRun;
+    return P.max_side <= 31 ? 1 : P.max_side <= 47 ? 2 : 4;
+}
 
 // The run of points of point i's CTA: [i, end), or false when an earlier one holds it.
 __device__ __forceinline__ bool point_run(int n_points, const int32_t *gal_index, int i, int &gal, int &end)
 {
     gal = gal_index[i];
-    if (i % kPointWarps != 0 && gal_index[i - 1] == gal) return false;
+    if (i % kPointRun != 0 && gal_index[i - 1] == gal) return false;
     end = i + 1;
-    while (end < n_points && end % kPointWarps != 0 && gal_index[end] == gal) ++end;
+    while (end < n_points && end % kPointRun != 0 && gal_index[end] == gal) ++end;
     return true;
 }
 
 template <int NC, int PROF>
-__global__ void __launch_bounds__(32 * kPointWarps, 5) logpost_points_kernel(const FitParams P, int n_points,
+__global__ void __launch_bounds__(32 * kPointRun, 5) logpost_points_kernel(const FitParams P, int n_points,
                                                                              const int32_t *gal_index,
                                                                              const float *theta, double *logp,
                                                                              float *grad)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const SmemView sm = smem_view(smem_raw, P.h_max, P.npad, P.max_side, kPointWarps);
+    const int warps = blockDim.x >> 5;
+    const SmemView sm = smem_view(smem_raw, P.h_max, P.npad, P.max_side, warps);
     int gal, end;
     if (!point_run(n_points, gal_index, blockIdx.x, gal, end)) return;
     GalCtx gc;
     const bool ok = gal >= 0 && gal < P.n_gal && side_ok(P, P.side[gal]) && setup_galaxy<NC>(P, gal, sm, gc);
-    const int k = blockIdx.x + warp;
-    if (k >= end) return;
-    if (!ok) {
-        if (lane == 0 && logp) logp[k] = NAN;
-        if (grad && lane < 6) grad[(size_t)k * 6 + lane] = NAN;
-        return;
+    for (int k = blockIdx.x + warp; k < end; k += warps) {
+        if (ok) {
+            point_eval<NC, PROF>(P, gc, sm, gal, warp, theta + (size_t)k * 6, logp ? logp + k : nullptr,
+                                 grad ? grad + (size_t)k * 6 : nullptr);
+        } else {
+            if (lane == 0 && logp) logp[k] = NAN;
+            if (grad && lane < 6) grad[(size_t)k * 6 + lane] = NAN;
+        }
     }
-    point_eval<NC, PROF>(P, gc, sm, gal, warp, theta + (size_t)k * 6, logp ? logp + k : nullptr,
-                         grad ? grad + (size_t)k * 6 : nullptr);
 }
 
 // The dense covariance's points: the same runs, a point per chain slot of one round.
@@ -1495,7 +1506,7 @@ __global__ void __launch_bounds__(32 * kDenseWarps, 1) logpost_points_dense_kern
                                                                                    const float *theta, double *logp,
                                                                                    float *grad)
 {
-    static_assert(kPointWarps == kDenseChains, "a run of points fills the chain slots");
+    static_assert(kPointRun == kDenseChains, "a run of points fills the chain slots");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const SmemView sm = smem_view(smem_raw, P.h_max, P.npad, P.max_side, kDenseChains);

@@ -32,7 +32,7 @@ FitKernel pix_kernel(int max_side, bool quad)
     if (quad) return max_side <= 31 ? fit_kernel_pix<1, 5> : fit_kernel_pix<2, 5>;
     return max_side <= 31 ? fit_kernel_pix<1, 3> : fit_kernel_pix<2, 3>;
 }
-static_assert(tc::Geo<4>::KV == kPixQuadSide + 1, "the four-chain layout's largest side");
+static_assert(tc::Geo<4>::KV == kPixQuadSide + 1 && tc::Geo<2>::kThreads == 256, "the chain layouts");
 
 bool is_pix(int profile) { return profile == 3; }
 
@@ -154,16 +154,14 @@ cudaError_t launch_fit_profile(const FitParams &p, int grid, cudaStream_t stream
 cudaError_t launch_logpost_points_profile(const FitParams &p, int n_points, const int32_t *gal_index,
                                           const float *theta, double *logp, float *grad, cudaStream_t stream)
 {
-    const size_t smem = smem_for(p.profile, p.max_side, is_pix(p.profile) ? 2 : kPointWarps);
+    const int warps = is_pix(p.profile) ? 8 : p.profile == 4 ? kDenseWarps : point_warps(p);
+    // (the dense path's CTA holds its four chain slots whatever its warps)
+    const size_t smem = smem_for(p.profile, p.max_side, is_pix(p.profile) ? 2 : p.profile == 4 ? kDenseChains : warps);
     PointsKernel k = points_for(p.profile, p.max_side);
     cudaError_t e = allow_smem((const void *)k, p.profile, p.max_side, 2);
     if (e != cudaSuccess) return e;
-    if (is_pix(p.profile)) {
-        const int grid = n_points < 4096 ? n_points : 4096;
-        k<<<grid, tc::Geo<2>::kThreads, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
-    } else {
-        k<<<n_points, threads_for(p.profile, kPointWarps, p.max_side), smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
-    }
+    const int grid = is_pix(p.profile) && n_points > 4096 ? 4096 : n_points;   // the others: a CTA per point
+    k<<<grid, 32 * warps, smem, stream>>>(p, n_points, gal_index, theta, logp, grad);
     bs::count_launches(1);
     return cudaGetLastError();
 }
