@@ -343,9 +343,10 @@ bs_status bs_fit_galaxies(const bs_fit_args *a, const bs_fit_out *o, void *works
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (p.profile == 4) p.cpc = dense_chains_per_cta(a->n_gal, p.n_chains, sms);
     if (p.profile == 3) p.cpc = bs::pixel_chains_per_cta(a->n_gal, p.n_chains, p.max_side, sms);
-    const int per_sm = bs::fit_blocks_per_sm(bs::cta_chains(p), a->max_side, p.regs, p.profile);
-    long long grid = (long long)sms * per_sm;
     const long long items = (long long)a->n_gal * bs::cta_groups(p);
+    if (p.profile == 4) p.dense_warps = bs::dense_warps_for(items, bs::cta_chains(p), p.max_side, sms);
+    const int per_sm = bs::fit_blocks_per_sm(bs::cta_chains(p), a->max_side, p.regs, p.profile, p.dense_warps);
+    long long grid = (long long)sms * per_sm;
     if (grid > items) grid = items;
     e = bs::launch_fit(p, (int)grid, s);
     return e == cudaSuccess ? BS_OK : cuda_fail(e, "bs_fit_galaxies: launch");

@@ -55,9 +55,9 @@ size_t fit_smem_bytes(int max_side, int n_chains)
            (size_t)scratch_float2(max_side, h, n_chains) * sizeof(float2) + (size_t)(h + 1) * sizeof(float2);
 }
 
-int fit_blocks_per_sm(int n_chains, int max_side, int regs, int profile)
+int fit_blocks_per_sm(int n_chains, int max_side, int regs, int profile, int dense_warps)
 {
-    if (profile != 0) return fit_blocks_per_sm_profile(profile, n_chains, max_side);
+    if (profile != 0) return fit_blocks_per_sm_profile(profile, n_chains, max_side, dense_warps);
     int nb = 0;
     const size_t smem = fit_smem_bytes(max_side, n_chains);
     FitKernel k = fit_kernel_for(max_side, regs, n_chains);

@@ -1514,11 +1514,11 @@ __global__ void __launch_bounds__(32 * kDenseWarps, 1) logpost_points_dense_kern
     if (!point_run(n_points, gal_index, blockIdx.x, gal, end)) return;
     GalCtx gc;
     const bool ok = gal >= 0 && gal < P.n_gal && side_ok(P, P.side[gal]) && setup_galaxy<NC>(P, gal, sm, gc);
-    const int k = blockIdx.x + warp;
+    const int k = blockIdx.x + warp, slots = end - (int)blockIdx.x;
     double v = ok ? -INFINITY : NAN;
     float gl = NAN;
     if (ok) {
-        dense_setup(P, gc, sm, dense_view(sm.kxr, P.h_max, P.npad, P.max_side), kDenseChains);
+        dense_setup(P, gc, sm, dense_view(sm.kxr, P.h_max, P.npad, P.max_side), slots);
         const float vcol[1] = {(float)(lane - gc.c)};
         float th[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (k < end)
@@ -1526,7 +1526,7 @@ __global__ void __launch_bounds__(32 * kDenseWarps, 1) logpost_points_dense_kern
             for (int i = 0; i < 6; ++i) th[i] = theta[(size_t)k * 6 + i];
         const bool active = k < end && in_support(P, th);
         double lp = 0.0;
-        dense_round<NC>(P, gc, sm, gal, kDenseChains, active, warp, vcol, th, gl, true, lp);
+        dense_round<NC>(P, gc, sm, gal, slots, active, warp, vcol, th, gl, true, lp);
         if (active) v = lp;
         else gl = NAN;
     }

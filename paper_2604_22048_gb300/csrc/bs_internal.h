@@ -70,6 +70,7 @@ struct FitParams {
     int h_max, npad;   // shared-memory geometry for max_side
     int cpc;           // chains per CTA (0: all n_chains): a galaxy's chains may be split
                        // over n_chains / cpc CTAs, each staging the galaxy itself
+    int dense_warps;   // warps of a dense-covariance CTA (0: 16)
     int regs;          // register cap of the kernel instance (128, 96 or 80;
                        // 0 = default)
     // serving: when `done` is set (host-mapped), each CTA copies its galaxy's
@@ -94,9 +95,11 @@ int pixel_chains_per_cta(int n_gal, int n_chains, int max_side, int sms);
 size_t fit_smem_bytes(int max_side, int n_chains);
 // Launch helpers implemented in the .cu files.
 cudaError_t launch_fit(const FitParams &p, int grid, cudaStream_t stream);
-int fit_blocks_per_sm(int n_chains, int max_side, int regs = 0, int profile = 0);
+// n_chains: of a CTA
+int fit_blocks_per_sm(int n_chains, int max_side, int regs = 0, int profile = 0, int dense_warps = 0);
 // Spergel / Gaussian instances (bs_fit_prof.cu)
-int fit_blocks_per_sm_profile(int profile, int n_chains, int max_side);
+int fit_blocks_per_sm_profile(int profile, int cc, int max_side, int dense_warps);
+int dense_warps_for(long long ctas, int cc, int max_side, int sms);
 cudaError_t launch_fit_profile(const FitParams &p, int grid, cudaStream_t stream);
 cudaError_t launch_logpost_points_profile(const FitParams &p, int n_points, const int32_t *gal_index,
                                           const float *theta, double *logp, float *grad, cudaStream_t stream);

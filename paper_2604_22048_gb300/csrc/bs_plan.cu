@@ -85,7 +85,7 @@ cudaError_t time_variant(const bs_fit_plan_s::Launch &L, int regs, int n_trial, 
     bs::FitParams p = L.p;
     p.regs = regs;
     p.n_work = n_trial;
-    const int per_sm = bs::fit_blocks_per_sm(bs::cta_chains(p), p.max_side, regs, p.profile);
+    const int per_sm = bs::fit_blocks_per_sm(bs::cta_chains(p), p.max_side, regs, p.profile, p.dense_warps);
     const int grid = std::min(n_trial * bs::cta_groups(p), sms * per_sm);
     cudaError_t e = cudaSuccess;
     for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
@@ -119,7 +119,7 @@ cudaError_t autotune(bs_fit_plan_s *pl, int sms)
     for (auto &L : pl->launches) {
         if (e != cudaSuccess) break;
         int waves = 1;
-        for (int r : kRegVariants) waves = std::max(waves, bs::fit_blocks_per_sm(L.p.n_chains, L.p.max_side, r, L.p.profile));
+        for (int r : kRegVariants) waves = std::max(waves, bs::fit_blocks_per_sm(L.p.n_chains, L.p.max_side, r, L.p.profile, L.p.dense_warps));
         const int n_trial = std::min(L.p.n_work, 2 * sms * waves);
         float best = 0.f;
         // all of a galaxy's chains; the pixel-weight path's two or four are not the tuner's to choose
@@ -157,7 +157,7 @@ cudaError_t autotune(bs_fit_plan_s *pl, int sms)
         L.p.cpc = best_cpc;
         const int groups = bs::cta_groups(L.p);
         L.grid = std::min(L.p.n_work * groups,
-                          sms * bs::fit_blocks_per_sm(bs::cta_chains(L.p), L.p.max_side, best_regs, L.p.profile));
+                          sms * bs::fit_blocks_per_sm(bs::cta_chains(L.p), L.p.max_side, best_regs, L.p.profile, L.p.dense_warps));
     }
     if (st) cudaStreamDestroy(st);
     if (e0) cudaEventDestroy(e0);
@@ -253,7 +253,8 @@ bs_status plan_create(const bs_fit_args *a, const bs_fit_out *o, const int32_t *
         L.trial_ms[0] = L.trial_ms[1] = L.trial_ms[2] = 0.f;
         L.trial_half[0] = L.trial_half[1] = L.trial_half[2] = 0.f;
         if (L.p.profile == 3) L.p.cpc = bs::pixel_chains_per_cta(count[c], a->n_chains, maxs[c], sms);
-        const int per_sm = bs::fit_blocks_per_sm(a->n_chains, maxs[c], L.p.regs, L.p.profile);
+        if (L.p.profile == 4) L.p.dense_warps = bs::dense_warps_for(count[c], a->n_chains, maxs[c], sms);
+        const int per_sm = bs::fit_blocks_per_sm(a->n_chains, maxs[c], L.p.regs, L.p.profile, L.p.dense_warps);
         L.grid = std::min(count[c], sms * per_sm);
         pl->launches.push_back(L);
         start += count[c];
@@ -276,7 +277,8 @@ bs_status plan_create(const bs_fit_args *a, const bs_fit_out *o, const int32_t *
             return bs::set_error(BS_ERR_CUDA, "bs_fit_plan_create: streams: %s", cudaGetErrorString(e));
         }
         // kernel attributes are set outside the capture
-        for (auto &L : pl->launches) bs::fit_blocks_per_sm(bs::cta_chains(L.p), L.p.max_side, L.p.regs, L.p.profile);
+        for (auto &L : pl->launches)
+            bs::fit_blocks_per_sm(bs::cta_chains(L.p), L.p.max_side, L.p.regs, L.p.profile, L.p.dense_warps);
         e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             bs::capture_launches(&pl->graph_kernels);   // recorded, not launched
