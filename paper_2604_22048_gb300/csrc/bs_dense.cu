@@ -47,25 +47,31 @@ struct DenseSmem {
 };
 
 // Right-looking Cholesky of the nb x nb pivot block in sm.D (all threads); sets sm.bad where a
-// pivot is not positive.  A column per step on the first warps, lane = row.
+// pivot is not positive.  A column per step: the first warp (lane = row) forms the reciprocal and scales
+// the column.  One warp, because the FP64 pipe is the SM's and a square root and a division
+// cost it as much for every warp that asks: formed by all eight they were two
+// microseconds of every column.
 __device__ void factor_pivot(DenseSmem &sm, int nb)
 {
     const int tid = threadIdx.x;
     bool bad = false;
     for (int j = 0; j < nb; ++j) {
-        const double d = sm.D[j][j];       // the same value in every thread
-        if (!(d > 0.0)) {
+        if (tid < 32) {
+            const double d = sm.D[j][j];
+            const double rd = d > 0.0 ? 1.0 / sqrt(d) : NAN;
+            __syncwarp();
+            if (tid == j) {
+                sm.D[j][j] = d * rd;
+                sm.rd[j] = rd;
+            } else if (tid > j && tid < nb) {
+                sm.D[tid][j] = sm.D[tid][j] * rd;
+            }
+        }
+        __syncthreads();
+        if (isnan(sm.rd[j])) {
             bad = true;
             break;
         }
-        const double rd = 1.0 / sqrt(d);
-        __syncthreads();
-        if (tid > j && tid < nb) sm.D[tid][j] = sm.D[tid][j] * rd;
-        if (tid == j) {
-            sm.D[j][j] = d * rd;
-            sm.rd[j] = rd;
-        }
-        __syncthreads();
         // the trailing part of the block: 8 threads per row
         const int i = tid >> 3;
         if (i > j && i < nb) {
@@ -78,23 +84,37 @@ __device__ void factor_pivot(DenseSmem &sm, int nb)
     __syncthreads();
 }
 
-// acc[a][b] = acc[a][b] -+ sum_k X[k][rx + a] Y[k][ry + b], k ascending, product and sum rounded apart.
-template <bool SUB>
-__device__ __forceinline__ void tile_terms(const DenseSmem &sm, int nk, int rx, int ry, double (&acc)[4][4])
+// Column of a tile of a thread's b-th (0..3): two in either half of the warp's 32 columns, ry the first.
+__device__ __forceinline__ int tile_col(int ry, int b) { return ry + (b & 1) + 16 * (b >> 1); }
+
+// acc[a][b] = acc[a][b] -+ sum_k X[k][rx + a] Y[k][column b], k0 <= k < nk ascending, product and sum rounded
+// apart, of the first NA of a thread's rows and NB of its columns.
+template <bool SUB, int NA, int NB>
+__device__ __forceinline__ void tile_part(const DenseSmem &sm, int k0, int nk, int rx, int ry, double (&acc)[4][4])
 {
 #pragma unroll 2
-    for (int k = 0; k < nk; ++k) {
-        double x[4], y[4];
+    for (int k = k0; k < nk; ++k) {
+        double x[NA], y[NB];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            x[a] = sm.X[k][rx + a];
-            y[a] = sm.Y[k][ry + a];
-        }
+        for (int a = 0; a < NA; ++a) x[a] = sm.X[k][rx + a];
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int b = 0; b < NB; ++b) y[b] = sm.Y[k][tile_col(ry, b)];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] = SUB ? acc[a][b] - x[a] * y[b] : acc[a][b] + x[a] * y[b];
+        for (int a = 0; a < NA; ++a)
+#pragma unroll
+            for (int b = 0; b < NB; ++b) acc[a][b] = SUB ? acc[a][b] - x[a] * y[b] : acc[a][b] + x[a] * y[b];
     }
+}
+// rows, cols: how many of the warp's 16 rows and 32 columns the matrix, or its lower triangle, has: the FP64
+// pipe takes as long for entries that are not needed.  (With n = N^2 the last row block of every
+// second side is one row.)
+template <bool SUB>
+__device__ __forceinline__ void tile_terms(const DenseSmem &sm, int k0, int nk, int rx, int ry, int rows, int cols,
+                                           double (&acc)[4][4])
+{
+    if (rows == 1) tile_part<SUB, 1, 4>(sm, k0, nk, rx, ry, acc);
+    else if (cols <= 16) tile_part<SUB, 4, 2>(sm, k0, nk, rx, ry, acc);
+    else tile_part<SUB, 4, 4>(sm, k0, nk, rx, ry, acc);
 }
 
 // Tile number -> (row, column) of the lower triangle of tiles, row by row.
@@ -120,15 +140,19 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_precision_kernel(int n
     double *A = scratch + (size_t)my_cluster * G * scratch_per_cta;
     const int tid = threadIdx.x, nth = blockDim.x;
     const int gtid = rank * nth + tid, gnth = G * nth;      // thread of the cluster
-    // a thread's 4 x 4 part of a 64 x 64 tile: warp w has rows 16 (w / 2) .. + 15 and columns
-    // 32 (w mod 2) .. + 31
+    // a thread's 4 x 4 entries of a 64 x 64 tile (tile_col): warp w has rows 16 (w mod 4) .. + 15 and columns
+    // 32 (w / 4) .. + 31 (the four quarters of the SM, each with its part of the FP64 pipe, take a row
+    // block each: the parts above the diagonal, and a small matrix's, leave none of them out)
     const int warp = tid >> 5, lane = tid & 31;
-    const int rx = 16 * (warp >> 1) + 4 * (lane >> 3), ry = 32 * (warp & 1) + 4 * (lane & 7);
+    const int wi = 16 * (warp & 3), wj = 32 * (warp >> 2);
+    const int rx = wi + 4 * (lane >> 3), ry = wj + 2 * (lane & 7);
     // whether the warp's 16 x 32 part of the tile at (i0, j0) meets the lower triangle of n rows
     auto part_of = [&](int i0, int j0, int n) {
-        const int i1 = i0 + 16 * (warp >> 1), j1 = j0 + 32 * (warp & 1);
+        const int i1 = i0 + wi, j1 = j0 + wj;
         return i1 < n && i1 + 15 >= j1;
     };
+    // and how many of its columns do
+    auto cols_of = [&](int i0, int j0, int n) { return min(i0 + wi + 15, n - 1) - (j0 + wj) + 1; };
     for (int gal = my_cluster; gal < n_gal; gal += n_clusters) {
         const int N = side[gal];
         if (N < 3 || N > max_side || !(N & 1)) {      // the scratch holds max_side only
@@ -201,15 +225,15 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_precision_kernel(int n
                     for (int a = 0; a < 4; ++a)
 #pragma unroll
                         for (int b = 0; b < 4; ++b) {
-                            const int i = i0 + rx + a, j = j0 + ry + b;
+                            const int i = i0 + rx + a, j = j0 + tile_col(ry, b);
                             acc[a][b] = i < n && j <= i ? A[(size_t)i * n + j] : 0.0;
                         }
-                    tile_terms<true>(sm, nb, rx, ry, acc);
+                    tile_terms<true>(sm, 0, nb, rx, ry, n - i0 - wi, cols_of(i0, j0, n), acc);
 #pragma unroll
                     for (int a = 0; a < 4; ++a)
 #pragma unroll
                         for (int b = 0; b < 4; ++b) {
-                            const int i = i0 + rx + a, j = j0 + ry + b;
+                            const int i = i0 + rx + a, j = j0 + tile_col(ry, b);
                             if (i < n && j <= i) A[(size_t)i * n + j] = acc[a][b];
                         }
                 }
@@ -224,7 +248,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_precision_kernel(int n
             continue;
         }
         // ---- W = L^-1:  W[i][c] = (delta_ic - sum_{c <= k < i} L[i][k] W[k][c]) / L[i][i]
-        for (size_t e = gtid; e < (size_t)n * n; e += gnth) W[e] = e % (n + 1) == 0 ? 1.0 : 0.0;
+        for (size_t e = gtid; e < (size_t)n * n; e += gnth) W[e] = (int)e % (n + 1) == 0 ? 1.0 : 0.0;
         cluster.sync();
         for (int p0 = 0; p0 < n; p0 += kPivot) {
             const int nb = min(kPivot, n - p0), r1 = p0 + nb;
@@ -264,21 +288,21 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_precision_kernel(int n
                     sm.Y[k][c] = c0 + c < r1 ? W[(size_t)(p0 + k) * n + c0 + c] : 0.0;
                 }
                 __syncthreads();
-                if (c0 + 32 * (warp & 1) < r1 && i0 + 16 * (warp >> 1) < n) {
+                if (c0 + wj < r1 && i0 + wi < n) {
                     double acc[4][4];
 #pragma unroll
                     for (int a = 0; a < 4; ++a)
 #pragma unroll
                         for (int b = 0; b < 4; ++b) {
-                            const int i = i0 + rx + a, c = c0 + ry + b;
+                            const int i = i0 + rx + a, c = c0 + tile_col(ry, b);
                             acc[a][b] = i < n && c < r1 ? W[(size_t)i * n + c] : 0.0;
                         }
-                    tile_terms<true>(sm, nb, rx, ry, acc);
+                    tile_terms<true>(sm, 0, nb, rx, ry, n - i0 - wi, r1 - c0 - wj, acc);
 #pragma unroll
                     for (int a = 0; a < 4; ++a)
 #pragma unroll
                         for (int b = 0; b < 4; ++b) {
-                            const int i = i0 + rx + a, c = c0 + ry + b;
+                            const int i = i0 + rx + a, c = c0 + tile_col(ry, b);
                             if (i < n && c < r1) W[(size_t)i * n + c] = acc[a][b];
                         }
                 }
@@ -306,13 +330,16 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_precision_kernel(int n
                     sm.Y[k][c] = j0 + c < n ? W[(size_t)(k0 + k) * n + j0 + c] : 0.0;
                 }
                 __syncthreads();
-                if (part_of(i0, j0, n)) tile_terms<false>(sm, nk, rx, ry, acc);
+                // (the terms before the first row of the warp's part are products with zeros of W)
+                if (part_of(i0, j0, n))
+                    tile_terms<false>(sm, max(0, i0 + wi - k0), nk, rx, ry, n - i0 - wi, cols_of(i0, j0, n),
+                                      acc);
             }
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
-                    const int i = i0 + rx + a, j = j0 + ry + b;
+                    const int i = i0 + rx + a, j = j0 + tile_col(ry, b);
                     if (i < n && j <= i) {
                         const float v = (float)acc[a][b];
                         Pout[(size_t)i * n + j] = v;
