@@ -51,6 +51,9 @@ def pack_stamps(sides, align=4):
     """Offsets of stamps packed back to back, each start rounded up to `align`
     elements.  Returns (offsets int64 array, total elements)."""
     sizes = np.array(sides, dtype=np.int64)
+    if sizes.shape == (1,):               # a single stamp: array operations cost more than the numbers
+        n = int(sizes[0])
+        return np.zeros(1, dtype=np.int64), (n * n + align - 1) // align * align
     sizes *= sizes
     sizes += align - 1
     sizes //= align
