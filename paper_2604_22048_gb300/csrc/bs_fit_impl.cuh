@@ -128,8 +128,8 @@ __device__ __forceinline__ void slot_offsets(int npad, int j, int l, int &ox, in
 }
 
 // cosh of the Moffat transform's integration nodes t_j = j / 4, written by setup_psf:
-// the nodes are the same for every grid point (x cosh t passes the stopping rule's 40
-// before node 64 for any x > 1e-5; later nodes are formed on the spot).
+// the nodes are the same for every grid point (the stopping rule x cosh t > nu t + 40 passes
+// before node 64 for x > 3e-5 and nu up to 4; later nodes are formed on the spot).
 constexpr int kCoshNodes = 64;
 __shared__ float s_cosh[kCoshNodes];
 

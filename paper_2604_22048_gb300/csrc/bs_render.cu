@@ -18,8 +18,8 @@
 // FP32x2 multiply-adds.
 // The PSF depends on |k| alone: it is formed for the H (H + 1) / 2 pairs (u, a <= u) and
 // read for (u, +-a) and (a, +-u).
-// Bound by instruction issue and by the CTAs that shared memory allows (24 warps per SM).  20,000 stamps of 25-101 px with a Moffat PSF each:
-// 2.7 ms with direct sums over a stamp's N^2 pixels, the PSF integrated at every grid
+// Bound by instruction issue and by the CTAs that shared memory allows (24 warps per SM).
+// 20,000 stamps of 25-101 px with a Moffat PSF each: 2.7 ms with direct sums over a stamp's N^2 pixels, the PSF integrated at every grid
 // point and one shared-memory load per two multiply-adds; 0.51 ms now (error against
 // 64 bits 3.6e-7 and 2.8e-7).
 #include "bs_device.cuh"
@@ -74,7 +74,7 @@ __device__ RenderPsf render_psf(const bs_psf &ps)
 // K_nu(x) = int_0^inf exp(-x cosh t) cosh(nu t) dt by the trapezoidal rule, whose nodes'
 // cosh t_j and cosh(nu t_j) do not depend on x, so that a node costs one exponential.
 // The rule's relative error is about 2 |Gamma(nu + 2 pi i / step)| / Gamma(nu) for small x:
-// 1e-9 at nu = 2 and 3e-8 at nu = 4 with step 3/8 (6e-7 at nu = 2 with step 1/2), and
+// 1e-9 at nu = 2 and 6e-8 at nu = 4 with step 3/8 (6e-7 at nu = 2 with step 1/2), and
 // nothing a float holds with step 1/4, taken from x = 2 on, where the integrand narrows,
 // and for larger nu.  Sums stop below 1e-9 of the total.  Very large nu or tiny x,
 // whose factors leave the range of a float, take the folded form.

@@ -495,8 +495,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
     for (;;) {
         uint32_t ok;
         asm volatile(
-                        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(ok)
             : "r"(bar), "r"(parity), "r"(20000u)
