@@ -521,13 +521,12 @@ bs_status bs_shear_loglike_multi(const bs_shear_data *d, int32_t n_points, const
             if (st != BS_OK) return st;
             if (p == 0) M.s = L;
             M.c[p] = L.c;
-            M.m0[p] = bs::multi_reference(L);
+            M.bounded = (p == 0 || M.bounded) && bs::weights_bounded(L);
             M.g1[p] = L.g1;
             M.g2[p] = L.g2;
         }
         for (int p = np; p < NP; ++p) {
             M.c[p] = M.c[0];
-            M.m0[p] = M.m0[0];
             M.g1[p] = M.g2[p] = 0.f;
         }
         M.n_points = np;

@@ -160,12 +160,11 @@ struct ShearMultiLaunch {
     int n_points;                   // 1..kMultiPoints
     ShearConst c[kMultiPoints];
     float g1[kMultiPoints], g2[kMultiPoints];
-    float m0[kMultiPoints];         // multi_reference of the point
+    bool bounded;                   // weights_bounded at every point
     double *partials;               // [kMultiPoints][grid][4]
 };
-// The reference log2 weight that a point's sums start from: 0 where the weights cannot leave the
-// range of a float, else none yet.  It depends on the point alone, not on the others of its pass.
-float multi_reference(const ShearLaunch &s);
+// Whether no sample's weight at this point can lie above another's by more than 2^32.
+bool weights_bounded(const ShearLaunch &s);
 int shear_multi_grid_blocks();
 cudaError_t launch_shear_multi(const ShearMultiLaunch &m, int grid, cudaStream_t stream);
 // Finalize the points of several passes in one launch: point q's partials (n_part blocks of

@@ -191,6 +191,8 @@ struct Lse {
     float2 tr;               // sum of weight rU r
 };
 
+constexpr float kNoReference = -1e30f;
+
 // Samples missing from a chunk (past K) get log weight -inf.
 __device__ __forceinline__ void mask_missing(const Chunk &ch, float2 (&x)[2])
 {
@@ -315,34 +317,41 @@ __device__ __forceinline__ void eval_quad(const ShearConst &c, const Chunk &ch, 
     for (int h = 0; h < 2; ++h) add_pair(L, pair_weight(x[h], nm, fw[h]), e1[h], e2[h], ru[h], pp[h], rr[h], qq[h]);
 }
 
-// Four samples of a galaxy against the reference 0 (L.m = 0), for points whose exponents are bounded: an
-// ellipticity in the unit disk has 0 <= Q < 1, so that x lies in (-a2, c0), and with a2 <= kMaxFall
-// (alpha >= 0.095) and c0 <= kMaxRise no weight leaves the range of a float and no reference is needed.
-// Four points of 50,000 x 300: 96-101 us.
-constexpr float kMaxFall = 80.0f, kMaxRise = 32.0f;
+// Four samples of a galaxy after its first four, against the reference as it stands, for points whose weights
+// cannot jump: an ellipticity in the unit disk has 0 <= Q < 1, so that x lies in (-a2, c0), and with
+// a2 + c0 <= kMaxSpan (alpha >= 0.173 at sigma_e0 = 0.3) no sample is above another by more than eval_quad
+// allows.  The bits are eval_quad's.  Four points of 50,000 x 300: 98-105 us.
+constexpr float kMaxSpan = 32.0f;
 template <int FAMILY>
-__device__ __forceinline__ void eval_bounded(const ShearConst &c, const Chunk &ch, Lse &L)
+__device__ __forceinline__ void eval_plain(const ShearConst &c, const Chunk &ch, Lse &L)
 {
+    const float2 nm = f2(-L.m);
     const float2 e1[2] = {make_float2(ch.e1.x, ch.e1.y), make_float2(ch.e1.z, ch.e1.w)};
     const float2 e2[2] = {make_float2(ch.e2.x, ch.e2.y), make_float2(ch.e2.z, ch.e2.w)};
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         float2 x, fw, ru, pp, rr, qq;
         pair_terms<FAMILY, false>(c, e1[h], e2[h], f2(0.f), x, fw, ru, pp, rr, qq);
-        add_pair(L, mul2(make_float2(ex2_ftz(x.x), ex2_ftz(x.y)), fw), e1[h], e2[h], ru, pp, rr, qq);
+        add_pair(L, pair_weight(x, nm, fw), e1[h], e2[h], ru, pp, rr, qq);
     }
 }
 
-// A galaxy's sum of weights outside these did leave that range: samples on or outside the unit circle, which
-// the BA14 weight does not exclude (the truncated Gaussian gives them none), or a shear near 1.
-// Its samples are then taken again with a reference (replay_galaxy).
-constexpr float kLeast = 0x1p-100f, kMost = 0x1p100f;
+// A galaxy's first chunk (e1 at r, e2 a tile further) by eval_chunk, for a lane whose first four samples have no
+// weight (the truncated Gaussian's far samples) and set no reference for eval_plain.
+template <int FAMILY>
+__device__ __noinline__ Lse first_chunk(const ShearConst &c, const float *r, int n_quads);
+
+// A galaxy's sum of weights that is not below this (or NaN) has left the range of a float all the same: the
+// whole first chunk of a lane had no weight (the truncated Gaussian's far samples), or samples lie on or
+// outside the unit circle.  The galaxy is then taken again by eval_chunk (replay_galaxy).
+constexpr float kMost = 0x1p100f;
 
 // Merge the lanes of a galaxy's group and add the galaxy's terms, times the galaxy's weight
 // w[n] (1 when w is NULL; a zero weight drops the galaxy), to the accumulators of the
 // group's first four lanes: lane 0 the log-sum-exp (log2), lanes 1-3 the softmax-weighted
 // derivative sums, each lane one of them: the FP64 pipe takes 16 cycles an operation for the
-// whole SM, so the four go through it side by side.  (g1, g2) is the shear of the evaluation.
+// whole SM, so the four go through it side by side.  (g1, g2) is the shear of the evaluation.  Returns the
+// galaxy's sum of weights.
 template <int G = kGroup>
 __device__ __forceinline__ float finish_galaxy(const Lse &L, float g1, float g2, unsigned gmask, int sub,
                                               const float *w, long long n, double &acc)
@@ -391,12 +400,13 @@ __device__ __forceinline__ float finish_galaxy(const Lse &L, float g1, float g2,
 
 __device__ __forceinline__ void lse_reset(Lse &L)
 {
-    L.m = -1e30f;
+    L.m = kNoReference;
     L.sw = L.t1 = L.t2 = L.tq = L.tr = f2(0.f);
 }
 
-// Galaxy n (BA14) at point p by the group's lanes, each its samples of the tile kernels' assignment (12 of
-// every 48) by eval_chunk; this lane's term as finish_galaxy adds it.
+// Galaxy n at point p by the group's lanes, each its samples of the tile kernels' assignment (12 of every 48)
+// by eval_chunk; this lane's term as finish_galaxy adds it.
+template <int FAMILY>
 __device__ __noinline__ double replay_galaxy(const ShearMultiLaunch &m, int p, long long n, int sub, unsigned gmask);
 
 // Block reduction of the lanes' FP64 accumulators (quantity = lane of the group of G, the
@@ -603,10 +613,15 @@ struct TmaRing {
 // Quad h (4 consecutive samples) of this thread's part of a chunk of its galaxy (4 lanes
 // per galaxy, 12 samples each) in item's stage, and how many quads of it lie below K.
 template <int NV>
-__device__ __forceinline__ Chunk tma_quad(const TmaRing<NV> &R, int item, int h)
+__device__ __forceinline__ const float *tma_row(const TmaRing<NV> &R, int item)
 {
     const int tid = threadIdx.x, sub = tid & (kAGroup - 1), gl = tid / kAGroup;
-    const float *r1 = R.ring + (size_t)(item % TmaRing<NV>::kStages) * NV * kTileFloats + gl * kTileK + kChunk * sub + 4 * h;
+    return R.ring + (size_t)(item % TmaRing<NV>::kStages) * NV * kTileFloats + gl * kTileK + kChunk * sub;
+}
+template <int NV>
+__device__ __forceinline__ Chunk tma_quad(const TmaRing<NV> &R, int item, int h)
+{
+    const float *r1 = tma_row(R, item) + 4 * h;
     Chunk ch;
     ch.nvalid = 4;
     ch.full = true;
@@ -678,6 +693,24 @@ __global__ void __launch_bounds__(kShearThreads, kTmaBlocks)
     block_partials<kAGroup>(s, s_fail ? NAN : acc);
 }
 
+template <int FAMILY>
+__device__ __noinline__ Lse first_chunk(const ShearConst &c, const float *r, int n_quads)
+{
+    Lse L;
+    lse_reset(L);
+    Chunk ch;
+    ch.nvalid = 4;
+    ch.full = true;
+    ch.b = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int h = 0; h < n_quads; ++h) {
+        ch.e1 = *reinterpret_cast<const float4 *>(r + 4 * h);
+        ch.e2 = *reinterpret_cast<const float4 *>(r + kTileFloats + 4 * h);
+        eval_chunk<FAMILY, false>(c, ch, L);
+    }
+    return L;
+}
+
+template <int FAMILY>
 __device__ __noinline__ double replay_galaxy(const ShearMultiLaunch &m, int p, long long n, int sub, unsigned gmask)
 {
     const ShearLaunch &s = m.s;
@@ -688,7 +721,7 @@ __device__ __noinline__ double replay_galaxy(const ShearMultiLaunch &m, int p, l
         for (int k = k0; k < k0 + kChunk && k < s.K; k += 4) {
             Chunk ch;
             load_chunk<false>(s, base, k, s.K, ch);
-            eval_chunk<BS_EPRIOR_BA14, false>(m.c[p], ch, L);
+            eval_chunk<FAMILY, false>(m.c[p], ch, L);
         }
     __syncwarp(gmask);
     double t = 0.0;
@@ -1185,8 +1218,8 @@ int shear_multi_grid_blocks() { return resident_grid(g_grid_multi, shear_kernel_
 // state; a galaxy's 4 lanes put their FP64 totals per point in their own shared-memory
 // slot, summed over the block in a fixed order.  On a wait that gives up, the block's
 // partials are NaN.
-// FULL: all kMultiPoints points are asked for (no test between them).  BOUNDED: eval_bounded's bounds
-// hold for every point.
+// FULL: all kMultiPoints points are asked for (no test between them).  BOUNDED: eval_plain's bound
+// holds for every point.
 template <int FAMILY, bool FULL, bool BOUNDED>
 __global__ void __launch_bounds__(kShearThreads, 2)
     shear_kernel_tma_multi(const __grid_constant__ ShearMultiLaunch m, const __grid_constant__ CUtensorMap m1,
@@ -1212,14 +1245,8 @@ __global__ void __launch_bounds__(kShearThreads, 2)
     if (tid == 0)
         for (int t = 0; t < kTmaStages - 1; ++t) R.issue(&m1, &m2, nullptr);
     Lse L[NP];
-    auto reset = [&]() {
 #pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            lse_reset(L[p]);
-            if (kChunk * sub < K) L[p].m = BOUNDED ? 0.0f : m.m0[p];   // a lane without samples has no reference
-        }
-    };
-    reset();
+    for (int p = 0; p < NP; ++p) lse_reset(L[p]);
     bool failed = false;
     int chunk = 0;
     long long tile = blockIdx.x;
@@ -1236,16 +1263,24 @@ __global__ void __launch_bounds__(kShearThreads, 2)
             for (int h = 0; h < kQuads; ++h) {
                 if (h < nq) {
                     const Chunk ch = tma_quad(R, item, h);
+                    auto all = [&](auto eval) {
 #pragma unroll
-                    for (int p = 0; p < NP; ++p) {
-                        if (FULL || p < m.n_points) {
-                            if constexpr (BOUNDED)
-                                eval_bounded<FAMILY>(m.c[p], ch, L[p]);
-                            else
-                                eval_quad<FAMILY>(m.c[p], ch, L[p]);
-                        }
-                    }
+                        for (int p = 0; p < NP; ++p)
+                            if (FULL || p < m.n_points) eval(p);
+                    };
+                    if (h == 0 && chunk == 0)
+                        all([&](int p) { eval_first<FAMILY, false>(m.c[p], ch, L[p]); });
+                    else if constexpr (BOUNDED)
+                        all([&](int p) { eval_plain<FAMILY>(m.c[p], ch, L[p]); });
+                    else
+                        all([&](int p) { eval_quad<FAMILY>(m.c[p], ch, L[p]); });
                 }
+            }
+            if (BOUNDED && FAMILY == BS_EPRIOR_TRUNC_GAUSS && chunk == 0 && nq > 0) {
+#pragma unroll
+                for (int p = 0; p < NP; ++p)
+                    if ((FULL || p < m.n_points) && L[p].m == kNoReference)
+                        L[p] = first_chunk<FAMILY>(m.c[p], tma_row(R, item), nq);
             }
         }
         R.release(item);
@@ -1256,14 +1291,13 @@ __global__ void __launch_bounds__(kShearThreads, 2)
                     if (p < m.n_points) {
                         double t = 0.0;
                         const float sw = finish_galaxy<kAGroup>(L[p], m.g1[p], m.g2[p], gmask, sub, s.w, n, t);
-                        if constexpr (FAMILY == BS_EPRIOR_BA14)
-                            if ((BOUNDED || m.m0[p] == 0.0f) && !(sw > kLeast && sw < kMost))
-                                t = replay_galaxy(m, p, n, sub, gmask);
+                        if (BOUNDED && !(sw < kMost)) t = replay_galaxy<FAMILY>(m, p, n, sub, gmask);
                         acc[gl][p][sub] += t;
                     }
                 }
             }
-            reset();
+#pragma unroll
+            for (int p = 0; p < NP; ++p) lse_reset(L[p]);
             chunk = 0;
             tile += gridDim.x;
         }
@@ -1291,7 +1325,7 @@ MultiKernel tma_multi_kernel(bool full, bool bounded)
 
 }  // namespace
 
-float multi_reference(const ShearLaunch &s) { return s.a2 <= kMaxFall && s.c0 <= kMaxRise ? 0.0f : -1e30f; }
+bool weights_bounded(const ShearLaunch &s) { return s.a2 + s.c0 <= kMaxSpan; }
 
 cudaError_t launch_shear_multi(const ShearMultiLaunch &m, int grid, cudaStream_t stream)
 {
@@ -1300,10 +1334,8 @@ cudaError_t launch_shear_multi(const ShearMultiLaunch &m, int grid, cudaStream_t
                      ((reinterpret_cast<uintptr_t>(s.e2) & 15) == 0) && s.b == nullptr;
     CUtensorMap m1, m2;
     if (vec && make_sample_map(m1, s.e1, s.n_gal, s.K) && make_sample_map(m2, s.e2, s.n_gal, s.K)) {
-        bool bounded = true;
-        for (int p = 0; p < m.n_points; ++p) bounded = bounded && m.m0[p] == 0.0f;
-        auto k = s.family == BS_EPRIOR_BA14 ? tma_multi_kernel<BS_EPRIOR_BA14>(m.n_points == kMultiPoints, bounded)
-                                            : tma_multi_kernel<BS_EPRIOR_TRUNC_GAUSS>(m.n_points == kMultiPoints, bounded);
+        auto k = s.family == BS_EPRIOR_BA14 ? tma_multi_kernel<BS_EPRIOR_BA14>(m.n_points == kMultiPoints, m.bounded)
+                                            : tma_multi_kernel<BS_EPRIOR_TRUNC_GAUSS>(m.n_points == kMultiPoints, m.bounded);
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)tma_smem_bytes(false));
         if (e != cudaSuccess) return e;

@@ -1,5 +1,5 @@
 """Shear passes whose log weights span a wide range, at several points and with per-sample offsets: narrow ellipticity
-distributions (alpha from 0.005 up, on either side of 0.095, from where the weights of a pass need no reference), samples on and
+distributions (alpha from 0.005 up, on either side of 0.173, from where no weight can be far above another), samples on and
 outside the unit circle (BA14 gives them a weight), galaxies whose first samples have none, and widely scattered offsets
 in both families.  Against one point at a time, which rescales as it goes, or the oracle.  Bounds as for the several-point kernel
 on ordinary data: 1e-6 of the larger of the point's largest output and one per galaxy; against the oracle 1e-5 and
@@ -19,14 +19,15 @@ FAMILIES = [O.EPRIOR_BA14, O.EPRIOR_TRUNC_GAUSS]
 def _rows(n, K, seed):
     rng = np.random.default_rng(seed)
     e1, e2 = rng.normal(0, 0.15, (2, n, K)).astype(np.float32).clip(-0.45, 0.45)
-    e1[::5, :min(K - 1, 9)] = 0.85             # outside the truncation radius
+    e1[::5, :min(K - 1, 9)] = 0.85             # outside the truncation radius: a lane's first samples
+    e1[3::10, :min(K - 1, 12)] = 0.85          # a lane's whole first chunk
     return e1, e2
 
 
 @pytest.mark.parametrize("K", [4, 48, 52, 300])
 @pytest.mark.parametrize("family", FAMILIES)
 @pytest.mark.parametrize("alphas", [(0.2, 0.3, 0.12, 0.15), (0.107, 0.105, 0.2, 0.02), (0.005, 0.01, 0.05, 0.1),
-                                    (0.094, 0.097, 0.2, 0.02)])
+                                    (0.172, 0.175, 0.2, 0.18)])
 def test_points_at_any_width(cuda, K, family, alphas):
     n = 70
     e1, e2 = _rows(n, K, K)
