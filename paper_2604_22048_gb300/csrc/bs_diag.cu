@@ -45,52 +45,6 @@ __device__ __forceinline__ void store_ess(float sum, const ChainMoments &m, int 
     if (rhat) rhat[out] = sqrtf(m.vp / m.W);
 }
 
-// The chains at x by one warp, each product's factors read again at every lag and each rho divided out.
-__device__ __noinline__ void ess_from_global(const float *x, int C, int S, size_t out, float *ess, float *rhat)
-{
-    const int lane = threadIdx.x & 31;
-    float mean[kMaxChains];
-    float wsum = 0.f, mbar = 0.f;
-    for (int c = 0; c < C; ++c) {
-        const float *xc = x + (size_t)c * S;
-        float s = 0.f;
-        for (int i = lane; i < S; i += 32) s += xc[i];
-        s = warp_sum(s) / (float)S;
-        float v = 0.f;
-        for (int i = lane; i < S; i += 32) {
-            const float d = xc[i] - s;
-            v = fmaf(d, d, v);
-        }
-        v = warp_sum(v) / (float)(S - 1);
-        mean[c] = s;
-        wsum += v;
-        mbar += s;
-    }
-    const ChainMoments cm = chain_moments(mean, wsum, mbar, C, S);
-    const float W = cm.W, vp = cm.vp;
-    auto rho = [&](int t) -> float {
-        float a = 0.f;
-        for (int c = 0; c < C; ++c) {
-            const float *xc = x + (size_t)c * S;
-            float s = 0.f;
-            for (int i = lane; i + t < S; i += 32) s = fmaf(xc[i] - mean[c], xc[i + t] - mean[c], s);
-            a += warp_sum(s) / (float)S;
-        }
-        a /= C;
-        return 1.0f - (W - a) / vp;
-    };
-    float sum = 0.f, prev = INFINITY;
-    for (int kk = 0; 2 * kk + 1 < S; ++kk) {
-        const float r0 = (kk == 0) ? 1.0f : rho(2 * kk);
-        const float P = r0 + rho(2 * kk + 1);
-        if (!(P > 0.f)) break;
-        const float Pm = P > prev ? prev : P;
-        sum += Pm;
-        prev = Pm;
-    }
-    if (lane == 0) store_ess(sum, cm, C, S, out, ess, rhat);
-}
-
 // The chains of a warp's (galaxy, parameter) are staged once in shared memory as deviations
 // from their means, two chains interleaved (zeros beside the last of an odd number), pair p at
 // p (S + kLagBlock) with zeros after it, and their autocovariances are taken kLagBlock lags at a
@@ -203,12 +157,15 @@ __global__ void __launch_bounds__(128, 8) ess_kernel(const float *samples, int n
         }
     }
     __syncwarp();
-    const ChainMoments m = chain_moments(mean, wsum, mbar, C, S);
-    // below, rho = 1 - (W - a) (1 / vp) with the chains' products in one sum: not for a variance whose
-    // reciprocal, or whose C S-fold sum, a float does not hold
-    if (!(m.vp >= 0x1p-120f && m.vp <= 0x1p100f)) {
-        ess_from_global(x, C, S, (size_t)gal * 6 + k, ess, rhat);
-        return;
+    ChainMoments m = chain_moments(mean, wsum, mbar, C, S);
+    // A variance whose reciprocal, or whose C S-fold sum, a float does not hold: the staged deviations are
+    // brought near 1 by a power of two, which no ratio below sees.
+    if (!(m.vp >= 0x1p-100f && m.vp <= 0x1p100f)) {
+        const float s = m.vp < 1.0f ? 0x1p60f : 0x1p-60f;
+        for (int i = lane; i < (C + 1) / 2 * stride; i += 32) d[i] = make_float2(d[i].x * s, d[i].y * s);
+        m.W *= s * s;
+        m.vp *= s * s;
+        __syncwarp();
     }
     const int L = ((S + 31) >> 5) | 1, i0 = lane * L;
     const float inv_n = 1.0f / ((float)C * (float)S), inv_vp = 1.0f / m.vp;
@@ -275,14 +232,56 @@ __global__ void __launch_bounds__(128, 8) ess_kernel(const float *samples, int n
     if (lane == 0) store_ess(sum, m, C, S, (size_t)gal * 6 + k, ess, rhat);
 }
 
-// Chains too long for shared memory: those whose number rounded up to even times S + 8 is above 57,344.
+// Chains too long for shared memory, those whose number rounded up to even times S + 8 is above 57,344: read
+// per lag.
 __global__ void __launch_bounds__(128) ess_kernel_global(const float *samples, int n_gal, int C, int S,
                                                          float *ess, float *rhat)
 {
+    const int lane = threadIdx.x & 31;
     const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (wid >= (long long)n_gal * 6) return;
     const int gal = (int)(wid / 6), k = (int)(wid % 6);
-    ess_from_global(samples + (((size_t)k * n_gal + gal) * C) * S, C, S, (size_t)gal * 6 + k, ess, rhat);
+    const float *x = samples + (((size_t)k * n_gal + gal) * C) * S;
+    float mean[kMaxChains];
+    float wsum = 0.f, mbar = 0.f;
+    for (int c = 0; c < C; ++c) {
+        const float *xc = x + (size_t)c * S;
+        float s = 0.f;
+        for (int i = lane; i < S; i += 32) s += xc[i];
+        s = warp_sum(s) / (float)S;
+        float v = 0.f;
+        for (int i = lane; i < S; i += 32) {
+            const float d = xc[i] - s;
+            v = fmaf(d, d, v);
+        }
+        v = warp_sum(v) / (float)(S - 1);
+        mean[c] = s;
+        wsum += v;
+        mbar += s;
+    }
+    const ChainMoments cm = chain_moments(mean, wsum, mbar, C, S);
+    const float W = cm.W, vp = cm.vp;
+    auto rho = [&](int t) -> float {
+        float a = 0.f;
+        for (int c = 0; c < C; ++c) {
+            const float *xc = x + (size_t)c * S;
+            float s = 0.f;
+            for (int i = lane; i + t < S; i += 32) s = fmaf(xc[i] - mean[c], xc[i + t] - mean[c], s);
+            a += warp_sum(s) / (float)S;
+        }
+        a /= C;
+        return 1.0f - (W - a) / vp;
+    };
+    float sum = 0.f, prev = INFINITY;
+    for (int kk = 0; 2 * kk + 1 < S; ++kk) {
+        const float r0 = (kk == 0) ? 1.0f : rho(2 * kk);
+        const float P = r0 + rho(2 * kk + 1);
+        if (!(P > 0.f)) break;
+        const float Pm = P > prev ? prev : P;
+        sum += Pm;
+        prev = Pm;
+    }
+    if (lane == 0) store_ess(sum, cm, C, S, (size_t)gal * 6 + k, ess, rhat);
 }
 
 // FP32 FMA throughput: eight independent chains per thread of x = x a + b on

@@ -11,7 +11,7 @@ from test_gpu_ess_sizes import _reference
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("exponent", [-66, -64, -40, 40])
+@pytest.mark.parametrize("exponent", [-66, -64, -40, 40, 58])
 def test_ess_of_small_and_large_units(cuda, exponent):
     rng = np.random.default_rng(4)
     n, C, S = 2, 4, 300
