@@ -18,7 +18,8 @@
 // n^3 of them); a tile's operands pass through shared memory, an element of it stays in a
 // register over kPivot (or, for P, all) terms.
 // 64 galaxies of 21 px: 50.1 ms a column at a time through global memory, one CTA per galaxy;
-// 18.5 ms in clusters of two (128 SMs, FP64 pipe 73% active).  Block sweeps with fused
+// 18.5 ms in clusters of two (128 SMs, FP64 pipe 73% active), 17.2 ms with the entries that are
+// not needed left out of the tiles; 2,000 of 7 px 3.67, 4.53 and 3.29 ms.  Block sweeps with fused
 // multiply-adds took 9 ms but round differently: some elements of P moved by an FP32 ulp.
 #include <cmath>
 
@@ -385,7 +386,7 @@ bs_status bs_dense_precision(int32_t n_gal, const int32_t *side, int32_t max_sid
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // CTAs per galaxy: as many (a power of two up to a portable cluster) as leave no CTA without an
-    // SM of its own, and no more than there are tiles to share (64 galaxies of 21 px: 18.5 ms in
+    // SM of its own, and no more than there are tiles to share (64 galaxies of 21 px: 17.2 ms in
     // clusters of two)
     const size_t n = (size_t)max_side * max_side;
     const int nt = ((int)n + bs::kTile - 1) / bs::kTile;

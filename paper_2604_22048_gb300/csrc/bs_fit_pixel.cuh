@@ -435,12 +435,13 @@ __device__ void pix_drain(const FitParams &P, const GalCtx &gc, const SmemView &
 // instance PROF 4).  The gradient is the half-plane pass on the effective spectrum
 // D' = M + DFT(y) (scaled as the table).
 //
-// One CTA of 16 warps runs a galaxy's chains (at most 4, or a share of them where there are SMs to
-// spare: dense_chains_per_cta), one evaluation of every chain at a time: the first warp of each chain (its leader) runs the chain's logic, and all
-// warps meet in dense_round, where one read of P serves every chain.  The transforms'
-// rows are split over the warps of the chain (16 / n_chains), the product's columns over
-// all 16 warps; every output is summed by one lane in a fixed order, so a chain's draws
-// do not depend on the others.  The product is bound by the read of P (778 KB at 21 px,
+// A CTA runs a galaxy's chains (at most 4, or a share of them where there are SMs to
+// spare: dense_chains_per_cta) on 16 warps, or on fewer where small stamps share an SM
+// (dense_warps_for), one evaluation of every chain at a time: the first warp of each chain
+// (its leader) runs the chain's logic, and all warps meet in dense_round, where one read of P
+// serves every chain.  The transforms' rows are split over the warps of the chain, the product's
+// columns over all warps; every output is summed by one lane in a fixed order, so a chain's
+// draws depend neither on the others nor on the number of warps.  The product is bound by the read of P (778 KB at 21 px,
 // from L2): 32 rows of loads are in flight per warp.
 // 64 galaxies of 21 px, 4 chains x (100 + 100), L <= 8: 332 ms with a warp per chain that
 // evaluated on its own (the product waiting for each row of P, transforms on 11 to 21 of 32
@@ -783,7 +784,7 @@ __device__ bool dense_round(const FitParams &P, const GalCtx &gc, const SmemView
     if (!any) return false;
     // this warp's share of one chain: member k of the nk warps of chain s (warps past
     // nk n_slots take part in the product only); rows are taken in passes of as many as
-    // share them evenly (H <= 16 rows over at least 4 warps)
+    // share them evenly, four at most
     const int s = warp % n_slots, k = warp / n_slots, nk = nwarp / n_slots;
     const bool in = k < nk && dv.req[8 * s + 6] != 0.f;
     const int ub = (H + nk - 1) / nk;

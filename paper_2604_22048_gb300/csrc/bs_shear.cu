@@ -481,7 +481,7 @@ constexpr int kTmaStages = 3;
 // Launch bounds for 2 CTAs per SM, of whose 128 registers the compiler takes 78: without b 3 CTAs are
 // resident and nothing is rebuilt or spilled.  10^6 x 300: 446 us so (5.4 TB/s), 472 us bounded
 // for 3 CTAs, 476 us before the constants were held, 539 us with 4 stages (2 CTAs fit).
-// With b, 3.6 GB, 2 CTAs fit: 580-590 us; 610 us with two stages, which let 3 in; 709 us through
+// With b, 3.6 GB, 2 CTAs fit: 580-600 us; 610 us with two stages, which let 3 in; 709 us through
 // per-lane cp.async copies, whose kernel this replaced.  What is left is the memory: the
 // warps' waits find their tile late, and deeper rings per warp or L2 prefetches of whole tiles made
 // the pass without b slower (516-690 us).
