@@ -211,13 +211,13 @@ def flops_per_eval(N):
 # to that file the traffic is reported as null until the next capture.
 CAPTURED_TRAFFIC = {
     # one galaxy of the plain workload (53x53, 4 chains x (200 + 300) draws), from a one-pass
-    # capture of the full 10,000-galaxy launch: (135,008,768 + 293,555,968) B / 10,000
+    # capture of the full 10,000-galaxy launch: (135,208,192 + 293,162,752) B / 10,000
     "fit": ("paper_2604_22048_gb300/csrc/bs_fit_impl.cuh",
-            "303672ef0b44afd67b5e4b2b7498b86e6d0e16a4a25a910ae55fcb27166eda58", 42856.5,
+            "e101e7c455f88575daf8a23dbcf546b622b44e8c82cc248b3cde1e8fd341ec57", 42837.1,
             {"side": 53, "chains": 4, "n_warmup": 200, "n_samples": 300}),
-    # one interim sample of the shear workload: (483,382,528 + 457,472) B / (200,000 x 300)
+    # one interim sample of the shear workload: (483,370,496 + 443,136) B / (200,000 x 300)
     "shear": ("paper_2604_22048_gb300/csrc/bs_shear.cu",
-              "65381469d210009cd3a12dbab856cfd3bb88604758825b9a003dd9fdee3e818a", 8.0640, {}),
+              "0f07753086178d27319a6868b78aac19bdfe69c48e3f9e3621cfec8d26536474", 8.0636, {}),
 }
 
 
